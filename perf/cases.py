@@ -70,8 +70,8 @@ def draw(rng):
             if 2.0 * m * n * k <= 1.1e12:
                 return {"kind": kind, "layout": rng.choice(["tn", "nn"]), "M": m, "N": n, "K": k}
     if kind == "moe":
-        return {"kind": kind, "T": _log_int(rng, 16, 4096), "C": 7168, "F": 2048, "E": 32, "K": rng.choice([2, 4, 8]) if
-                rng.random() < 0.5 else 4}
+        k = rng.choice([2, 4, 4, 4, 8])
+        return {"kind": kind, "T": _log_int(rng, 16, 16384 // k), "C": 7168, "F": 2048, "E": 32, "K": k}
     hkv = rng.choice([1, 2, 4, 8, 8, 16])
     group = rng.choice([1, 1, 2, 4, 4, 8])
     causal = rng.random() < 0.7
@@ -85,9 +85,10 @@ def draw(rng):
     while True:
         b, sq = _log_int(rng, 1, 16), _log_int(rng, 64, 16384)
         sk = sq if kind != "fwd" or rng.random() < 0.7 else sq + _log_int(rng, 64, 8192)  # a chunk after cached keys
-        if 4.0 * b * hkv * group * sq * sk * d <= (2.0e12 if kind == "varlen" or not causal else 4.0e12):
-            return {"kind": kind, "B": b, "H": hkv * group, "Hkv": hkv, "Sq": sq, "Sk": sk, "D": d, "causal": causal,
-                    "dist": rng.choice(["normal", "normal", "uniform"]), "peaked": rng.choice([0, 0, 64]) if causal else 0}
+        c = {"kind": kind, "B": b, "H": hkv * group, "Hkv": hkv, "Sq": sq, "Sk": sk, "D": d, "causal": causal,
+             "dist": rng.choice(["normal", "normal", "uniform"]), "peaked": rng.choice([0, 0, 64]) if causal else 0}
+        if work(c)["flops"] <= 2.0e12:
+            return c
 
 
 def _lengths(case):

@@ -166,7 +166,8 @@ size_t ave_attn_host_workspace_bytes(int B, int H, int Hkv, int Sq, int Sk, int 
  * workspace: DEVICE scratch of at least ave_attn_splitkv_workspace_bytes(...)
  * bytes, 256-byte aligned, owned by the caller; it holds the fp32 partial
  * outputs and log-sum-exps, is fully rewritten by each call, and may be
- * reused by later calls on the same stream.  Two kernels are enqueued.
+ * reused by later calls on the same stream.  Two kernels are enqueued (one, and
+ * no scratch is touched, with n_splits = 1).
  */
 #define AVE_SPLITKV_MAX_SPLITS 64
 int ave_attn_fwd_splitkv(const void *q, const void *k, const void *v, void *o, float *lse,

@@ -380,7 +380,7 @@ attn_fwd_1t_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                 // no key visible to any row of this tile: O = 0, LSE = -inf
                 if (i < sq) {
                     const uint4 z = make_uint4(0, 0, 0, 0);
-                    if (SPLIT) {
+                    if (SPLIT && p.o_partial) {
                         const size_t row = (size_t(split_of(w)) * p.BH + bh) * p.Sq + i;
                         for (int c = 0; c < D / 4; ++c) reinterpret_cast<uint4 *>(p.o_partial + row * D)[c] = z;
                         p.lse_partial[row] = -INFINITY;
@@ -526,7 +526,8 @@ attn_fwd_1t_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                     const size_t prow = SPLIT ? (size_t(split_of(w)) * p.BH + bh) * p.Sq + i : 0;
                     __nv_bfloat16 *o_row = reinterpret_cast<__nv_bfloat16 *>(p.o) + batch_coord(w) * p.o_stride_b +
                                            w.h * p.o_stride_h + (q_base_of(w) + i) * p.o_stride_r;
-                    if (SPLIT) {
+                    const bool partial = SPLIT && p.o_partial != nullptr;  // a single key range writes the result itself
+                    if (partial) {
                         if (i < p.Sq) p.lse_partial[prow] = lse_row;
                     } else {
                         if (i < sq) p.lse[lse_index(w, p, i)] = lse_row;
@@ -541,7 +542,7 @@ attn_fwd_1t_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                             __syncwarp();
                             if (lane == 0) mbar_arrive(smem_u32(&bar_o_free));
                         }
-                        if (SPLIT) {
+                        if (partial) {
                             // partial result of this key range: normalised O in fp32, straight to global
                             if (i < p.Sq) {
 #pragma unroll

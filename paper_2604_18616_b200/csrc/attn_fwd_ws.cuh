@@ -531,7 +531,7 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                 // no key visible to any row of this sub-tile: O = 0, LSE = -inf
                 if (i < sq) {
                     const uint4 z = make_uint4(0, 0, 0, 0);
-                    if (SPLIT) {
+                    if (SPLIT && p.o_partial) {
                         const size_t row = (size_t(split_of(w)) * p.BH + bh) * p.Sq + i;
                         for (int c = 0; c < D / 4; ++c) reinterpret_cast<uint4 *>(p.o_partial + row * D)[c] = z;
                         p.lse_partial[row] = -INFINITY;
@@ -720,15 +720,28 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                     const float inv_l = (l_run > 0.f) ? 1.f / l_run : 0.f;
                     const float lse_row = (l_run > 0.f) ? (m_run + log2f(l_run)) * 0.6931471805599453f : -INFINITY;
                     if (SPLIT) {
-                        // partial result of this key range: normalised O in fp32 and its LSE, straight to global
+                        // partial result of this key range: normalised O in fp32 and its LSE, straight to global (with
+                        // a single key range this is the result: O in bf16)
+                        const bool partial = p.o_partial != nullptr;
                         const size_t row = (size_t(split_of(w)) * p.BH + bh) * p.Sq + i;
-                        if (i < p.Sq) p.lse_partial[row] = lse_row;
+                        __nv_bfloat16 *o_row = reinterpret_cast<__nv_bfloat16 *>(p.o) + row * D;
+                        if (i < p.Sq) (partial ? p.lse_partial : p.lse)[row] = lse_row;
 #pragma unroll
                         for (int c = 0; c < D / 32; ++c) {
                             uint32_t oc[32];
                             tmem_ld_x32(tO + c * 32, oc);
                             tmem_wait_ld();
-                            if (i < p.Sq) {
+                            if (i < p.Sq && !partial) {
+#pragma unroll
+                                for (int e = 0; e < 32; e += 8) {
+                                    uint4 v4;
+                                    v4.x = pack_bf16x2(__uint_as_float(oc[e]) * inv_l, __uint_as_float(oc[e + 1]) * inv_l);
+                                    v4.y = pack_bf16x2(__uint_as_float(oc[e + 2]) * inv_l, __uint_as_float(oc[e + 3]) * inv_l);
+                                    v4.z = pack_bf16x2(__uint_as_float(oc[e + 4]) * inv_l, __uint_as_float(oc[e + 5]) * inv_l);
+                                    v4.w = pack_bf16x2(__uint_as_float(oc[e + 6]) * inv_l, __uint_as_float(oc[e + 7]) * inv_l);
+                                    *reinterpret_cast<uint4 *>(o_row + c * 32 + e) = v4;
+                                }
+                            } else if (i < p.Sq) {
 #pragma unroll
                                 for (int e = 0; e < 32; e += 4)
                                     reinterpret_cast<float4 *>(p.o_partial + row * D + c * 32)[e >> 2] =

@@ -297,9 +297,9 @@ bool use_one_subtile(int B, int H, int Hkv, int Sq, int Sk, int causal, bool spl
     return Sq <= ave::BM;
 }
 
-// Encode the tensor maps, fill the kernel parameters and launch.  n_splits == 1 with no partial
-// buffers is the ordinary forward; otherwise every work tile covers one range of keys_per_split keys
-// and writes fp32 partials.
+// Encode the tensor maps, fill the kernel parameters and launch.  In a `split` launch every work tile covers
+// one range of keys_per_split keys and writes fp32 partials (with a single range and no partial buffers: the
+// result itself).
 // Variable-length launch: token-major tensors [rows, heads, D] and the sequences' row ranges.
 struct VarlenArgs {
     const int *cu_q, *cu_k;  // device, B + 1 entries
@@ -309,16 +309,15 @@ struct VarlenArgs {
 // `layout` (strides of q, k, v, o in this order) is NULL for contiguous [B, heads, rows, D] tensors; `varlen`
 // is NULL unless the launch is a variable-length one (Sq and Sk are then the longest sequences).
 int launch_attention(const void *q, const void *k, const void *v, void *o, float *lse, int B, int H, int Hkv, int Sq,
-                     int Sk, int D, int causal, float scale, int n_splits, int keys_per_split, float *o_partial,
-                     float *lse_partial, int rows_per_head, const Strides *layout, const VarlenArgs *varlen,
-                     cudaStream_t s) {
+                     int Sk, int D, int causal, float scale, bool split, int n_splits, int keys_per_split,
+                     float *o_partial, float *lse_partial, int rows_per_head, const Strides *layout,
+                     const VarlenArgs *varlen, cudaStream_t s) {
     auto token_major = [&](int heads, int rows) { return Strides{(long long)rows * heads * D, (long long)D, (long long)heads * D}; };
     const int rows_q = varlen ? varlen->total_q : Sq, rows_k = varlen ? varlen->total_k : Sk, n_batch = varlen ? 1 : B;
     const Strides sq = layout ? layout[0] : varlen ? token_major(H, rows_q) : contiguous_strides(H, Sq, D);
     const Strides sk = layout ? layout[1] : varlen ? token_major(Hkv, rows_k) : contiguous_strides(Hkv, Sk, D);
     const Strides sv = layout ? layout[2] : varlen ? token_major(Hkv, rows_k) : contiguous_strides(Hkv, Sk, D);
     const Strides so = layout ? layout[3] : varlen ? token_major(H, rows_q) : contiguous_strides(H, Sq, D);
-    const bool split = o_partial != nullptr;
     // a head dimension above 128 leaves no TMEM for a second sub-tile: only the single-sub-tile kernel has it
     const bool one = D > 128 || use_one_subtile(B, H, Hkv, Sq, Sk, causal, split, varlen != nullptr);
     CUtensorMap tq, tk, tv, to;
@@ -385,37 +384,69 @@ int launch_attention(const void *q, const void *k, const void *v, void *o, float
 
 // Combine the partial results of the key ranges of every query row:
 //   LSE = ln sum_s exp(LSE_s),  O = sum_s exp(LSE_s - LSE) * O_s.
-// One thread per (row, 8 output columns).
-__global__ void splitkv_merge_kernel(const float *__restrict__ o_partial, const float *__restrict__ lse_partial,
-                                     __nv_bfloat16 *__restrict__ o, float *__restrict__ lse, long long rows, int D,
-                                     int n_splits) {
-    const int chunks = D / 8;
-    const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= rows * chunks) return;
-    const long long row = idx / chunks;
-    const int ch = int(idx - row * chunks);
-    float m = -INFINITY;
-    for (int s = 0; s < n_splits; ++s) m = fmaxf(m, lse_partial[s * rows + row]);
-    float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    float denom = 0.f;
-    if (m != -INFINITY) {
-        for (int s = 0; s < n_splits; ++s) {
-            const float w = __expf(lse_partial[s * rows + row] - m);
-            denom += w;
-            const float4 *src = reinterpret_cast<const float4 *>(o_partial + (s * rows + row) * D + ch * 8);
-            const float4 a = src[0], b = src[1];
-            acc[0] += w * a.x; acc[1] += w * a.y; acc[2] += w * a.z; acc[3] += w * a.w;
-            acc[4] += w * b.x; acc[5] += w * b.y; acc[6] += w * b.z; acc[7] += w * b.w;
+// One or more warps per row (`warps_per_row`, a power of two up to 8), which share out the row's key ranges; a lane
+// holds four neighbouring output columns (at D = 64 the half-warps take ranges in turn).  The bound is latency: a decode step has few rows and up to
+// 64 ranges, and a thread that walks the ranges by itself waits for one load after the other (measured with 32 rows
+// and 37 ranges: 23 us for a thread per 8 columns, 4 us with eight warps per row).
+constexpr int kMergeThreads = 256;
+__global__ void __launch_bounds__(kMergeThreads)
+splitkv_merge_kernel(const float *__restrict__ o_partial, const float *__restrict__ lse_partial,
+                     __nv_bfloat16 *__restrict__ o, float *__restrict__ lse, long long rows, int D, int n_splits,
+                     int warps_per_row) {
+    __shared__ float4 part[kMergeThreads];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int sub = warp & (warps_per_row - 1);  // which of the row's warps
+    const long long row = (long long)blockIdx.x * (kMergeThreads / 32 / warps_per_row) + warp / warps_per_row;
+    const bool live = row < rows;
+    const int lanes_per_range = D / 4, ranges_at_once = 32 / lanes_per_range;  // 32 and 1, or 16 and 2
+    const int col4 = lane & (lanes_per_range - 1);
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    float m = -INFINITY, denom = 0.f;
+    if (live) {
+        // the ranges' weights: lane l holds those of ranges l and l + 32
+        static_assert(AVE_SPLITKV_MAX_SPLITS <= 64, "two ranges per lane");
+        const float l0 = lane < n_splits ? lse_partial[lane * rows + row] : -INFINITY;
+        const float l1 = lane + 32 < n_splits ? lse_partial[(lane + 32) * rows + row] : -INFINITY;
+        m = fmaxf(l0, l1);
+#pragma unroll
+        for (int x = 16; x > 0; x >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, x));
+        const float w0 = m == -INFINITY ? 0.f : __expf(l0 - m);
+        const float w1 = m == -INFINITY ? 0.f : __expf(l1 - m);
+        denom = w0 + w1;
+#pragma unroll
+        for (int x = 16; x > 0; x >>= 1) denom += __shfl_xor_sync(0xffffffffu, denom, x);
+        const int stride = warps_per_row * ranges_at_once;
+#pragma unroll 4
+        for (int s0 = sub * ranges_at_once; s0 < n_splits; s0 += stride) {
+            const int s = s0 + lane / lanes_per_range;  // (beyond the last range: weight 0, the last range's values)
+            const float w_lo = __shfl_sync(0xffffffffu, w0, s & 31), w_hi = __shfl_sync(0xffffffffu, w1, s & 31);
+            const float ws = s < n_splits ? (s < 32 ? w_lo : w_hi) : 0.f;
+            const float4 v = reinterpret_cast<const float4 *>(o_partial + (min(s, n_splits - 1) * rows + row) * D)[col4];
+            acc.x += ws * v.x; acc.y += ws * v.y; acc.z += ws * v.z; acc.w += ws * v.w;
         }
     }
+    if (ranges_at_once == 2) {
+        acc.x += __shfl_xor_sync(0xffffffffu, acc.x, 16); acc.y += __shfl_xor_sync(0xffffffffu, acc.y, 16);
+        acc.z += __shfl_xor_sync(0xffffffffu, acc.z, 16); acc.w += __shfl_xor_sync(0xffffffffu, acc.w, 16);
+    }
+    if (warps_per_row > 1) {
+        part[threadIdx.x] = acc;
+        __syncthreads();
+        if (sub != 0) return;
+        for (int x = 1; x < warps_per_row; ++x) {
+            const float4 v = part[threadIdx.x + x * 32];
+            acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
+        }
+    }
+    if (!live) return;
     const float inv = denom > 0.f ? 1.f / denom : 0.f;
-    uint4 out;
-    out.x = ave::pack_bf16x2(acc[0] * inv, acc[1] * inv);
-    out.y = ave::pack_bf16x2(acc[2] * inv, acc[3] * inv);
-    out.z = ave::pack_bf16x2(acc[4] * inv, acc[5] * inv);
-    out.w = ave::pack_bf16x2(acc[6] * inv, acc[7] * inv);
-    reinterpret_cast<uint4 *>(o + row * D)[ch] = out;
-    if (ch == 0) lse[row] = (denom > 0.f) ? m + logf(denom) : -INFINITY;
+    if (lane < lanes_per_range) {
+        uint2 out;
+        out.x = ave::pack_bf16x2(acc.x * inv, acc.y * inv);
+        out.y = ave::pack_bf16x2(acc.z * inv, acc.w * inv);
+        reinterpret_cast<uint2 *>(o + row * D)[col4] = out;
+    }
+    if (lane == 0) lse[row] = (denom > 0.f) ? m + logf(denom) : -INFINITY;
 }
 
 // One warp waits, with the library's bounded wait, on an mbarrier that nobody ever arrives on: the
@@ -438,16 +469,22 @@ int run_splitkv(const void *q, const void *k, const void *v, void *o, float *lse
     const int kps = ave::splitkv_keys_per_split(Sk, n_splits);
     const int G = H / Hkv;
     const bool pack = ave::splitkv_packs_heads(H, Hkv, Sq);  // query heads of a KV head as rows of one problem
-    int st = pack ? launch_attention(q, k, v, o, lse, B, Hkv, Hkv, G * Sq, Sk, D, causal, scale, n_splits, kps,
-                                     o_partial, lse_partial, Sq, nullptr, nullptr, s)
-                  : launch_attention(q, k, v, o, lse, B, H, Hkv, Sq, Sk, D, causal, scale, n_splits, kps, o_partial,
-                                     lse_partial, 0, nullptr, nullptr, s);
-    if (st != AVE_OK) return st;
+    // a single key range needs no merge: the attention kernel writes the result
+    float *const op = n_splits > 1 ? o_partial : nullptr;
+    float *const lp = n_splits > 1 ? lse_partial : nullptr;
+    const int st = pack ? launch_attention(q, k, v, o, lse, B, Hkv, Hkv, G * Sq, Sk, D, causal, scale, true, n_splits, kps,
+                                           op, lp, Sq, nullptr, nullptr, s)
+                        : launch_attention(q, k, v, o, lse, B, H, Hkv, Sq, Sk, D, causal, scale, n_splits > 1, n_splits,
+                                           kps, op, lp, 0, nullptr, nullptr, s);
+    if (st != AVE_OK || n_splits == 1) return st;
     const long long rows = (long long)B * H * Sq;
-    const long long work = rows * (D / 8);
-    const int threads = 256;
-    splitkv_merge_kernel<<<unsigned((work + threads - 1) / threads), threads, 0, s>>>(
-        o_partial, lse_partial, static_cast<__nv_bfloat16 *>(o), lse, rows, D, n_splits);
+    // enough warps to cover the chip a few times over, none with less than two ranges to add up
+    constexpr int kWarps = kMergeThreads / 32;
+    int wpr = 1;
+    while (wpr < kWarps && rows * wpr < 148 * 16 && 4 * wpr <= n_splits) wpr *= 2;
+    const long long ctas = (rows * wpr + kWarps - 1) / kWarps;
+    splitkv_merge_kernel<<<unsigned(ctas), kMergeThreads, 0, s>>>(o_partial, lse_partial, static_cast<__nv_bfloat16 *>(o), lse,
+                                                                 rows, D, n_splits, wpr);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
         t_last_cuda_error = int(e);
@@ -733,7 +770,7 @@ int ave_attn_fwd(const void *q, const void *k, const void *v, void *o, float *ls
     if (st != AVE_OK) return st;
     st = check_device();
     if (st != AVE_OK) return st;
-    return launch_attention(q, k, v, o, lse, B, H, Hkv, Sq, Sk, D, causal, scale, 1, 0, nullptr, nullptr, 0, nullptr,
+    return launch_attention(q, k, v, o, lse, B, H, Hkv, Sq, Sk, D, causal, scale, false, 1, 0, nullptr, nullptr, 0, nullptr,
                             nullptr, static_cast<cudaStream_t>(stream));
 }
 
@@ -758,7 +795,7 @@ int ave_attn_fwd_strided(const void *q, const void *k, const void *v, void *o, f
     if (st != AVE_OK) return st;
     st = check_device();
     if (st != AVE_OK) return st;
-    return launch_attention(q, k, v, o, lse, B, H, Hkv, Sq, Sk, D, causal, scale, 1, 0, nullptr, nullptr, 0, layout,
+    return launch_attention(q, k, v, o, lse, B, H, Hkv, Sq, Sk, D, causal, scale, false, 1, 0, nullptr, nullptr, 0, layout,
                             nullptr, static_cast<cudaStream_t>(stream));
 }
 
@@ -777,7 +814,7 @@ int ave_attn_fwd_varlen(const void *q, const void *k, const void *v, void *o, fl
     st = check_device();
     if (st != AVE_OK) return st;
     const VarlenArgs vl{cu_seqlens_q, cu_seqlens_k, total_q, total_k};
-    return launch_attention(q, k, v, o, lse, B, H, Hkv, max_Sq, max_Sk, D, causal, scale, 1, 0, nullptr, nullptr, 0,
+    return launch_attention(q, k, v, o, lse, B, H, Hkv, max_Sq, max_Sk, D, causal, scale, false, 1, 0, nullptr, nullptr, 0,
                             nullptr, &vl, static_cast<cudaStream_t>(stream));
 }
 

@@ -40,7 +40,8 @@ struct FwdParams {
     float scale_log2; // scale * log2(e)
     int causal_off;   // key j is visible to query i iff j <= i + causal_off (Sk - Sq of the whole problem)
     // Split-KV launches only: the keys are cut into n_splits ranges of keys_per_split (a multiple of
-    // BN); a work tile handles one range and writes a normalised fp32 partial result.
+    // BN); a work tile handles one range and writes a normalised fp32 partial result, or (o_partial NULL: a
+    // single range) the result itself.
     int n_splits;
     int keys_per_split;
     int rows_per_head;   // > 0: rows are (query head in group, query position) pairs, this many positions per head

@@ -237,6 +237,23 @@ int prepare_kernel(Kernel kern, int smem_bytes, int check_register_split, PerDev
     return AVE_OK;
 }
 
+// Launch a kernel that begins with grid_dependency_wait(): its blocks may be set up while the kernel before it in the
+// stream still runs (programmatic dependent launch), which takes the launch latency out of a chain of kernels.
+template <class... Params, class... Args>
+cudaError_t launch_dependent(void (*kern)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args... args) {
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, Params(args)...);
+}
+
 template <int D, bool CAUSAL, bool SPLIT, bool VARLEN = false>
 int launch_ws(const CUtensorMap &tq, const CUtensorMap &tk, const CUtensorMap &tv, const CUtensorMap &to,
               const ave::FwdParams &p, cudaStream_t stream) {
@@ -398,6 +415,7 @@ splitkv_merge_kernel(const float *__restrict__ o_partial, const float *__restric
     const int sub = warp & (warps_per_row - 1);  // which of the row's warps
     const long long row = (long long)blockIdx.x * (kMergeThreads / 32 / warps_per_row) + warp / warps_per_row;
     const bool live = row < rows;
+    ave::grid_dependency_wait();
     const int lanes_per_range = D / 4, ranges_at_once = 32 / lanes_per_range;  // 32 and 1, or 16 and 2
     const int col4 = lane & (lanes_per_range - 1);
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -483,9 +501,8 @@ int run_splitkv(const void *q, const void *k, const void *v, void *o, float *lse
     int wpr = 1;
     while (wpr < kWarps && rows * wpr < 148 * 16 && 4 * wpr <= n_splits) wpr *= 2;
     const long long ctas = (rows * wpr + kWarps - 1) / kWarps;
-    splitkv_merge_kernel<<<unsigned(ctas), kMergeThreads, 0, s>>>(o_partial, lse_partial, static_cast<__nv_bfloat16 *>(o), lse,
-                                                                 rows, D, n_splits, wpr);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_dependent(splitkv_merge_kernel, dim3(unsigned(ctas)), dim3(kMergeThreads), 0, s, o_partial, lse_partial,
+                                     static_cast<__nv_bfloat16 *>(o), lse, rows, D, n_splits, wpr);
     if (e != cudaSuccess) {
         t_last_cuda_error = int(e);
         return AVE_ERR_CUDA;

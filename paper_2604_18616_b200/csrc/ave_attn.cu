@@ -513,9 +513,9 @@ int run_splitkv(const void *q, const void *k, const void *v, void *o, float *lse
 
 
 // C[M, N] = A[M, K] * B[N, K]^T: tensor maps of the three matrices, tile order, persistent launch.
-template <int TN, bool B_NMAJOR>
+template <bool B_NMAJOR>
 int launch_gemm_tile(const void *a, const void *b, void *c, int M, int N, int K, int sms, cudaStream_t s) {
-    using Cfg = ave::GemmCfg<TN>;
+    using Cfg = ave::GemmCfg;
     CUtensorMap ta, tb, tc;
     const Strides sa{(long long)M * K, (long long)M * K, (long long)K};
     const Strides sb{(long long)N * K, (long long)N * K, (long long)(B_NMAJOR ? N : K)};
@@ -533,10 +533,8 @@ int launch_gemm_tile(const void *a, const void *b, void *c, int M, int N, int K,
     p.K = K;
     p.tiles_m = (M + Cfg::kTileM - 1) / Cfg::kTileM;
     p.tiles_n = (N + Cfg::kTileN - 1) / Cfg::kTileN;
-    // The ~148 tiles in flight at a time should cover a near-square part of C, which minimises the A and B
-    // bytes they pull through L2: 16 block rows x 9 block columns of 128 x 256 is 2048 x 2304 elements.
     p.group_m = 16;
-    auto kern = ave::gemm_bf16_kernel<TN, B_NMAJOR>;
+    auto kern = ave::gemm_bf16_kernel<B_NMAJOR>;
     static PerDeviceOnce once;  // per instantiation
     const int st = prepare_kernel(kern, Cfg::kSmemBytes, 0, once);
     if (st != AVE_OK) return st;
@@ -545,6 +543,44 @@ int launch_gemm_tile(const void *a, const void *b, void *c, int M, int N, int K,
     const unsigned grid = unsigned(n_tiles < sms ? n_tiles : sms);
     kern<<<dim3(grid), dim3(Cfg::kThreads), Cfg::kSmemBytes, s>>>(ta, tb, tc, p);
     e = cudaGetLastError();
+    if (e != cudaSuccess) {
+        t_last_cuda_error = int(e);
+        return AVE_ERR_CUDA;
+    }
+    g_launches.fetch_add(1, std::memory_order_relaxed);
+    return AVE_OK;
+}
+
+// The same on CTA pairs with 256 x 256 tiles.
+template <bool B_NMAJOR>
+int launch_gemm_pair(const void *a, const void *b, void *c, int M, int N, int K, int sms, cudaStream_t s) {
+    using Cfg = ave::GemmPairCfg;
+    CUtensorMap ta, tb, tc;
+    const Strides sa{(long long)M * K, (long long)M * K, (long long)K};
+    const Strides sb{(long long)N * K, (long long)N * K, (long long)(B_NMAJOR ? N : K)};
+    const Strides sc{(long long)M * N, (long long)M * N, (long long)N};
+    if (!encode_map(&ta, a, K, M, 1, 1, sa, 128)) return AVE_ERR_CUDA;
+    if (B_NMAJOR) {  // B [K, N]: rows of N elements, boxes of 64 columns x 64 rows of K
+        if (!encode_map(&tb, b, N, K, 1, 1, sb, Cfg::kSliceK)) return AVE_ERR_CUDA;
+    } else {         // B [N, K]: rows of K elements, boxes of 64 columns of K x 128 rows
+        if (!encode_map(&tb, b, K, N, 1, 1, sb, 128)) return AVE_ERR_CUDA;
+    }
+    if (!encode_map(&tc, c, N, M, 1, 1, sc, Cfg::kOutBoxRows)) return AVE_ERR_CUDA;
+    ave::GemmParams p;
+    p.M = M;
+    p.N = N;
+    p.K = K;
+    p.tiles_m = (M + Cfg::kTileM - 1) / Cfg::kTileM;
+    p.tiles_n = (N + Cfg::kTileN - 1) / Cfg::kTileN;
+    p.group_m = 8;  // the ~74 tiles in flight cover 8 x 9.25 tiles, a near-square part of C
+    auto kern = ave::gemm_bf16_pair_kernel<B_NMAJOR>;
+    static PerDeviceOnce once;  // per instantiation
+    const int st = prepare_kernel(kern, Cfg::kSmemBytes, 0, once);
+    if (st != AVE_OK) return st;
+    const long long n_tiles = (long long)p.tiles_m * p.tiles_n;
+    const long long pairs = n_tiles < sms / 2 ? n_tiles : sms / 2;
+    kern<<<dim3(unsigned(2 * pairs)), dim3(Cfg::kThreads), Cfg::kSmemBytes, s>>>(ta, tb, tc, p);
+    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
         t_last_cuda_error = int(e);
         return AVE_ERR_CUDA;
@@ -562,12 +598,12 @@ int launch_gemm(const void *a, const void *b, void *c, int M, int N, int K, cuda
         t_last_cuda_error = int(e);
         return AVE_ERR_CUDA;
     }
-    // 128 x 256 tiles for no more than half of the SMs: halve the tile, so that twice as many SMs work and each
-    // finishes earlier (measured: n = 1024 gains a third, while at n = 2048, 128 tiles on 148 SMs, the narrow
-    // tile's second wave costs a third)
-    const long long wide_tiles = (long long)((M + 127) / 128) * ((N + 255) / 256);
-    if (2 * wide_tiles <= sms) return launch_gemm_tile<128, B_NMAJOR>(a, b, c, M, N, K, sms, s);
-    return launch_gemm_tile<256, B_NMAJOR>(a, b, c, M, N, K, sms, s);
+    // CTA pairs with 256 x 256 tiles move the fewest bytes per product (n = 4096: 96 us, against 105 us for 128 x 256 tiles of one
+    // CTA; 8192 x 8192 x 4096: 351 / 425 us).  Products whose 128 x 128 tiles fit the SMs all at once take those: with pairs
+    // most of the SMs would stand idle.
+    const long long tiles = (long long)((M + 127) / 128) * ((N + 127) / 128);
+    if (tiles <= sms) return launch_gemm_tile<B_NMAJOR>(a, b, c, M, N, K, sms, s);
+    return launch_gemm_pair<B_NMAJOR>(a, b, c, M, N, K, sms, s);
 }
 
 // E4M3 codes [d2, rows, inner] (inner contiguous) as a 4-D map with boxes of 128 bytes x box_rows rows, 128-byte

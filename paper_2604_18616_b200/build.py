@@ -34,9 +34,9 @@ ATTN_REGS_NEEDED = 128 * 64 + 256 * 216
 # The single-sub-tile kernel (OneCfg in csrc/attn_fwd_1t.cuh): 256 threads, 48 and 208 registers.
 ONE_THREADS = 256
 ONE_REGS_NEEDED = 128 * 48 + 128 * 208
-# The MoE GEMM (MoeGemmCfg in csrc/moe_fp8.cuh): 384 threads, 40 and 232 registers.
+# The MoE GEMM (MoeGemmCfg in csrc/moe_fp8.cuh): 384 threads, 56 and 224 registers.
 MOE_THREADS = 384
-MOE_REGS_NEEDED = 128 * 40 + 256 * 232
+MOE_REGS_NEEDED = 128 * 56 + 256 * 224
 
 
 def _sources():

@@ -203,7 +203,7 @@ bool register_split_fits_one_subtile(int regs_per_thread_at_launch) {
 }
 
 bool register_split_fits_moe_gemm(int regs_per_thread_at_launch) {
-    using Cfg = ave::MoeGemmCfg;
+    using Cfg = ave::MoeGemmCfg<true>;
     return 128 * Cfg::kRegsLight + 256 * Cfg::kRegsEpilogue <= Cfg::kThreads * regs_per_thread_at_launch;
 }
 
@@ -656,7 +656,7 @@ bool encode_map_f32(CUtensorMap *map, const void *base, long long cols, long lon
 // Scratch of one fused-MoE call, carved out of the caller's workspace (every part 256-byte aligned).
 struct MoeWorkspace {
     long long rows_cap;  // rows of the sorted order, padding included: a multiple of 128
-    size_t xq_s, sx_s, ho, aq, sa, row_of, pair_of, w_s, expert_off, cursor, tile_expert, bad_id, total;
+    size_t xq_s, sx_s, o, aq, sa, row_of, w_s, counts, cursor, tiles, n_row_tiles, total;
 };
 bool moe_layout(MoeWorkspace &w, int T, int C, int F, int E, int K) {
     if (T <= 0 || C <= 0 || F <= 0 || E <= 0 || K <= 0 || C % 128 || F % 128 || E > 1024) return false;
@@ -672,51 +672,41 @@ bool moe_layout(MoeWorkspace &w, int T, int C, int F, int E, int K) {
     const size_t rows = size_t(w.rows_cap);
     w.xq_s = take(rows * C);
     w.sx_s = take(rows * (C / 128) * 4);
-    // the up projection's result h [rows, 2F] is dead once the activations are requantised: the down projection's
-    // result o [rows, C] takes the same space
-    w.ho = take(rows * size_t(2 * F > C ? 2 * F : C) * 4);
+    w.o = take(rows * size_t(C) * 4);
     w.aq = take(rows * F);
     w.sa = take(rows * (F / 128) * 4);
     w.row_of = take(size_t(pairs) * 4);
-    w.pair_of = take(rows * 4);
     w.w_s = take(rows * 4);
-    w.expert_off = take(size_t(E + 1) * 4);
+    w.counts = take(size_t(E) * 4);
     w.cursor = take(size_t(E) * 4);
-    w.tile_expert = take(rows / 128 * 4);
-    w.bad_id = take(4);
+    w.tiles = take(rows / 128 * sizeof(ave::MoeRowTile));
+    w.n_row_tiles = take(4);
     w.total = off;
     return true;
 }
 
-int launch_moe_gemm(const void *a, long long rows, const float *a_scale, const void *b, const float *b_scale, int E,
-                    int N, int K, const int *tile_expert, const float *row_weight, float *out, int sms, cudaStream_t s) {
-    using Cfg = ave::MoeGemmCfg;
-    CUtensorMap ta, tb, tc;
-    if (!encode_map_u8(&ta, a, K, rows, 1, Cfg::kTile)) return AVE_ERR_CUDA;
-    if (!encode_map_u8(&tb, b, K, N, E, Cfg::kTileN)) return AVE_ERR_CUDA;
-    if (!encode_map_f32(&tc, out, N, rows)) return AVE_ERR_CUDA;
-    ave::MoeGemmParams p;
-    p.a_scale = a_scale;
-    p.b_scale = b_scale;
-    p.tile_expert = tile_expert;
-    p.row_weight = row_weight;
-    p.out = out;
-    p.tiles_m = int(rows / 128);
-    p.tiles_n = (N + Cfg::kTileN - 1) / Cfg::kTileN;
+// One GEMM of the layer: A codes [rows_cap, K], B codes [E, N, K]; `out` (down projection): fp32 [rows_cap, N].
+template <bool UP>
+int launch_moe_gemm(const void *a, const void *b, int E, int N, int K, float *out, ave::MoeGemmParams p, int sms, cudaStream_t s) {
+    using Cfg = ave::MoeGemmCfg<UP>;
+    CUtensorMap ta, tb, tc{};
+    if (!encode_map_u8(&ta, a, K, p.rows_cap, 1, Cfg::kBoxRows)) return AVE_ERR_CUDA;
+    if (!encode_map_u8(&tb, b, K, N, E, 128)) return AVE_ERR_CUDA;
+    if (!UP && !encode_map_f32(&tc, out, N, p.rows_cap)) return AVE_ERR_CUDA;
     p.nblk = N / 128;
+    p.tiles_n = (p.nblk + 1) / 2;  // 256 columns per tile (up: 128 of the gate and 128 of the up half)
     p.kb = K / 128;
-    p.N = N;
-    static PerDeviceOnce once;
-    const int st = prepare_kernel(ave::moe_gemm_fp8_kernel, Cfg::kSmemBytes, 3, once);
+    auto kern = ave::moe_gemm_fp8_kernel<UP>;
+    static PerDeviceOnce once;  // per instantiation
+    const int st = prepare_kernel(kern, Cfg::kSmemBytes, 3, once);
     if (st != AVE_OK) return st;
     if (take_injected(g_inject_launch_failures)) {
         t_last_cuda_error = int(cudaErrorLaunchFailure);
         return AVE_ERR_CUDA;
     }
-    const long long n_tiles = (long long)p.tiles_m * p.tiles_n;
+    const long long n_tiles = p.rows_cap / 128 * p.tiles_n;
     const unsigned grid = unsigned(n_tiles < sms ? n_tiles : sms);
-    ave::moe_gemm_fp8_kernel<<<dim3(grid), dim3(Cfg::kThreads), Cfg::kSmemBytes, s>>>(ta, tb, tc, p);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_dependent(kern, dim3(grid), dim3(Cfg::kThreads), Cfg::kSmemBytes, s, ta, tb, tc, p);
     if (e != cudaSuccess) {
         t_last_cuda_error = int(e);
         return AVE_ERR_CUDA;
@@ -725,9 +715,8 @@ int launch_moe_gemm(const void *a, long long rows, const float *a_scale, const v
     return AVE_OK;
 }
 
-// One of the layer's small kernels has been launched: count it or report the launch error.
-int after_small_launch() {
-    cudaError_t e = cudaGetLastError();
+// One of the layer's small kernels has been launched with status e: count it or report the launch error.
+int after_small_launch(cudaError_t e) {
     if (e != cudaSuccess) {
         t_last_cuda_error = int(e);
         return AVE_ERR_CUDA;
@@ -771,48 +760,52 @@ int ave_moe_fused_fwd(const void *xq, const float *sx, const void *w13q, const f
     uint8_t *base = static_cast<uint8_t *>(workspace);
     uint8_t *xq_s = base + w.xq_s;
     float *sx_s = reinterpret_cast<float *>(base + w.sx_s);
-    float *ho = reinterpret_cast<float *>(base + w.ho);
+    float *o = reinterpret_cast<float *>(base + w.o);
     uint8_t *aq = base + w.aq;
     float *sa = reinterpret_cast<float *>(base + w.sa);
     int *row_of = reinterpret_cast<int *>(base + w.row_of);
-    int *pair_of = reinterpret_cast<int *>(base + w.pair_of);
     float *w_s = reinterpret_cast<float *>(base + w.w_s);
-    int *expert_off = reinterpret_cast<int *>(base + w.expert_off);
+    int *counts = reinterpret_cast<int *>(base + w.counts);
     int *cursor = reinterpret_cast<int *>(base + w.cursor);
-    int *tile_expert = reinterpret_cast<int *>(base + w.tile_expert);
-    int *bad_id = reinterpret_cast<int *>(base + w.bad_id);
+    ave::MoeRowTile *tiles = reinterpret_cast<ave::MoeRowTile *>(base + w.tiles);
+    int *n_row_tiles = reinterpret_cast<int *>(base + w.n_row_tiles);
     const int pairs = T * K;
-    const int rows = int(w.rows_cap);
 
-    // 1. sort the (token, k) pairs by expert
-    ave::moe_count_kernel<<<1, 1024, size_t(E) * sizeof(int), s>>>(ids, pairs, E, rows, expert_off, cursor, tile_expert,
-                                                                  pair_of, bad_id);
-    if ((st = after_small_launch()) != AVE_OK) return st;
-    ave::moe_scatter_kernel<<<(pairs + 255) / 256, 256, 0, s>>>(ids, pairs, E, expert_off, cursor, row_of, pair_of);
-    if ((st = after_small_launch()) != AVE_OK) return st;
-    // 2. the tokens' codes and scales in sorted order
-    ave::moe_gather_kernel<<<rows, 128, 0, s>>>(static_cast<const uint8_t *>(xq), sx, wts, pair_of, tile_expert, C, K, xq_s,
-                                               sx_s, w_s);
-    if ((st = after_small_launch()) != AVE_OK) return st;
-    // 3. up projection: h = x W13^T
-    st = launch_moe_gemm(xq_s, rows, sx_s, w13q, s13, E, 2 * F, C, tile_expert, nullptr, ho, sms, s);
+    // 1.-3. pairs per expert, rows and row tiles of every expert
+    ave::moe_clear_kernel<<<1, 256, 0, s>>>(counts, E);
+    if ((st = after_small_launch(cudaGetLastError())) != AVE_OK) return st;
+    const int count_ctas = (pairs + 2047) / 2048 < 2 * sms ? (pairs + 2047) / 2048 : 2 * sms;
+    st = after_small_launch(launch_dependent(ave::moe_count_kernel, dim3(count_ctas), dim3(512), size_t(E) * sizeof(int), s, ids,
+                                             pairs, E, counts));
     if (st != AVE_OK) return st;
-    // 4. activation and requantisation
-    {
-        const long long warps = (long long)rows * (F / 128);
-        ave::moe_act_quant_kernel<<<unsigned((warps + 7) / 8), 256, 0, s>>>(ho, tile_expert, F, rows, aq, sa);
-        if ((st = after_small_launch()) != AVE_OK) return st;
-    }
-    // 5. down projection, weighted: o = w * (a W2^T)
-    st = launch_moe_gemm(aq, rows, sa, w2q, s2, E, C, F, tile_expert, w_s, ho, sms, s);
+    st = after_small_launch(launch_dependent(ave::moe_plan_kernel, dim3(1), dim3(1024), 0, s, counts, E, cursor, tiles, n_row_tiles));
     if (st != AVE_OK) return st;
-    // 6. every token's K rows summed
-    {
-        const long long n = (long long)T * (C / 4);
-        ave::moe_combine_kernel<<<unsigned((n + 255) / 256), 256, 0, s>>>(ho, row_of, T, C, K, static_cast<__nv_bfloat16 *>(y));
-        if ((st = after_small_launch()) != AVE_OK) return st;
-    }
-    return AVE_OK;
+    // 4. the tokens' codes and scales in sorted order
+    st = after_small_launch(launch_dependent(ave::moe_gather_kernel, dim3(T), dim3(ave::kMoeGatherThreads), 0, s,
+                                             static_cast<const uint8_t *>(xq), sx, ids, wts, C, E, K, w.rows_cap, cursor, row_of, xq_s,
+                                             sx_s, w_s));
+    if (st != AVE_OK) return st;
+    // 5. up projection, activation and requantisation
+    ave::MoeGemmParams p{};
+    p.tiles = tiles;
+    p.n_row_tiles = n_row_tiles;
+    p.rows_cap = w.rows_cap;
+    p.a_scale = sx_s;
+    p.b_scale = s13;
+    p.q_out = aq;
+    p.q_scale = sa;
+    st = launch_moe_gemm<true>(xq_s, w13q, E, 2 * F, C, nullptr, p, sms, s);
+    if (st != AVE_OK) return st;
+    // 6. down projection, weighted: o = w * (a W2^T)
+    p.a_scale = sa;
+    p.b_scale = s2;
+    p.row_weight = w_s;
+    st = launch_moe_gemm<false>(aq, w2q, E, C, F, o, p, sms, s);
+    if (st != AVE_OK) return st;
+    // 7. every token's K rows summed
+    const long long n = (long long)T * (C / 4);
+    return after_small_launch(launch_dependent(ave::moe_combine_kernel, dim3(unsigned((n + 255) / 256)), dim3(256), 0, s, o, row_of, T,
+                                               C, K, static_cast<__nv_bfloat16 *>(y)));
 }
 
 int ave_attn_fwd(const void *q, const void *k, const void *v, void *o, float *lse, int B, int H, int Hkv, int Sq,

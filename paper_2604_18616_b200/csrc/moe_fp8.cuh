@@ -4,24 +4,29 @@
 //
 // Format: E4M3 codes; activations carry one fp32 scale per (token, 128 channels), weights one per 128 x 128
 // block.  Steps of one call (all on the caller's stream, scratch in the caller's workspace):
-//   1. moe_count_kernel / moe_scatter_kernel: (token, k) pairs sorted by expert; every expert's rows start on
-//      a multiple of 128, so a 128-row tile of the sorted order belongs to one expert
-//   2. moe_gather_kernel: the tokens' codes and scales copied into the sorted order (padding rows are zero)
-//   3. moe_gemm_fp8_kernel: h = x W13^T, rows x 2F, fp32       (grouped by expert, block-scaled, tensor cores)
-//   4. moe_act_quant_kernel: a = silu(gate) * up, requantised to E4M3 per 128 columns, fp32 scale
-//   5. moe_gemm_fp8_kernel: o = w * (a W2^T), rows x C, fp32   (w: the pair's routing weight)
-//   6. moe_combine_kernel: y[t] = sum over the token's K rows of o, rounded to bf16
+//   1. moe_clear_kernel, 2. moe_count_kernel, 3. moe_plan_kernel: pairs per expert, every expert's first row in the
+//      sorted order (a multiple of 128, so a 128-row tile belongs to one expert), the list of row tiles
+//   4. moe_gather_kernel: every (token, k) pair gets a row of its expert; the token's codes and scales are copied there
+//   5. moe_gemm_fp8_kernel<true>: a = silu(x Wg^T) * (x Wu^T), requantised to E4M3 per 128 columns (grouped by expert,
+//      block-scaled, tensor cores)
+//   6. moe_gemm_fp8_kernel<false>: o = w * (a W2^T), rows x C, fp32   (w: the pair's routing weight)
+//   7. moe_combine_kernel: y[t] = sum over the token's K rows of o, rounded to bf16
+// Kernels 2 to 7 are launched with programmatic stream serialisation; each waits for the one before it at its top.
 //
 // The GEMM: persistent CTAs over 128 x 256 output tiles; K is streamed in blocks of 128 (one scale block)
-// through a TMA ring; each block is four M128 x N256 x K32 tcgen05 MMAs (kind::f8f6f4) into one of two TMEM
+// through a TMA ring; each block is four M128 x N256 x K32 tcgen05 MMAs (kind::f8f6f4, 512 clk) into one of two TMEM
 // accumulators, which the epilogue warps read out and add, multiplied by the block's scales, to fp32
 // registers (the accumulation across scale blocks cannot stay in the tensor core: every block has its own
-// factor).  Rows are TMEM lanes; two epilogue threads per row, 128 columns (one weight scale block) each.
+// factor).  Rows are TMEM lanes; two epilogue threads per row, 128 columns each.  Adding a block up takes 350 clk of
+// the 512 (bound by the issue of its FMAs), so the read-out keeps up only if its loop does nothing else: a warp
+// of its own fetches the scales, blocks ahead, and leaves each block's in shared memory; "accumulator full" then stands for
+// the products and their scales.  (With every epilogue thread fetching its own scales a block took 1150-1400 clk.)
+// In the up projection a tile is 128 gate columns and the same 128 up columns (one requantisation group); a thread
+// holds 64 of each, so the activation needs no exchange but the group's maximum.
 //
 //   warp 0       producer: TMA loads of the A and B blocks
-//   warp 1       MMA issuer
-//   warp 2       TMEM allocation / release
-//   warp 3       -
+//   warps 1, 2   MMA issuers (even and odd K blocks); warp 2 also allocates and releases TMEM
+//   warp 3       scales
 //   warps 4..11  epilogue (thread = output row x half of the tile's columns)
 #pragma once
 
@@ -33,35 +38,51 @@ namespace ave {
 
 constexpr int kMoeGroup = 128;  // channels per activation scale, rows and columns per weight scale block
 
+template <bool UP>
 struct MoeGemmCfg {
     static constexpr int kThreads = 384;
     static constexpr int kTile = 128;                          // rows of an output tile; K block; columns per epilogue thread
-    static constexpr int kTileN = 256;                         // columns of an output tile
-    static constexpr int kStages = 4;
+    static constexpr int kTileN = 256;                         // columns of an output tile (two weight scale blocks)
+    static constexpr int kBoxRows = 32;                        // rows of A per TMA load: only 32-row groups with a token are loaded
+    // The down projection's tiles have few K blocks and a large fp32 result: it trades a ring slot for a second
+    // staging buffer per epilogue warp, so that a tile's stores do not wait for one another.
+    static constexpr int kStages = UP ? 4 : 3;
+    static constexpr int kStoreBufs = 2;
     static constexpr int kABytes = kTile * kMoeGroup;          // 16 KB of E4M3
     static constexpr int kBBytes = kTileN * kMoeGroup;         // 32 KB
     static constexpr int kStageBytes = kABytes + kBBytes;
-    static constexpr int kStageCBytes = 8 * 32 * 128;          // result staging: 32 rows x 32 fp32 per epilogue warp
-    static constexpr int kSmemBytes = kStages * kStageBytes + kStageCBytes + 1024;
+    static constexpr int kStageCBytes = 8 * kStoreBufs * 32 * 128;  // result staging: buffers of 32 rows x 32 fp32 per epilogue warp
+    static constexpr int kSmemBytes = kStages * kStageBytes + (UP ? 0 : kStageCBytes) + 1024;
     static constexpr int kAccs = 2;                            // TMEM accumulators of 256 columns
     static constexpr uint32_t kTmemCols = kAccs * kTileN;
-    // The epilogue threads hold 128 fp32 sums plus two 32-column chunks in flight: they take registers from the
+    // The epilogue threads hold 128 fp32 sums plus a 32-column chunk in flight: they take registers from the
     // producer / MMA warpgroup (setmaxnreg moves them inside the CTA's allocation of kThreads x kRegsAtLaunch;
     // the build and the launch code check the compiled image against this split).
-    static constexpr int kRegsLight = 40, kRegsEpilogue = 232, kRegsAtLaunch = 168;
+    static constexpr int kRegsLight = 56, kRegsEpilogue = 224, kRegsAtLaunch = 168;
     static_assert(128 * kRegsLight + 256 * kRegsEpilogue <= kThreads * kRegsAtLaunch, "register split exceeds the CTA's allocation");
 };
 
+// One 128-row tile of the sorted order.  Row tiles of an expert are visited in groups (of at most kMoeGroupTiles), all of a
+// group's row tiles under one column tile before the next column tile, so that weights are read from HBM about once.
+constexpr int kMoeGroupTiles = 8;
+struct __align__(16) MoeRowTile {
+    int expert;
+    int group_first, group_tiles;  // the group this tile belongs to
+    int rows;                      // rows of this tile that hold a token (the rest is padding: whatever is there is never used)
+};
+
 struct MoeGemmParams {
-    const float *a_scale;     // [rows, K/128]
-    const float *b_scale;     // [E, N/128, K/128]
-    const int *tile_expert;   // [rows/128]: expert of each 128-row tile of the sorted order, -1 = unused tile
-    const float *row_weight;  // [rows] or NULL: factor applied to every output row
-    float *out;               // [rows, N] fp32
-    int tiles_m, tiles_n;     // rows / 128, ceil(N / 256)
-    int nblk;                 // N / 128: weight scale blocks along N
-    int kb;                   // K / 128
-    int N;
+    const float *a_scale;       // [K/128, rows_cap]
+    const float *b_scale;       // [E, N/128, K/128]
+    const MoeRowTile *tiles;    // [tiles in use]
+    const int *n_row_tiles;     // row tiles in use
+    const float *row_weight;    // down projection: [rows_cap], factor applied to every output row
+    uint8_t *q_out;             // up projection: codes [rows_cap, F] and scales [F/128, rows_cap]
+    float *q_scale;
+    long long rows_cap;
+    int tiles_n;                // up: F / 128; down: ceil(N / 256)
+    int nblk;                   // weight scale blocks along N: up 2F / 128, down N / 128
+    int kb;                     // K / 128
 };
 
 // tcgen05 instruction descriptor, kind::f8f6f4: fp32 accumulator, E4M3 A and B, both K-major.
@@ -88,30 +109,67 @@ __device__ __forceinline__ void umma_f8_ss_words(uint32_t d_tmem, uint32_t a_lo,
         : "memory");
 }
 
-// Output tile number -> (row tile, column tile): groups of 4 row tiles (about one expert's rows at the paper's
-// sizes), column-major inside a group, so that CTAs at work together share a few experts' weights in L2.
-__device__ __forceinline__ void moe_tile_coords(int id, const MoeGemmParams &p, int &bm, int &bn) {
-    constexpr int kGroupM = 4;
-    const int per_group = kGroupM * p.tiles_n;
-    const int grp = id / per_group;
-    const int rem = id - grp * per_group;
-    const int m0 = grp * kGroupM;
-    const int gm = min(kGroupM, p.tiles_m - m0);
-    bn = rem / gm;
-    bm = m0 + (rem - bn * gm);
+// The n-th output tile of the launch: row tile, column tile, the row tile's record.
+__device__ __forceinline__ MoeRowTile moe_tile(int id, const MoeGemmParams &p, int &bm, int &bn) {
+    const int r = id / p.tiles_n;  // a group of row tiles owns the ids [group_first, group_first + group_tiles) * tiles_n
+    const MoeRowTile g = p.tiles[r];
+    const int rem = id - g.group_first * p.tiles_n;
+    bn = rem / g.group_tiles;
+    bm = g.group_first + (rem - bn * g.group_tiles);
+    return p.tiles[bm];
 }
 
-// tm_a: A codes [rows, K] as {K, rows, 1, 1}, boxes of 128 bytes x 128 rows; tm_b: B codes [E, N, K] as
-// {K, N, E, 1}, boxes of 128 bytes x 256 rows (rows beyond N read as zero); tm_c: the fp32 result [rows, N] as
-// {N, rows, 1, 1}, boxes of 32 columns x 32 rows (a thread-per-row store of fp32 rows would touch 32 rows per
-// instruction, one sector each: measured, that cost more than the tile's products).
+// Two fp32 values -> two E4M3 codes (round to nearest even, saturating at +-448); `lo` lands in bits 0..7.
+__device__ __forceinline__ uint32_t cvt_e4m3x2(float lo, float hi) {
+    uint16_t r;
+    asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(r) : "f"(hi), "f"(lo));
+    return r;
+}
+
+// x / d for two values, given r = 1 / d to within an ulp: one residual step, q + (x - q d) r with the residual exact in an
+// FMA (Markstein, IBM J. Res. Dev. 34, 1990).  Nothing here may overflow or be subnormal: the callers see to it.
+__device__ __forceinline__ float2 div2_residual(float2 x, float2 d, float2 r) {
+    const float2 q = __fmul2_rn(x, r);
+    const float2 e = __ffma2_rn(make_float2(-q.x, -q.y), d, x);
+    return __ffma2_rn(e, r, q);
+}
+// silu(z) = z / (1 + exp(-z)) for two values in fp32.  Below -87 the exponential is held at exp(87): the result is then
+// z * 1.6e-38 instead of a subnormal or zero.
+__device__ __forceinline__ float2 silu2(float2 z) {
+    const float2 d = make_float2(1.f + expf(-fmaxf(z.x, -87.f)), 1.f + expf(-fmaxf(z.y, -87.f)));
+    float2 r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r.x) : "f"(d.x));
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r.y) : "f"(d.y));
+    const float2 nd = make_float2(-d.x, -d.y);
+    r = __ffma2_rn(__ffma2_rn(nd, r, make_float2(1.f, 1.f)), r, r);  // one Newton step
+    return div2_residual(z, d, r);
+}
+
+// Keeps the additions to 16 pairs of sums ahead of what follows: the compiler otherwise loads further blocks of products
+// first and, with 128 sums in registers, spills.
+__device__ __forceinline__ void pin_sums(float2 *a) {
+    asm volatile("" : "+f"(a[0].x), "+f"(a[0].y), "+f"(a[1].x), "+f"(a[1].y), "+f"(a[2].x), "+f"(a[2].y), "+f"(a[3].x), "+f"(a[3].y),
+          "+f"(a[4].x), "+f"(a[4].y), "+f"(a[5].x), "+f"(a[5].y), "+f"(a[6].x), "+f"(a[6].y), "+f"(a[7].x), "+f"(a[7].y));
+    asm volatile("" : "+f"(a[8].x), "+f"(a[8].y), "+f"(a[9].x), "+f"(a[9].y), "+f"(a[10].x), "+f"(a[10].y), "+f"(a[11].x), "+f"(a[11].y),
+          "+f"(a[12].x), "+f"(a[12].y), "+f"(a[13].x), "+f"(a[13].y), "+f"(a[14].x), "+f"(a[14].y), "+f"(a[15].x), "+f"(a[15].y));
+}
+
+// UP: the up projection with activation and requantisation; else the down projection.
+// tm_a: A codes [rows_cap, K] as {K, rows_cap, 1, 1}, boxes of 128 bytes x 32 rows; tm_b: B codes [E, N, K] as
+// {K, N, E, 1}, boxes of 128 bytes x 128 rows (rows beyond N read as zero); tm_c: the down projection's fp32 result
+// [rows_cap, N] as {N, rows_cap, 1, 1}, boxes of 32 columns x 32 rows (a thread-per-row store of fp32 rows would touch 32
+// rows per instruction, one sector each: measured, that cost more than the tile's products).
+template <bool UP>
 __global__ void __launch_bounds__(384, 1)
 moe_gemm_fp8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b,
                     const __grid_constant__ CUtensorMap tm_c, const MoeGemmParams p) {
-    using Cfg = MoeGemmCfg;
+    using Cfg = MoeGemmCfg<UP>;
     constexpr int NS = Cfg::kStages, NA = Cfg::kAccs;
     extern __shared__ uint8_t smem_raw[];
-    __shared__ __align__(8) uint64_t bar_full[NS], bar_empty[NS], bar_acc_full[NA], bar_acc_empty[NA], bar_drain;
+    __shared__ __align__(8) uint64_t bar_full[NS], bar_empty[NS], bar_acc_full[NA], bar_acc_empty[NA], bar_pair[4], bar_drain[NA];
+    __shared__ float row_max[UP ? 2 : 1][2][UP ? Cfg::kTile : 1];  // [tile parity][half of the columns][row]
+    __shared__ __align__(16) float row_scale[NA][Cfg::kTile];  // scales of the K block in each accumulator: the rows',
+    __shared__ __align__(8) float2 col_scale[NA];              // and those of its two weight blocks
     __shared__ uint32_t tmem_base_slot;
     __shared__ int abort_flag;
 
@@ -121,22 +179,27 @@ moe_gemm_fp8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
     const uint32_t sRing = (smem_u32(smem_raw) + 1023u) & ~1023u;
 
     if (tid == 0) {
-        abort_flag = (*reinterpret_cast<volatile unsigned int *>(&g_device_status) != 0) ? 1 : 0;
         for (int s = 0; s < NS; ++s) {
             mbar_init(smem_u32(&bar_full[s]), 1);
             mbar_init(smem_u32(&bar_empty[s]), 1);
         }
         for (int a = 0; a < NA; ++a) {
-            mbar_init(smem_u32(&bar_acc_full[a]), 1);
+            mbar_init(smem_u32(&bar_acc_full[a]), 2);   // the MMAs' commit and the scale warp
             mbar_init(smem_u32(&bar_acc_empty[a]), 8);  // one arrival per epilogue warp
         }
-        mbar_init(smem_u32(&bar_drain), 1);
+        for (int x = 0; x < 4; ++x) mbar_init(smem_u32(&bar_pair[x]), 2);  // the two warps of a row
+        for (int a = 0; a < NA; ++a) mbar_init(smem_u32(&bar_drain[a]), 1);
         fence_mbar_init();
+        tma_prefetch_desc(&tm_a);
+        tma_prefetch_desc(&tm_b);
     }
     if (warp == 2) {
         tmem_alloc(smem_u32(&tmem_base_slot), Cfg::kTmemCols);
         tmem_relinquish();
     }
+    grid_dependency_wait();
+    grid_dependency_launch();
+    if (tid == 0) abort_flag = (*reinterpret_cast<volatile unsigned int *>(&g_device_status) != 0) ? 1 : 0;
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -148,7 +211,7 @@ moe_gemm_fp8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
         return __all_sync(0xffffffffu, r);
     };
 
-    const int n_tiles = p.tiles_m * p.tiles_n;
+    const int n_tiles = *p.n_row_tiles * p.tiles_n;
 
     if (poisoned) {
         // nothing: fall through to the common exit
@@ -157,17 +220,13 @@ moe_gemm_fp8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
       if (warp == 0) {
         // =============================== producer ===============================
         const bool leader = elect_one();
-        if (leader) {
-            tma_prefetch_desc(&tm_a);
-            tma_prefetch_desc(&tm_b);
-        }
         bool ok = true;
         int ring = 0;  // K blocks loaded so far
-        for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
+        for (int id = blockIdx.x; id < n_tiles && ok; id += gridDim.x) {
             int bm, bn;
-            moe_tile_coords(tile, p, bm, bn);
-            const int e = p.tile_expert[bm];
-            if (e < 0) continue;  // a row tile beyond the sorted rows
+            const MoeRowTile t = moe_tile(id, p, bm, bn);
+            const int boxes = (t.rows + Cfg::kBoxRows - 1) / Cfg::kBoxRows;
+            const int n0 = UP ? bn * 128 : bn * 256, n1 = UP ? (p.nblk / 2 + bn) * 128 : bn * 256 + 128;  // rows of B
             for (int kb = 0; kb < p.kb && ok; ++kb, ++ring) {
                 const int slot = ring % NS, round = ring / NS;
                 if (round > 0) {
@@ -177,9 +236,12 @@ moe_gemm_fp8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
                 if (leader) {
                     const uint32_t bar = smem_u32(&bar_full[slot]);
                     const uint32_t dst = sRing + slot * Cfg::kStageBytes;
-                    mbar_arrive_expect_tx(bar, Cfg::kStageBytes);
-                    tma_load_4d(dst, &tm_a, bar, kb * kMoeGroup, bm * Cfg::kTile, 0, 0);
-                    tma_load_4d(dst + Cfg::kABytes, &tm_b, bar, kb * kMoeGroup, bn * Cfg::kTileN, e, 0);
+                    mbar_arrive_expect_tx(bar, boxes * (Cfg::kBoxRows * kMoeGroup) + Cfg::kBBytes);
+                    tma_load_4d(dst + Cfg::kABytes, &tm_b, bar, kb * kMoeGroup, n0, t.expert, 0);
+                    tma_load_4d(dst + Cfg::kABytes + Cfg::kBBytes / 2, &tm_b, bar, kb * kMoeGroup, n1, t.expert, 0);
+                    for (int x = 0; x < boxes; ++x)
+                        tma_load_4d(dst + x * (Cfg::kBoxRows * kMoeGroup), &tm_a, bar, kb * kMoeGroup,
+                                    bm * Cfg::kTile + x * Cfg::kBoxRows, 0, 0);
                 }
             }
         }
@@ -187,121 +249,222 @@ moe_gemm_fp8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
             for (int it = max(0, ring - NS); it < ring; ++it)
                 for (uint32_t w = 0; w < WAIT_LIMIT && !mbar_test_wait(smem_u32(&bar_full[it % NS]), (it / NS) & 1); ++w) {}
         }
-    } else if (warp == 1) {
-        // =============================== MMA issuer ===============================
-        const bool leader = elect_one();
-        constexpr uint32_t idesc = make_idesc_e4m3(Cfg::kTile, Cfg::kTileN);
-        constexpr uint64_t desc_kmajor = make_sdesc_sw128(16, 1024);  // rows of 128 bytes, 8-row atoms of 1024 bytes
-        constexpr uint32_t hi = uint32_t(desc_kmajor >> 32), lo = uint32_t(desc_kmajor);
-        bool ok = true;
-        int ring = 0;  // K blocks issued so far = accumulators filled so far
-        for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
-            int bm, bn;
-            moe_tile_coords(tile, p, bm, bn);
-            if (p.tile_expert[bm] < 0) continue;
-            for (int kb = 0; kb < p.kb && ok; ++kb, ++ring) {
-                const int slot = ring % NS, acc = ring % NA;
-                if (ring >= NA) {  // the epilogue must have read this accumulator's previous block out of TMEM
-                    ok = wait_bar(&bar_acc_empty[acc], ((ring / NA) - 1) & 1, STATUS_TIMEOUT_SOFTMAX);
-                    if (!ok) break;
-                }
-                ok = wait_bar(&bar_full[slot], (ring / NS) & 1, STATUS_TIMEOUT_LOAD);
+      } else if (warp < 3) {
+        // =============================== MMA issuers ===============================
+        // Warp 1 issues the even K blocks (into accumulator 0), warp 2 the odd ones: issuing blocks the thread for about as
+        // long as the MMAs take, so with one issuer the tensor pipe stood still while it went through the next
+        // block's barriers (a ready wait costs some 100 clk; a block took 900 clk for 512 of work).
+        static_assert(NA == 2, "one issuer per accumulator");
+        if (elect_one()) {
+            constexpr uint32_t idesc = make_idesc_e4m3(Cfg::kTile, Cfg::kTileN);
+            constexpr uint64_t desc_kmajor = make_sdesc_sw128(16, 1024);  // rows of 128 bytes, 8-row atoms of 1024 bytes
+            constexpr uint32_t hi = uint32_t(desc_kmajor >> 32), lo = uint32_t(desc_kmajor);
+            const int acc = warp - 1;
+            const uint32_t d_tmem = tmem + acc * Cfg::kTileN;
+            int n_blocks = 0;  // K blocks of this CTA
+            for (int id = blockIdx.x; id < n_tiles; id += gridDim.x) n_blocks += p.kb;
+            bool ok = true;
+            for (int ring = acc; ring < n_blocks; ring += NA) {
+                const int slot = ring % NS;
+                // Polled, not slept on: what passes from a barrier's completion to the first MMA is idle time of the tensor pipe.
+                // The accumulator's wait (the epilogue must have read its previous block out of TMEM) comes last where
+                // the ring allows it.  It does if this issuer sees every use of a slot: with an odd number of slots the
+                // other issuer takes every second one, and "full" has only two phases to tell uses apart; there the
+                // accumulator comes first, because by then the epilogue has gone past the other issuer's use.
+                auto wait_full = [&]() { return mbar_poll_bounded(smem_u32(&bar_full[slot]), (ring / NS) & 1, &abort_flag, STATUS_TIMEOUT_LOAD); };
+                if (NS % NA == 0) ok = wait_full();
+                if (ok && ring >= NA)
+                    ok = mbar_poll_bounded(smem_u32(&bar_acc_empty[acc]), ((ring / NA) - 1) & 1, &abort_flag, STATUS_TIMEOUT_SOFTMAX);
+                if (ok && NS % NA != 0) ok = wait_full();
                 if (!ok) break;
                 tc_fence_after();
-                if (leader) {
-                    const uint32_t a_lo = lo | ((sRing + slot * Cfg::kStageBytes) >> 4);
-                    const uint32_t b_lo = lo | ((sRing + slot * Cfg::kStageBytes + Cfg::kABytes) >> 4);
-                    const uint32_t d_tmem = tmem + acc * Cfg::kTileN;
+                const uint32_t a_lo = lo | ((sRing + slot * Cfg::kStageBytes) >> 4);
+                const uint32_t b_lo = lo | ((sRing + slot * Cfg::kStageBytes + Cfg::kABytes) >> 4);
 #pragma unroll
-                    for (int kk = 0; kk < kMoeGroup / 32; ++kk)  // K = 32 bytes per instruction
-                        umma_f8_ss_words(d_tmem, a_lo + ((kk * 32) >> 4), hi, b_lo + ((kk * 32) >> 4), hi, idesc, kk > 0);
-                    umma_commit(smem_u32(&bar_empty[slot]));
-                    umma_commit(smem_u32(&bar_acc_full[acc]));
-                }
+                for (int kk = 0; kk < kMoeGroup / 32; ++kk)  // K = 32 bytes per instruction
+                    umma_f8_ss_words(d_tmem, a_lo + ((kk * 32) >> 4), hi, b_lo + ((kk * 32) >> 4), hi, idesc, kk > 0);
+                umma_commit(smem_u32(&bar_empty[slot]));
+                umma_commit(smem_u32(&bar_acc_full[acc]));
+            }
+            if (!ok) {  // abandoned: let the MMAs already issued finish before TMEM is released
+                umma_commit(smem_u32(&bar_drain[acc]));
+                for (uint32_t w = 0; w < WAIT_LIMIT && !mbar_test_wait(smem_u32(&bar_drain[acc]), 0); ++w) {}
             }
         }
-        if (!ok) {  // abandoned: let the MMAs already issued finish before TMEM is released
-            if (leader) umma_commit(smem_u32(&bar_drain));
-            for (uint32_t w = 0; w < WAIT_LIMIT && !mbar_test_wait(smem_u32(&bar_drain), 0); ++w) {}
+        __syncwarp();
+      } else if (warp == 3) {
+        // =============================== scales ===============================
+        constexpr int kAhead = 4;  // K blocks fetched ahead
+        bool ok = true;
+        int ring = 0;
+        for (int id = blockIdx.x; id < n_tiles && ok; id += gridDim.x) {
+            int bm, bn;
+            const MoeRowTile t = moe_tile(id, p, bm, bn);
+            const float *sa = p.a_scale + bm * Cfg::kTile + lane * 4;
+            // weight blocks of the tile's two halves (the last tile's second may lie beyond N: any value will do)
+            const int nb0 = UP ? bn : bn * 2, nb1 = UP ? p.nblk / 2 + bn : min(bn * 2 + 1, p.nblk - 1);
+            const float *sb = p.b_scale + (size_t(t.expert) * p.nblk + (lane == 0 ? nb0 : nb1)) * p.kb;
+            float4 ra[kAhead];
+            float rb[kAhead];
+            auto fetch = [&](int kb, float4 &a, float &b) {
+                kb = min(kb, p.kb - 1);
+                a = *reinterpret_cast<const float4 *>(sa + kb * p.rows_cap);
+                if (lane < 2) b = sb[kb];
+            };
+#pragma unroll
+            for (int x = 0; x < kAhead; ++x) fetch(x, ra[x], rb[x]);
+#pragma unroll 1
+            for (int kb0 = 0; kb0 < p.kb && ok; kb0 += kAhead) {
+#pragma unroll
+                for (int x = 0; x < kAhead; ++x) {
+                    if (kb0 + x >= p.kb) break;
+                    const int acc = ring % NA;
+                    if (ring >= NA) {
+                        ok = wait_bar(&bar_acc_empty[acc], ((ring / NA) - 1) & 1, STATUS_TIMEOUT_SOFTMAX);
+                        if (!ok) break;
+                    }
+                    ++ring;
+                    *reinterpret_cast<float4 *>(&row_scale[acc][lane * 4]) = ra[x];
+                    if (lane < 2) reinterpret_cast<float *>(&col_scale[acc])[lane] = rb[x];
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(smem_u32(&bar_acc_full[acc]));
+                    fetch(kb0 + x + kAhead, ra[x], rb[x]);
+                }
+            }
         }
       }
     } else {
         // =============================== epilogue ===============================
         setmaxnreg_inc<Cfg::kRegsEpilogue>();
         const int wq = warp & 3;           // TMEM lane quadrant of this warp
-        const int half = (warp - 4) >> 2;  // which 128 of the tile's 256 columns
+        const int half = (warp - 4) >> 2;  // which half of the tile's columns
         const uint32_t lane_sel = uint32_t(wq * 32) << 16;
-        const uint32_t sC = sRing + NS * Cfg::kStageBytes + (warp - 4) * (32 * 128);  // this warp's 32 staging rows
-        bool store_pending = false;  // (lane 0) a TMA store may still be reading the staging rows
+        const uint32_t sC = sRing + NS * Cfg::kStageBytes + (warp - 4) * (Cfg::kStoreBufs * 32 * 128);  // this warp's staging buffers
         bool ok = true;
         int ring = 0;
-        for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
+        uint32_t n_done = 0;         // tiles this warp has finished (up projection: phase of bar_pair)
+        for (int id = blockIdx.x; id < n_tiles && ok; id += gridDim.x) {
             int bm, bn;
-            moe_tile_coords(tile, p, bm, bn);
-            const int e = p.tile_expert[bm];
-            if (e < 0) continue;
+            const MoeRowTile t = moe_tile(id, p, bm, bn);
+            const int nb = UP ? bn : bn * 2 + half;  // this thread's weight scale block along N (up: and F/128 further on)
+            if (wq * 32 >= t.rows || nb >= p.nblk) {
+                // no token among this warp's rows, or its half lies beyond N: only hand the accumulators back
+                for (int kb = 0; kb < p.kb && ok; ++kb, ++ring) {
+                    ok = wait_bar(&bar_acc_full[ring % NA], (ring / NA) & 1, STATUS_TIMEOUT_MMA);
+                    if (ok && lane == 0) mbar_arrive(smem_u32(&bar_acc_empty[ring % NA]));
+                }
+                continue;
+            }
             const int row = bm * Cfg::kTile + wq * 32 + lane;
-            const int nb = bn * 2 + half;              // this thread's weight scale block along N
-            const bool live = nb < p.nblk;             // (the last tile's second half lies beyond N when N % 256 == 128)
-            const float *sa = p.a_scale + size_t(row) * p.kb;
-            const float *sb = p.b_scale + (size_t(e) * p.nblk + (live ? nb : 0)) * p.kb;
-            float acc[Cfg::kTile];
+            float2 acc[Cfg::kTile / 2];  // up: 64 gate columns, then 64 up columns; down: 128 columns
 #pragma unroll
-            for (int c = 0; c < Cfg::kTile; ++c) acc[c] = 0.f;
-            float s_next = sa[0] * sb[0];
-            for (int kb = 0; kb < p.kb && ok; ++kb, ++ring) {
-                const float s = s_next;
-                if (kb + 1 < p.kb) s_next = sa[kb + 1] * sb[kb + 1];  // fetched while this block is awaited
+            for (int c = 0; c < Cfg::kTile / 2; ++c) acc[c] = make_float2(0.f, 0.f);
+#pragma unroll 1
+            for (int kb = 0; kb < p.kb; ++kb) {
                 const int a = ring % NA;
                 ok = wait_bar(&bar_acc_full[a], (ring / NA) & 1, STATUS_TIMEOUT_MMA);
                 if (!ok) break;
+                ++ring;
                 tc_fence_after();
-                const uint32_t t_acc = tmem + a * Cfg::kTileN + half * Cfg::kTile + lane_sel;
-                // 32 columns at a time, the next chunk's load in flight while this chunk is added up
+                const float sr = row_scale[a][wq * 32 + lane];
+                const float2 sc = col_scale[a];
+                const float f0 = sr * ((UP || half == 0) ? sc.x : sc.y), f1 = UP ? sr * sc.y : f0;
+                const uint32_t t_acc = tmem + a * Cfg::kTileN + lane_sel + half * (UP ? 64 : 128);
+                // 32 columns at a time, in an order that has the last of them out of TMEM, and the accumulator handed back,
+                // after half of the additions: the MMAs of the block after next wait for that
                 uint32_t v[2][32];
-                tmem_ld_x32(t_acc, v[0]);
+                auto load = [&](int c) { tmem_ld_x32(t_acc + ((UP && c >= 2) ? 64 : 0) + c * 32, v[c & 1]); };
+                auto add = [&](int c) {
+                    const float s = c < 2 ? f0 : f1;
 #pragma unroll
-                for (int c = 0; c < Cfg::kTile / 32; ++c) {
-                    tmem_wait_ld();
-                    if (c + 1 < Cfg::kTile / 32) {
-                        tmem_ld_x32(t_acc + (c + 1) * 32, v[(c + 1) & 1]);
-                    } else {  // the block's products are in registers: the accumulator is free
-                        tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(smem_u32(&bar_acc_empty[a]));
-                    }
-#pragma unroll
-                    for (int x = 0; x < 32; ++x) acc[c * 32 + x] = fmaf(__uint_as_float(v[c & 1][x]), s, acc[c * 32 + x]);
-                }
+                    for (int e = 0; e < 16; ++e)
+                        acc[c * 16 + e] = __ffma2_rn(make_float2(__uint_as_float(v[c & 1][2 * e]), __uint_as_float(v[c & 1][2 * e + 1])),
+                                                     make_float2(s, s), acc[c * 16 + e]);
+                    pin_sums(acc + c * 16);
+                };
+                load(0);
+                load(1);
+                tmem_wait_ld();
+                tmem_pin_x32(v[0]);
+                tmem_pin_x32(v[1]);
+                add(0);
+                load(2);
+                add(1);
+                load(3);
+                tmem_wait_ld();
+                tmem_pin_x32(v[0]);
+                tmem_pin_x32(v[1]);
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&bar_acc_empty[a]));
+                add(2);
+                add(3);
             }
             if (!ok) break;
-            if (!live) continue;
-            const float w = p.row_weight ? p.row_weight[row] : 1.f;
-            // 32 columns at a time through this warp's staging rows (128 bytes each, 128-byte swizzle) and out by TMA
+            if constexpr (UP) {
+                // a = silu(gate) * up; the group's maximum with the thread that has the row's other 64 columns; codes
+                float amax = 0.f;
 #pragma unroll
-            for (int c = 0; c < Cfg::kTile / 32; ++c) {
-                if (store_pending) {
-                    if (lane == 0) tma_store_wait_read();
-                    __syncwarp();
+                for (int c = 0; c < 32; ++c) {
+                    acc[c] = __fmul2_rn(silu2(acc[c]), acc[c + 32]);
+                    amax = fmaxf(amax, fmaxf(fabsf(acc[c].x), fabsf(acc[c].y)));
                 }
-#pragma unroll
-                for (int x = 0; x < 32; x += 4) {
-                    const uint32_t addr = sC + lane * 128 + ((uint32_t(x >> 2) ^ uint32_t(lane & 7)) << 4);
-                    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr),
-                                 "r"(__float_as_uint(acc[c * 32 + x] * w)), "r"(__float_as_uint(acc[c * 32 + x + 1] * w)),
-                                 "r"(__float_as_uint(acc[c * 32 + x + 2] * w)), "r"(__float_as_uint(acc[c * 32 + x + 3] * w))
-                                 : "memory");
-                }
-                fence_proxy_async_smem();
+                float *const buf = &row_max[n_done & 1][0][wq * 32 + lane];
+                buf[half * Cfg::kTile] = amax;
                 __syncwarp();
-                if (lane == 0) {
-                    tma_store_4d(&tm_c, sC, nb * Cfg::kTile + c * 32, bm * Cfg::kTile + wq * 32, 0, 0);
-                    tma_store_commit();
+                if (lane == 0) mbar_arrive(smem_u32(&bar_pair[wq]));
+                ok = wait_bar(&bar_pair[wq], n_done & 1, STATUS_TIMEOUT_SOFTMAX);
+                if (!ok) break;
+                amax = fmaxf(buf[0], buf[Cfg::kTile]);
+                ++n_done;
+                const float s = amax > 0.f ? __fdiv_rn(amax, 448.f) : 1.f;
+                if (half == 0) p.q_scale[(long long)bn * p.rows_cap + row] = s;
+                float sd = s;
+                if (s < 0x1p-60f) {  // a tiny group: scaled up exactly, so that 1 / s and the residuals stay normal
+                    sd = s * 0x1p64f;
+#pragma unroll
+                    for (int c = 0; c < 32; ++c) acc[c] = __fmul2_rn(acc[c], make_float2(0x1p64f, 0x1p64f));
                 }
-                store_pending = true;
+                const float r = __frcp_rn(sd);
+                uint4 *dst = reinterpret_cast<uint4 *>(p.q_out + (size_t(row) * (p.nblk / 2) + bn) * kMoeGroup + half * 64);
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    uint32_t w[4];
+#pragma unroll
+                    for (int x = 0; x < 4; ++x) {
+                        const float2 lo = div2_residual(acc[c * 8 + x * 2], make_float2(sd, sd), make_float2(r, r));
+                        const float2 hi = div2_residual(acc[c * 8 + x * 2 + 1], make_float2(sd, sd), make_float2(r, r));
+                        w[x] = cvt_e4m3x2(lo.x, lo.y) | (cvt_e4m3x2(hi.x, hi.y) << 16);
+                    }
+                    dst[c] = make_uint4(w[0], w[1], w[2], w[3]);
+                }
+            } else {
+                const float w = p.row_weight[row];
+                // 32 columns at a time through this warp's staging buffers (rows of 128 bytes, 128-byte swizzle) and out by
+                // TMA; a buffer is written again once the store before the last has read it
+#pragma unroll
+                for (int c = 0; c < Cfg::kTile / 32; ++c) {
+                    const uint32_t buf = sC + (c % Cfg::kStoreBufs) * (32 * 128);
+                    if (lane == 0) tma_store_wait_read_but<Cfg::kStoreBufs - 1>();
+                    __syncwarp();
+#pragma unroll
+                    for (int x = 0; x < 16; x += 2) {
+                        const uint32_t addr = buf + lane * 128 + ((uint32_t(x >> 1) ^ uint32_t(lane & 7)) << 4);
+                        const float2 lo = acc[c * 16 + x], hi = acc[c * 16 + x + 1];
+                        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(__float_as_uint(lo.x * w)),
+                                     "r"(__float_as_uint(lo.y * w)), "r"(__float_as_uint(hi.x * w)), "r"(__float_as_uint(hi.y * w))
+                                     : "memory");
+                    }
+                    fence_proxy_async_smem();
+                    __syncwarp();
+                    if (lane == 0) {
+                        tma_store_4d(&tm_c, buf, nb * Cfg::kTile + c * 32, bm * Cfg::kTile + wq * 32, 0, 0);
+                        tma_store_commit();
+                    }
+                }
             }
         }
-        if (lane == 0 && store_pending) tma_store_wait_all();
+        if (!UP && lane == 0) tma_store_wait_all();
     }
 
     // ---- common exit: every thread arrives, then TMEM is released
@@ -311,103 +474,114 @@ moe_gemm_fp8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
 }
 
 // ------------------------------------------------------------------ routing: sort (token, k) pairs by expert
-// One CTA: counts per expert, padded offsets (every expert starts on a multiple of 128 rows), the expert of every
-// 128-row tile (-1 beyond the last used tile), pair_of = -1 for every row (padding until the scatter fills it in).
-__global__ void moe_count_kernel(const int *__restrict__ ids, int n_pairs, int E, int rows_cap, int *expert_off,
-                                 int *cursor, int *tile_expert, int *pair_of, int *bad_id) {
-    extern __shared__ int counts[];  // E
+__global__ void moe_clear_kernel(int *counts, int E) {
     for (int e = threadIdx.x; e < E; e += blockDim.x) counts[e] = 0;
+}
+
+// Pairs per expert: a histogram per CTA in shared memory, added to the global one.
+__global__ void moe_count_kernel(const int *__restrict__ ids, int n_pairs, int E, int *counts) {
+    extern __shared__ int hist[];  // E
+    for (int e = threadIdx.x; e < E; e += blockDim.x) hist[e] = 0;
     __syncthreads();
-    for (int i = threadIdx.x; i < n_pairs; i += blockDim.x) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_pairs; i += gridDim.x * blockDim.x) {
         const int e = ids[i];
-        if (e >= 0 && e < E) atomicAdd(&counts[e], 1);
-        else *bad_id = 1;
+        if (e >= 0 && e < E) atomicAdd(&hist[e], 1);
     }
-    for (int r = threadIdx.x; r < rows_cap; r += blockDim.x) pair_of[r] = -1;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        int off = 0;
-        for (int e = 0; e < E; ++e) {
-            expert_off[e] = off;
-            cursor[e] = 0;
-            const int tiles = (counts[e] + 127) / 128;
-            for (int t = 0; t < tiles; ++t) tile_expert[off / 128 + t] = e;
-            off += tiles * 128;
-        }
-        expert_off[E] = off;
-        for (int t = off / 128; t < rows_cap / 128; ++t) tile_expert[t] = -1;
-    }
+    grid_dependency_wait();
+    grid_dependency_launch();
+    for (int e = threadIdx.x; e < E; e += blockDim.x)
+        if (hist[e]) atomicAdd(&counts[e], hist[e]);
 }
 
-__global__ void moe_scatter_kernel(const int *__restrict__ ids, int n_pairs, int E, const int *__restrict__ expert_off,
-                                   int *cursor, int *row_of, int *pair_of) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n_pairs) return;
-    const int e = ids[i];
-    if (e < 0 || e >= E) {
-        row_of[i] = -1;
-        return;
-    }
-    const int row = expert_off[e] + atomicAdd(&cursor[e], 1);
-    row_of[i] = row;
-    pair_of[row] = i;
-}
-
-// Codes and scales of every sorted row's token (zeros for padding rows), and the row's routing weight.
-// One CTA per row; C / 16 threads' worth of 16-byte copies.
-__global__ void moe_gather_kernel(const uint8_t *__restrict__ xq, const float *__restrict__ sx, const float *__restrict__ wts,
-                                  const int *__restrict__ pair_of, const int *__restrict__ tile_expert, int C, int K,
-                                  uint8_t *xq_s, float *sx_s, float *w_s) {
-    const int row = blockIdx.x;
-    if (tile_expert[row / 128] < 0) return;  // beyond the sorted rows: never read
-    const int pair = pair_of[row];
-    const int CG = C / kMoeGroup;
-    uint4 *dst = reinterpret_cast<uint4 *>(xq_s + size_t(row) * C);
-    if (pair < 0) {
-        for (int i = threadIdx.x; i < C / 16; i += blockDim.x) dst[i] = make_uint4(0, 0, 0, 0);
-        for (int i = threadIdx.x; i < CG; i += blockDim.x) sx_s[size_t(row) * CG + i] = 0.f;
-        if (threadIdx.x == 0) w_s[row] = 0.f;
-        return;
-    }
-    const int t = pair / K;
-    const uint4 *src = reinterpret_cast<const uint4 *>(xq + size_t(t) * C);
-    for (int i = threadIdx.x; i < C / 16; i += blockDim.x) dst[i] = src[i];
-    for (int i = threadIdx.x; i < CG; i += blockDim.x) sx_s[size_t(row) * CG + i] = sx[size_t(t) * CG + i];
-    if (threadIdx.x == 0) w_s[row] = wts[pair];
-}
-
-// Two fp32 values -> two E4M3 codes (round to nearest even, saturating at +-448); `lo` lands in bits 0..7.
-__device__ __forceinline__ uint32_t cvt_e4m3x2(float lo, float hi) {
-    uint16_t r;
-    asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(r) : "f"(hi), "f"(lo));
-    return r;
-}
-
-// a = silu(gate) * up in fp32, requantised per group of 128 columns: one warp per (row, group), four columns per
-// lane.  s = max|a| / 448 and a / s are fp32 divisions rounded to nearest, as the format's definition has them.
-__global__ void moe_act_quant_kernel(const float *__restrict__ h, const int *__restrict__ tile_expert, int F, int rows,
-                                     uint8_t *aq, float *sa) {
-    const int FG = F / kMoeGroup;
-    const long long wid = (long long)blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
-    if (wid >= (long long)rows * FG) return;
-    const int row = int(wid / FG), g = int(wid - (long long)row * FG);
-    if (tile_expert[row / 128] < 0) return;
-    const int lane = threadIdx.x & 31;
-    const float4 gate = reinterpret_cast<const float4 *>(h + size_t(row) * 2 * F + g * kMoeGroup)[lane];
-    const float4 up = reinterpret_cast<const float4 *>(h + size_t(row) * 2 * F + F + g * kMoeGroup)[lane];
-    float a[4];
-    a[0] = __fdiv_rn(gate.x, 1.f + expf(-gate.x)) * up.x;
-    a[1] = __fdiv_rn(gate.y, 1.f + expf(-gate.y)) * up.y;
-    a[2] = __fdiv_rn(gate.z, 1.f + expf(-gate.z)) * up.z;
-    a[3] = __fdiv_rn(gate.w, 1.f + expf(-gate.w)) * up.w;
-    float amax = fmaxf(fmaxf(fabsf(a[0]), fabsf(a[1])), fmaxf(fabsf(a[2]), fabsf(a[3])));
+// One CTA of 1024 threads: every expert's first row (a multiple of 128; its cursor starts there) and the list of row tiles.
+__global__ void __launch_bounds__(1024) moe_plan_kernel(const int *counts, int E, int *cursor, MoeRowTile *tiles, int *n_row_tiles) {
+    __shared__ int first[1025], rows[1024], warp_sum[32];  // first row tile and rows of every expert
+    const int e = threadIdx.x, lane = e & 31, warp = e >> 5;
+    grid_dependency_wait();
+    grid_dependency_launch();
+    const int n = e < E ? counts[e] : 0;
+    int x = (n + 127) / 128;
+    const int mine = x;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-    const float s = amax > 0.f ? __fdiv_rn(amax, 448.f) : 1.f;
-    const uint32_t c01 = cvt_e4m3x2(__fdiv_rn(a[0], s), __fdiv_rn(a[1], s));
-    const uint32_t c23 = cvt_e4m3x2(__fdiv_rn(a[2], s), __fdiv_rn(a[3], s));
-    reinterpret_cast<uint32_t *>(aq + size_t(row) * F + g * kMoeGroup)[lane] = c01 | (c23 << 16);
-    if (lane == 0) sa[size_t(row) * FG + g] = s;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) warp_sum[warp] = x;
+    __syncthreads();
+    if (warp == 0) {
+        int w = warp_sum[lane];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, w, o);
+            if (lane >= o) w += y;
+        }
+        warp_sum[lane] = w;
+    }
+    __syncthreads();
+    const int before = x - mine + (warp > 0 ? warp_sum[warp - 1] : 0);
+    first[e] = before;
+    rows[e] = n;
+    if (e < E) cursor[e] = before * 128;
+    if (e == 1023) first[1024] = before + mine;
+    __syncthreads();
+    const int total = first[1024];
+    if (e == 0) *n_row_tiles = total;
+    for (int t = e; t < total; t += 1024) {
+        int lo = 0, hi = E;  // the expert with first[lo] <= t < first[lo + 1]
+        while (hi - lo > 1) {
+            const int m = (lo + hi) / 2;
+            if (first[m] <= t) lo = m;
+            else hi = m;
+        }
+        const int k = t - first[lo], n_tiles = (rows[lo] + 127) / 128;
+        MoeRowTile r;
+        r.expert = lo;
+        r.group_first = first[lo] + k / kMoeGroupTiles * kMoeGroupTiles;
+        r.group_tiles = min(kMoeGroupTiles, first[lo] + n_tiles - r.group_first);
+        r.rows = min(128, rows[lo] - k * 128);
+        tiles[t] = r;
+    }
+}
+
+// One CTA per token: every one of its K pairs takes the next row of its expert, and the token's codes, scales (into
+// [channel group, row] order) and the pair's routing weight are copied there.  Rows that no pair takes stay as they are.
+// (The order of an expert's rows depends on timing; no result does.)
+constexpr int kMoeGatherThreads = 128;
+__global__ void __launch_bounds__(kMoeGatherThreads)
+moe_gather_kernel(const uint8_t *__restrict__ xq, const float *__restrict__ sx, const int *__restrict__ ids,
+                  const float *__restrict__ wts, int C, int E, int K, long long rows_cap, int *cursor, int *row_of, uint8_t *xq_s,
+                  float *sx_s, float *w_s) {
+    __shared__ int row[kMoeGatherThreads];
+    const long long t = blockIdx.x;
+    const int CG = C / kMoeGroup;
+    grid_dependency_wait();
+    grid_dependency_launch();
+    const uint4 *src = reinterpret_cast<const uint4 *>(xq + t * C);
+    for (int k0 = 0; k0 < K; k0 += kMoeGatherThreads) {
+        const int k = k0 + threadIdx.x;
+        __syncthreads();
+        if (k < K) {
+            const int e = ids[t * K + k];
+            const int r = (e >= 0 && e < E) ? atomicAdd(&cursor[e], 1) : -1;
+            row[threadIdx.x] = r;
+            row_of[t * K + k] = r;
+            if (r >= 0) w_s[r] = wts[t * K + k];
+        }
+        __syncthreads();
+        const int n = min(K - k0, kMoeGatherThreads);
+        for (int i = threadIdx.x; i < C / 16; i += kMoeGatherThreads) {
+            const uint4 v = src[i];
+            for (int x = 0; x < n; ++x)
+                if (row[x] >= 0) reinterpret_cast<uint4 *>(xq_s + (long long)row[x] * C)[i] = v;
+        }
+        for (int i = threadIdx.x; i < CG; i += kMoeGatherThreads) {
+            const float v = sx[t * CG + i];
+            for (int x = 0; x < n; ++x)
+                if (row[x] >= 0) sx_s[i * rows_cap + row[x]] = v;
+        }
+    }
 }
 
 // y[t, :] = sum over the token's K sorted rows of o (already weighted), in the order k = 0..K-1, rounded to bf16.
@@ -415,7 +589,8 @@ __global__ void moe_combine_kernel(const float *__restrict__ o, const int *__res
                                    __nv_bfloat16 *y) {
     const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const int per_row = C / 4;
-    if (idx >= (long long)T * per_row) return;
+    grid_dependency_wait();
+    if (idx >= (long long)T * per_row || *reinterpret_cast<volatile unsigned int *>(&g_device_status) != 0) return;
     const int t = int(idx / per_row), c4 = int(idx - (long long)t * per_row);
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
     for (int k = 0; k < K; ++k) {

@@ -159,6 +159,28 @@ def _stream_ptr(stream):
     return ctypes.c_void_p(stream.cuda_stream)
 
 
+# A small call is bound by the host, so the wrappers below go the short way: device and stream as integers from torch's
+# C functions (a `torch.cuda.device` block and a Stream object take some 4 us), addresses as plain integers (the
+# functions' argtypes convert them).  Measured on a 128-token attention call: 18.4 us before.
+_current_device = getattr(torch._C, "_cuda_getDevice", torch.cuda.current_device)
+_Strides = ctypes.c_longlong * 3
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or (
+    lambda device: torch.cuda.current_stream(device).cuda_stream)
+
+
+def _call(name, tensor, stream, *args):
+    """Run the library function on the tensor's device and stream (the device's current one if None); raise on error."""
+    fn = getattr(lib(), name)
+    device = tensor.get_device()
+    if device == _current_device():
+        st = fn(*args, _raw_stream(device) if stream is None else stream.cuda_stream)
+    else:
+        with torch.cuda.device(device):
+            st = fn(*args, _raw_stream(device) if stream is None else stream.cuda_stream)
+    if st != AVE_OK:
+        raise AveAttnError(st, name)
+
+
 def ave_attn_fwd_raw(q_ptr, k_ptr, v_ptr, o_ptr, lse_ptr, B, H, Hkv, Sq, Sk, D, causal, scale, stream_ptr=None) -> int:
     """The C call with plain integers for pointers; returns the status code."""
     return int(lib().ave_attn_fwd(
@@ -175,25 +197,21 @@ def ave_attn_fwd(q, k, v, o=None, lse=None, causal=False, scale=None, stream=Non
     non-zero status.
     """
     for t in (q, k, v):
-        if not (t.is_cuda and t.dtype == torch.bfloat16 and t.is_contiguous() and t.dim() == 4):
+        if not (t.is_cuda and t.dtype is torch.bfloat16 and t.dim() == 4 and t.is_contiguous()):
             raise ValueError("q, k, v must be contiguous 4-D CUDA bfloat16 tensors")
     B, H, Sq, D = q.shape
-    Bk, Hkv, Sk, Dk = k.shape
-    if tuple(v.shape) != tuple(k.shape) or Bk != B or Dk != D:
+    kshape = k.shape
+    Bk, Hkv, Sk, Dk = kshape
+    if v.shape != kshape or Bk != B or Dk != D:
         raise ValueError("inconsistent q/k/v shapes")
     if o is None:
         o = torch.empty_like(q)
     if lse is None:
-        lse = torch.empty((B, H, Sq), dtype=torch.float32, device=q.device)
+        lse = q.new_empty((B, H, Sq), dtype=torch.float32)
     if scale is None:
         scale = D ** -0.5
-    with torch.cuda.device(q.device):
-        st = lib().ave_attn_fwd(
-            ctypes.c_void_p(q.data_ptr()), ctypes.c_void_p(k.data_ptr()), ctypes.c_void_p(v.data_ptr()),
-            ctypes.c_void_p(o.data_ptr()), ctypes.c_void_p(lse.data_ptr()),
-            B, H, Hkv, Sq, Sk, D, int(bool(causal)), float(scale), _stream_ptr(stream))
-    if st != AVE_OK:
-        raise AveAttnError(st, "ave_attn_fwd")
+    _call("ave_attn_fwd", q, stream, q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), lse.data_ptr(),
+          B, H, Hkv, Sq, Sk, D, 1 if causal else 0, scale)
     return o, lse
 
 
@@ -202,26 +220,20 @@ def ave_attn_fwd_strided(q, k, v, o, lse=None, causal=False, scale=None, stream=
     batch/head/row strides (last dimension contiguous), e.g. permuted views of (B,S,H,D) storage or slices
     of a packed QKV buffer; ``o`` is written in place through its strides.  ``lse`` is contiguous fp32."""
     for t in (q, k, v, o):
-        if not (t.is_cuda and t.dtype == torch.bfloat16 and t.dim() == 4 and t.stride(3) == 1):
+        if not (t.is_cuda and t.dtype is torch.bfloat16 and t.dim() == 4 and t.stride(3) == 1):
             raise ValueError("q, k, v, o must be 4-D CUDA bfloat16 tensors whose last dimension is contiguous")
     B, H, Sq, D = q.shape
-    Bk, Hkv, Sk, Dk = k.shape
-    if tuple(v.shape) != tuple(k.shape) or Bk != B or Dk != D or tuple(o.shape) != tuple(q.shape):
+    kshape = k.shape
+    Bk, Hkv, Sk, Dk = kshape
+    if v.shape != kshape or Bk != B or Dk != D or o.shape != q.shape:
         raise ValueError("inconsistent q/k/v/o shapes")
     if lse is None:
-        lse = torch.empty((B, H, Sq), dtype=torch.float32, device=q.device)
+        lse = q.new_empty((B, H, Sq), dtype=torch.float32)
     if scale is None:
         scale = D ** -0.5
-    arrs = [(ctypes.c_longlong * 3)(t.stride(0), t.stride(1), t.stride(2)) for t in (q, k, v, o)]
-    with torch.cuda.device(q.device):
-        st = lib().ave_attn_fwd_strided(
-            ctypes.c_void_p(q.data_ptr()), ctypes.c_void_p(k.data_ptr()), ctypes.c_void_p(v.data_ptr()),
-            ctypes.c_void_p(o.data_ptr()), ctypes.c_void_p(lse.data_ptr()),
-            B, H, Hkv, Sq, Sk, D, ctypes.cast(arrs[0], ctypes.c_void_p), ctypes.cast(arrs[1], ctypes.c_void_p),
-            ctypes.cast(arrs[2], ctypes.c_void_p), ctypes.cast(arrs[3], ctypes.c_void_p),
-            int(bool(causal)), float(scale), _stream_ptr(stream))
-    if st != AVE_OK:
-        raise AveAttnError(st, "ave_attn_fwd_strided")
+    arrs = [_Strides(*t.stride()[:3]) for t in (q, k, v, o)]
+    _call("ave_attn_fwd_strided", q, stream, q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), lse.data_ptr(),
+          B, H, Hkv, Sq, Sk, D, arrs[0], arrs[1], arrs[2], arrs[3], 1 if causal else 0, scale)
     return o, lse
 
 
@@ -230,31 +242,26 @@ def ave_attn_fwd_varlen(q, k, v, cu_seqlens_q, cu_seqlens_k, max_sq, max_sk, o=N
     """Variable-length batch: q [total_q,H,D], k/v [total_k,Hkv,D] contiguous CUDA bf16, cu_seqlens_* CUDA int32
     [B+1].  Returns o [total_q,H,D] bf16 and lse [H,total_q] fp32."""
     for t in (q, k, v):
-        if not (t.is_cuda and t.dtype == torch.bfloat16 and t.is_contiguous() and t.dim() == 3):
+        if not (t.is_cuda and t.dtype is torch.bfloat16 and t.dim() == 3 and t.is_contiguous()):
             raise ValueError("q, k, v must be contiguous 3-D CUDA bfloat16 tensors")
     for t in (cu_seqlens_q, cu_seqlens_k):
-        if not (t.is_cuda and t.dtype == torch.int32 and t.is_contiguous() and t.dim() == 1):
+        if not (t.is_cuda and t.dtype is torch.int32 and t.dim() == 1 and t.is_contiguous()):
             raise ValueError("cu_seqlens must be contiguous 1-D CUDA int32 tensors")
     total_q, H, D = q.shape
-    total_k, Hkv, Dk = k.shape
+    kshape = k.shape
+    total_k, Hkv, Dk = kshape
     B = cu_seqlens_q.numel() - 1
-    if tuple(v.shape) != tuple(k.shape) or Dk != D or cu_seqlens_k.numel() != B + 1:
+    if v.shape != kshape or Dk != D or cu_seqlens_k.numel() != B + 1:
         raise ValueError("inconsistent shapes")
     if o is None:
         o = torch.empty_like(q)
     if lse is None:
-        lse = torch.empty((H, total_q), dtype=torch.float32, device=q.device)
+        lse = q.new_empty((H, total_q), dtype=torch.float32)
     if scale is None:
         scale = D ** -0.5
-    with torch.cuda.device(q.device):
-        st = lib().ave_attn_fwd_varlen(
-            ctypes.c_void_p(q.data_ptr()), ctypes.c_void_p(k.data_ptr()), ctypes.c_void_p(v.data_ptr()),
-            ctypes.c_void_p(o.data_ptr()), ctypes.c_void_p(lse.data_ptr()),
-            ctypes.c_void_p(cu_seqlens_q.data_ptr()), ctypes.c_void_p(cu_seqlens_k.data_ptr()),
-            B, H, Hkv, int(max_sq), int(max_sk), total_q, total_k, D, int(bool(causal)), float(scale),
-            _stream_ptr(stream))
-    if st != AVE_OK:
-        raise AveAttnError(st, "ave_attn_fwd_varlen")
+    _call("ave_attn_fwd_varlen", q, stream, q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), lse.data_ptr(),
+          cu_seqlens_q.data_ptr(), cu_seqlens_k.data_ptr(), B, H, Hkv, int(max_sq), int(max_sk), total_q, total_k, D,
+          1 if causal else 0, scale)
     return o, lse
 
 
@@ -300,20 +307,14 @@ def ave_attn_fwd_splitkv(q, k, v, n_splits, workspace=None, o=None, lse=None, ca
     if o is None:
         o = torch.empty_like(q)
     if lse is None:
-        lse = torch.empty((B, H, Sq), dtype=torch.float32, device=q.device)
+        lse = q.new_empty((B, H, Sq), dtype=torch.float32)
     if scale is None:
         scale = D ** -0.5
     if workspace is None:
         workspace = torch.empty(max(256, splitkv_workspace_bytes(B, H, Sq, D, n_splits)), dtype=torch.uint8,
                                 device=q.device)
-    with torch.cuda.device(q.device):
-        st = lib().ave_attn_fwd_splitkv(
-            ctypes.c_void_p(q.data_ptr()), ctypes.c_void_p(k.data_ptr()), ctypes.c_void_p(v.data_ptr()),
-            ctypes.c_void_p(o.data_ptr()), ctypes.c_void_p(lse.data_ptr()),
-            B, H, Hkv, Sq, Sk, D, int(bool(causal)), float(scale), int(n_splits),
-            ctypes.c_void_p(workspace.data_ptr()), ctypes.c_size_t(workspace.numel()), _stream_ptr(stream))
-    if st != AVE_OK:
-        raise AveAttnError(st, "ave_attn_fwd_splitkv")
+    _call("ave_attn_fwd_splitkv", q, stream, q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), lse.data_ptr(),
+          B, H, Hkv, Sq, Sk, D, 1 if causal else 0, scale, int(n_splits), workspace.data_ptr(), workspace.numel())
     return o, lse
 
 
@@ -328,13 +329,8 @@ def ave_attn_fwd_splitkv_static(q, k, v, n_splits, o, lse, causal=False, scale=N
     _, Hkv, Sk, _ = k.shape
     if scale is None:
         scale = D ** -0.5
-    with torch.cuda.device(q.device):
-        st = lib().ave_attn_fwd_splitkv_static(
-            ctypes.c_void_p(q.data_ptr()), ctypes.c_void_p(k.data_ptr()), ctypes.c_void_p(v.data_ptr()),
-            ctypes.c_void_p(o.data_ptr()), ctypes.c_void_p(lse.data_ptr()),
-            B, H, Hkv, Sq, Sk, D, int(bool(causal)), float(scale), int(n_splits), _stream_ptr(stream))
-    if st != AVE_OK:
-        raise AveAttnError(st, "ave_attn_fwd_splitkv_static")
+    _call("ave_attn_fwd_splitkv_static", q, stream, q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), lse.data_ptr(),
+          B, H, Hkv, Sq, Sk, D, 1 if causal else 0, scale, int(n_splits))
     return o, lse
 
 
@@ -347,19 +343,15 @@ def ave_gemm_bf16_tn_raw(a_ptr, b_ptr, c_ptr, M, N, K, stream_ptr=None) -> int:
 def ave_gemm_bf16_tn(a, b, c=None, stream=None):
     """C [M, N] = a [M, K] . b [N, K]^T on the tensors' CUDA device (contiguous bf16)."""
     for t in (a, b):
-        if not (t.is_cuda and t.dtype == torch.bfloat16 and t.is_contiguous() and t.dim() == 2):
+        if not (t.is_cuda and t.dtype is torch.bfloat16 and t.dim() == 2 and t.is_contiguous()):
             raise ValueError("a and b must be contiguous 2-D CUDA bfloat16 tensors")
     M, K = a.shape
     N, Kb = b.shape
     if Kb != K:
         raise ValueError("a is [M, K] and b is [N, K]: the K sizes differ")
     if c is None:
-        c = torch.empty((M, N), dtype=torch.bfloat16, device=a.device)
-    with torch.cuda.device(a.device):
-        st = lib().ave_gemm_bf16_tn(ctypes.c_void_p(a.data_ptr()), ctypes.c_void_p(b.data_ptr()),
-                                    ctypes.c_void_p(c.data_ptr()), M, N, K, _stream_ptr(stream))
-    if st != AVE_OK:
-        raise AveAttnError(st, "ave_gemm_bf16_tn")
+        c = a.new_empty((M, N))
+    _call("ave_gemm_bf16_tn", a, stream, a.data_ptr(), b.data_ptr(), c.data_ptr(), M, N, K)
     return c
 
 
@@ -372,19 +364,15 @@ def ave_gemm_bf16_nn_raw(a_ptr, b_ptr, c_ptr, M, N, K, stream_ptr=None) -> int:
 def ave_gemm_bf16_nn(a, b, c=None, stream=None):
     """C [M, N] = a [M, K] . b [K, N] on the tensors' CUDA device (contiguous bf16)."""
     for t in (a, b):
-        if not (t.is_cuda and t.dtype == torch.bfloat16 and t.is_contiguous() and t.dim() == 2):
+        if not (t.is_cuda and t.dtype is torch.bfloat16 and t.dim() == 2 and t.is_contiguous()):
             raise ValueError("a and b must be contiguous 2-D CUDA bfloat16 tensors")
     M, K = a.shape
     Kb, N = b.shape
     if Kb != K:
         raise ValueError("a is [M, K] and b is [K, N]: the K sizes differ")
     if c is None:
-        c = torch.empty((M, N), dtype=torch.bfloat16, device=a.device)
-    with torch.cuda.device(a.device):
-        st = lib().ave_gemm_bf16_nn(ctypes.c_void_p(a.data_ptr()), ctypes.c_void_p(b.data_ptr()),
-                                    ctypes.c_void_p(c.data_ptr()), M, N, K, _stream_ptr(stream))
-    if st != AVE_OK:
-        raise AveAttnError(st, "ave_gemm_bf16_nn")
+        c = a.new_empty((M, N))
+    _call("ave_gemm_bf16_nn", a, stream, a.data_ptr(), b.data_ptr(), c.data_ptr(), M, N, K)
     return c
 
 
@@ -412,12 +400,6 @@ def ave_moe_fused_fwd(xq, sx, w13q, s13, w2q, s2, ids, wts, y=None, workspace=No
         y = torch.empty((T, C), dtype=torch.bfloat16, device=xq.device)
     if workspace is None:
         workspace = torch.empty(max(256, moe_workspace_bytes(T, C, F, E, K)), dtype=torch.uint8, device=xq.device)
-    with torch.cuda.device(xq.device):
-        st = lib().ave_moe_fused_fwd(
-            ctypes.c_void_p(xq.data_ptr()), ctypes.c_void_p(sx.data_ptr()), ctypes.c_void_p(w13q.data_ptr()),
-            ctypes.c_void_p(s13.data_ptr()), ctypes.c_void_p(w2q.data_ptr()), ctypes.c_void_p(s2.data_ptr()),
-            ctypes.c_void_p(ids.data_ptr()), ctypes.c_void_p(wts.data_ptr()), ctypes.c_void_p(y.data_ptr()),
-            T, C, F, E, K, ctypes.c_void_p(workspace.data_ptr()), ctypes.c_size_t(workspace.numel()), _stream_ptr(stream))
-    if st != AVE_OK:
-        raise AveAttnError(st, "ave_moe_fused_fwd")
+    _call("ave_moe_fused_fwd", xq, stream, xq.data_ptr(), sx.data_ptr(), w13q.data_ptr(), s13.data_ptr(), w2q.data_ptr(),
+          s2.data_ptr(), ids.data_ptr(), wts.data_ptr(), y.data_ptr(), T, C, F, E, K, workspace.data_ptr(), workspace.numel())
     return y

@@ -435,7 +435,7 @@ gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_con
                 if (c == Cfg::kTileN / 64 - 1) {  // the accumulator is in registers: the MMAs may reuse it
                     tc_fence_before();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive_cluster(map_to_cta(smem_u32(&bar_acc_empty[acc]), 0));
+                    if (lane == 0) mbar_arrive_cluster_relaxed(map_to_cta(smem_u32(&bar_acc_empty[acc]), 0));
                 }
                 // this warp's previous TMA store must have finished reading the staging rows
                 if (lane == 0 && store_pending) tma_store_wait_read();

@@ -207,8 +207,10 @@ __device__ __forceinline__ int ld_cluster_s32(uint32_t cluster_addr) {
 __device__ __forceinline__ void cluster_sync() {
     asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_bar) {
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
+// Arrive on a barrier of either CTA, without ordering this thread's memory accesses before it (a release at cluster scope
+// takes some 1100 clk): for hand-overs of TMEM whose loads a tcgen05.wait has completed.
+__device__ __forceinline__ void mbar_arrive_cluster_relaxed(uint32_t cluster_bar) {
+    asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
 }
 // Loads into this CTA's shared memory; the bytes are counted on a barrier that may be the other CTA's.
 __device__ __forceinline__ void tma_load_4d_pair(uint32_t dst, const void *tmap, uint32_t cluster_bar, int x, int y, int z, int w) {

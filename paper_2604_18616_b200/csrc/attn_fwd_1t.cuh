@@ -84,7 +84,6 @@ attn_fwd_1t_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     const uint32_t sRing = sQ + Cfg::kTileBytes;
 
     if (tid == 0) {
-        abort_flag = (*reinterpret_cast<volatile unsigned int *>(&g_device_status) != 0) ? 1 : 0;
         mbar_init(smem_u32(&bar_q_full), 1);
         mbar_init(smem_u32(&bar_q_empty), 1);
         mbar_init(smem_u32(&bar_s), 1);
@@ -107,6 +106,10 @@ attn_fwd_1t_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
         tmem_alloc(smem_u32(&tmem_base_slot), Cfg::kTmemCols);
         tmem_relinquish();
     }
+    // what precedes overlaps the end of the kernel before this one in the stream
+    grid_dependency_wait();
+    grid_dependency_launch();
+    if (tid == 0) abort_flag = (*reinterpret_cast<volatile unsigned int *>(&g_device_status) != 0) ? 1 : 0;
     tc_fence_before();
     __syncthreads();
     tc_fence_after();

@@ -289,8 +289,7 @@ int launch_1t(const CUtensorMap &tq, const CUtensorMap &tk, const CUtensorMap &t
         t_last_cuda_error = int(cudaErrorLaunchFailure);
         return AVE_ERR_CUDA;
     }
-    kern<<<dim3(p.total_blocks), dim3(Cfg::kThreads), Cfg::kSmemBytes, stream>>>(tq, tk, tv, p);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_dependent(kern, dim3(p.total_blocks), dim3(Cfg::kThreads), Cfg::kSmemBytes, stream, tq, tk, tv, p);
     if (e != cudaSuccess) {
         t_last_cuda_error = int(e);
         return AVE_ERR_CUDA;
@@ -538,11 +537,9 @@ int launch_gemm_tile(const void *a, const void *b, void *c, int M, int N, int K,
     static PerDeviceOnce once;  // per instantiation
     const int st = prepare_kernel(kern, Cfg::kSmemBytes, 0, once);
     if (st != AVE_OK) return st;
-    cudaError_t e;
     const long long n_tiles = (long long)p.tiles_m * p.tiles_n;
     const unsigned grid = unsigned(n_tiles < sms ? n_tiles : sms);
-    kern<<<dim3(grid), dim3(Cfg::kThreads), Cfg::kSmemBytes, s>>>(ta, tb, tc, p);
-    e = cudaGetLastError();
+    cudaError_t e = launch_dependent(kern, dim3(grid), dim3(Cfg::kThreads), Cfg::kSmemBytes, s, ta, tb, tc, p);
     if (e != cudaSuccess) {
         t_last_cuda_error = int(e);
         return AVE_ERR_CUDA;
@@ -579,8 +576,7 @@ int launch_gemm_pair(const void *a, const void *b, void *c, int M, int N, int K,
     if (st != AVE_OK) return st;
     const long long n_tiles = (long long)p.tiles_m * p.tiles_n;
     const long long pairs = n_tiles < sms / 2 ? n_tiles : sms / 2;
-    kern<<<dim3(unsigned(2 * pairs)), dim3(Cfg::kThreads), Cfg::kSmemBytes, s>>>(ta, tb, tc, p);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_dependent(kern, dim3(unsigned(2 * pairs)), dim3(Cfg::kThreads), Cfg::kSmemBytes, s, ta, tb, tc, p);
     if (e != cudaSuccess) {
         t_last_cuda_error = int(e);
         return AVE_ERR_CUDA;

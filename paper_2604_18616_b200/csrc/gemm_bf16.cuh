@@ -76,7 +76,6 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
     const uint32_t sStage = sRing + NS * Cfg::kStageBytes;
 
     if (tid == 0) {
-        abort_flag = (*reinterpret_cast<volatile unsigned int *>(&g_device_status) != 0) ? 1 : 0;
         for (int s = 0; s < NS; ++s) {
             mbar_init(smem_u32(&bar_full[s]), 1);
             mbar_init(smem_u32(&bar_empty[s]), 1);
@@ -92,6 +91,10 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
         tmem_alloc(smem_u32(&tmem_base_slot), Cfg::kTmemCols);
         tmem_relinquish();
     }
+    // what precedes overlaps the end of the kernel before this one in the stream
+    grid_dependency_wait();
+    grid_dependency_launch();
+    if (tid == 0) abort_flag = (*reinterpret_cast<volatile unsigned int *>(&g_device_status) != 0) ? 1 : 0;
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -298,7 +301,6 @@ gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_con
 
     if (tid == 0) {
         abort_flag = 0;
-        poison_flag = (*reinterpret_cast<volatile unsigned int *>(&g_device_status) != 0) ? 1 : 0;
         for (int s = 0; s < NS; ++s) {
             mbar_init(smem_u32(&bar_full[s]), 1);
             mbar_init(smem_u32(&bar_empty[s]), 1);
@@ -316,6 +318,9 @@ gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_con
         tmem_alloc_pair(smem_u32(&tmem_base_slot), Cfg::kTmemCols);
         tmem_relinquish_pair();
     }
+    grid_dependency_wait();
+    grid_dependency_launch();
+    if (tid == 0) poison_flag = (*reinterpret_cast<volatile unsigned int *>(&g_device_status) != 0) ? 1 : 0;
     tc_fence_before();
     __syncthreads();
     cluster_sync();

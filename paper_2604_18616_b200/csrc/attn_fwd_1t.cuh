@@ -396,6 +396,19 @@ attn_fwd_1t_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                 }
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&bar_o_free));  // O was not used: hand it back at once
+            } else if (D <= 128 && i0 + wq * 32 >= sq) {
+                // None of this warp's rows exists (a decode step has a handful of rows in the tile's 128): it only passes the
+                // hand-overs on.  Whatever P and O hold in its lanes stays in its rows and is not stored.  The work this
+                // saves is energy: decode runs at the power limit, where the clocks follow it (64 sequences of 4001 keys 198 ->
+                // 190 us, 11 of 21249 with D = 64 60 -> 53 us).
+                for (int j = 0; j < n_t && ok; ++j) {
+                    ok = wait_bar(&bar_s, ns & 1, STATUS_TIMEOUT_MMA);
+                    ++ns;
+                    if (ok && lane == 0) mbar_arrive(smem_u32(&bar_p));
+                }
+                if (ok) ok = wait_bar(&bar_o, n_out & 1, STATUS_TIMEOUT_MMA);
+                ++n_out;
+                if (ok && lane == 0) mbar_arrive(smem_u32(&bar_o_free));
             } else {
                 float m_run = -INFINITY, l_run = 0.f;
                 const int k_end = key_end(w, p);

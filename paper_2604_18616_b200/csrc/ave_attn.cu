@@ -238,20 +238,29 @@ int prepare_kernel(Kernel kern, int smem_bytes, int check_register_split, PerDev
 }
 
 // Launch a kernel that begins with grid_dependency_wait(): its blocks may be set up while the kernel before it in the
-// stream still runs (programmatic dependent launch), which takes the launch latency out of a chain of kernels.
+// stream still runs (programmatic dependent launch), which takes the launch latency out of a chain of kernels.  `cluster`:
+// CTAs of a cluster.
 template <class... Params, class... Args>
-cudaError_t launch_dependent(void (*kern)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args... args) {
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
+cudaError_t launch_dependent_clusters(void (*kern)(Params...), dim3 grid, dim3 block, int cluster, size_t smem, cudaStream_t s,
+                                      Args... args) {
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kern, Params(args)...);
+}
+template <class... Params, class... Args>
+cudaError_t launch_dependent(void (*kern)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args... args) {
+    return launch_dependent_clusters(kern, grid, block, 1, smem, s, args...);
 }
 
 template <int D, bool CAUSAL, bool SPLIT, bool VARLEN = false>
@@ -511,9 +520,9 @@ int run_splitkv(const void *q, const void *k, const void *v, void *o, float *lse
 }
 
 
-// C[M, N] = A[M, K] * B[N, K]^T: tensor maps of the three matrices, tile order, persistent launch.
+// C[M, N] = A[M, K] * B[N, K]^T (or * B[K, N]) in 128 x 128 tiles, one cluster of `splits` CTAs each.
 template <bool B_NMAJOR>
-int launch_gemm_tile(const void *a, const void *b, void *c, int M, int N, int K, int sms, cudaStream_t s) {
+int launch_gemm_tile(const void *a, const void *b, void *c, int M, int N, int K, int splits, cudaStream_t s) {
     using Cfg = ave::GemmCfg;
     CUtensorMap ta, tb, tc;
     const Strides sa{(long long)M * K, (long long)M * K, (long long)K};
@@ -526,20 +535,21 @@ int launch_gemm_tile(const void *a, const void *b, void *c, int M, int N, int K,
         if (!encode_map(&tb, b, K, N, 1, 1, sb, Cfg::kTileN)) return AVE_ERR_CUDA;
     }
     if (!encode_map(&tc, c, N, M, 1, 1, sc, Cfg::kOutBoxRows)) return AVE_ERR_CUDA;
-    ave::GemmParams p;
+    ave::GemmParams p{};
     p.M = M;
     p.N = N;
     p.K = K;
     p.tiles_m = (M + Cfg::kTileM - 1) / Cfg::kTileM;
     p.tiles_n = (N + Cfg::kTileN - 1) / Cfg::kTileN;
     p.group_m = 16;
+    p.splits = splits;
+    p.c = c;
     auto kern = ave::gemm_bf16_kernel<B_NMAJOR>;
     static PerDeviceOnce once;  // per instantiation
     const int st = prepare_kernel(kern, Cfg::kSmemBytes, 0, once);
     if (st != AVE_OK) return st;
-    const long long n_tiles = (long long)p.tiles_m * p.tiles_n;
-    const unsigned grid = unsigned(n_tiles < sms ? n_tiles : sms);
-    cudaError_t e = launch_dependent(kern, dim3(grid), dim3(Cfg::kThreads), Cfg::kSmemBytes, s, ta, tb, tc, p);
+    cudaError_t e = launch_dependent_clusters(kern, dim3(unsigned(p.tiles_m) * p.tiles_n * splits), dim3(Cfg::kThreads), splits,
+                                              Cfg::kSmemBytes, s, ta, tb, tc, p);
     if (e != cudaSuccess) {
         t_last_cuda_error = int(e);
         return AVE_ERR_CUDA;
@@ -548,9 +558,9 @@ int launch_gemm_tile(const void *a, const void *b, void *c, int M, int N, int K,
     return AVE_OK;
 }
 
-// The same on CTA pairs with 256 x 256 tiles.
+// The same on CTA pairs, with tiles of 256 x tile_n.
 template <bool B_NMAJOR>
-int launch_gemm_pair(const void *a, const void *b, void *c, int M, int N, int K, int sms, cudaStream_t s) {
+int launch_gemm_pair(const void *a, const void *b, void *c, int M, int N, int K, int tile_n, int sms, cudaStream_t s) {
     using Cfg = ave::GemmPairCfg;
     CUtensorMap ta, tb, tc;
     const Strides sa{(long long)M * K, (long long)M * K, (long long)K};
@@ -559,16 +569,17 @@ int launch_gemm_pair(const void *a, const void *b, void *c, int M, int N, int K,
     if (!encode_map(&ta, a, K, M, 1, 1, sa, 128)) return AVE_ERR_CUDA;
     if (B_NMAJOR) {  // B [K, N]: rows of N elements, boxes of 64 columns x 64 rows of K
         if (!encode_map(&tb, b, N, K, 1, 1, sb, Cfg::kSliceK)) return AVE_ERR_CUDA;
-    } else {         // B [N, K]: rows of K elements, boxes of 64 columns of K x 128 rows
-        if (!encode_map(&tb, b, K, N, 1, 1, sb, 128)) return AVE_ERR_CUDA;
+    } else {         // B [N, K]: rows of K elements, boxes of 64 columns of K x half of the tile's columns
+        if (!encode_map(&tb, b, K, N, 1, 1, sb, tile_n / 2)) return AVE_ERR_CUDA;
     }
     if (!encode_map(&tc, c, N, M, 1, 1, sc, Cfg::kOutBoxRows)) return AVE_ERR_CUDA;
-    ave::GemmParams p;
+    ave::GemmParams p{};
     p.M = M;
     p.N = N;
     p.K = K;
     p.tiles_m = (M + Cfg::kTileM - 1) / Cfg::kTileM;
-    p.tiles_n = (N + Cfg::kTileN - 1) / Cfg::kTileN;
+    p.tile_n = tile_n;
+    p.tiles_n = (N + tile_n - 1) / tile_n;
     p.group_m = 8;  // the ~74 tiles in flight cover 8 x 9.25 tiles, a near-square part of C
     auto kern = ave::gemm_bf16_pair_kernel<B_NMAJOR>;
     static PerDeviceOnce once;  // per instantiation
@@ -594,12 +605,35 @@ int launch_gemm(const void *a, const void *b, void *c, int M, int N, int K, cuda
         t_last_cuda_error = int(e);
         return AVE_ERR_CUDA;
     }
-    // CTA pairs with 256 x 256 tiles move the fewest bytes per product (n = 4096: 96 us, against 105 us for 128 x 256 tiles of one
-    // CTA; 8192 x 8192 x 4096: 351 / 425 us).  Products whose 128 x 128 tiles fit the SMs all at once take those: with pairs
-    // most of the SMs would stand idle.
+    // The time of a tile goes with the bytes its slices bring into an SM, in units of 64 elements x 128 rows (16 KB, about
+    // 270 clk); whole tiles are dealt out, so it also goes with the number of waves.
+    // CTA pairs move the fewest bytes per product (n = 4096: 96 us, against 105 us for 128 x 256 tiles of one CTA;
+    // 8192 x 8192 x 4096: 351 / 425 us); a tile width that just fills the last wave saves up to a third of it
+    // (420 x 6544 x 3840: 24.4 us 256 wide, 19.5 us 192 wide).
+    const long long slices = (K + 63) / 64;
+    const double kUnit = 270., kTile = 4000.;  // clk: 16 KB; filling the ring, and the epilogue that nothing overlaps
+    const long long pairs = sms / 2, rows = (M + 255) / 256;
+    int tile_n = 256;
+    double best = 0.;
+    for (int w = 256; w >= 64; w -= 64) {
+        const long long waves = (rows * ((N + w - 1) / w) + pairs - 1) / pairs;
+        const double cost = waves * slices * kUnit * (1. + w / 256.) + kTile;
+        if (w == 256 || cost < best) best = cost, tile_n = w;
+    }
+    // Few tiles: 128 x 128 tiles of one CTA each, or of a cluster that shares out K, which costs an exchange of the sums.
     const long long tiles = (long long)((M + 127) / 128) * ((N + 127) / 128);
-    if (tiles <= sms) return launch_gemm_tile<B_NMAJOR>(a, b, c, M, N, K, sms, s);
-    return launch_gemm_pair<B_NMAJOR>(a, b, c, M, N, K, sms, s);
+    int splits = 0;
+    for (int x = 1; x <= ave::GemmCfg::kMaxSplits; x *= 2) {
+        // (a cluster sits inside a GPC, so that not all SMs can be used by large ones: sixteen clusters of eight, or 35 of four,
+        // were not resident at once, and a second wave costs more than sharing K gains)
+        const long long resident = x == 8 ? 2 * sms / 3 : x == 4 ? 7 * sms / 8 : sms;
+        if (x > 1 && (x * 4 > slices || x * tiles > resident)) break;
+        const long long waves = (tiles * x + sms - 1) / sms;
+        const double cost = waves * ((slices + x - 1) / x * kUnit * 2. + kTile) + (x > 1 ? 2500. : 0.);
+        if (cost < best) best = cost, splits = x;
+    }
+    if (splits > 0) return launch_gemm_tile<B_NMAJOR>(a, b, c, M, N, K, splits, s);
+    return launch_gemm_pair<B_NMAJOR>(a, b, c, M, N, K, tile_n, sms, s);
 }
 
 // E4M3 codes [d2, rows, inner] (inner contiguous) as a 4-D map with boxes of 128 bytes x box_rows rows, 128-byte

@@ -617,7 +617,8 @@ int launch_gemm(const void *a, const void *b, void *c, int M, int N, int K, cuda
     double best = 0.;
     for (int w = 256; w >= 64; w -= 64) {
         const long long waves = (rows * ((N + w - 1) / w) + pairs - 1) / pairs;
-        const double cost = waves * slices * kUnit * (1. + w / 256.) + kTile;
+        const int loaded = B_NMAJOR ? (w + 127) / 128 * 128 : w;  // N-contiguous B comes in 64 columns per CTA at a time
+        const double cost = waves * slices * kUnit * (1. + loaded / 256.) + kTile;
         if (w == 256 || cost < best) best = cost, tile_n = w;
     }
     // Few tiles: 128 x 128 tiles of one CTA each, or of a cluster that shares out K, which costs an exchange of the sums.

@@ -143,6 +143,7 @@ attn_fwd_1t_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
             const bool leader = elect_one();
             bool ok = true;
             int last_id = blockIdx.x;   // the newest tile this CTA holds
+            unsigned requests = 0;      // phase of each slot's bar_tile_full
             for (int k = 0; ok; ++k) {
                 const int slot = k & 1;
                 if (k >= 2) {  // every consumer has read the tile this slot held two requests ago
@@ -154,18 +155,25 @@ attn_fwd_1t_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                     ok = wait_bar(&bar_tile_empty[slot ^ 1], ((k - 1) >> 1) & 1, STATUS_TIMEOUT_SLOT);
                     if (!ok) break;
                 }
-                if (leader) {
-                    mbar_arrive_expect_tx(smem_u32(&bar_tile_full[slot]), 16);
-                    clc_try_cancel(smem_u32(&clc_response[slot][0]), smem_u32(&bar_tile_full[slot]));
-                }
-                ok = wait_bar(&bar_tile_full[slot], (k >> 1) & 1, STATUS_TIMEOUT_SLOT);
-                if (!ok) break;
-                const int id = clc_decode(clc_response[slot]);
-                fence_proxy_async_smem();  // order the read before the slot's next asynchronous write
-                if (id >= 0) {
+                int id;
+                for (;;) {  // (past tiles beyond their sequence's end, see the two-sub-tile kernel)
+                    if (leader) {
+                        mbar_arrive_expect_tx(smem_u32(&bar_tile_full[slot]), 16);
+                        clc_try_cancel(smem_u32(&clc_response[slot][0]), smem_u32(&bar_tile_full[slot]));
+                    }
+                    ok = wait_bar(&bar_tile_full[slot], (requests >> slot) & 1, STATUS_TIMEOUT_SLOT);
+                    if (!ok) break;
+                    requests ^= 1u << slot;
+                    id = clc_decode(clc_response[slot]);
+                    fence_proxy_async_smem();  // order the read before the slot's next asynchronous write
+                    if (id < 0) break;
                     const Tile w = decode_tile<CAUSAL, SPLIT, VARLEN>(id, p);
+                    if constexpr (VARLEN)
+                        if (w.q0 >= w.sq) continue;
                     if (lane == 0) tile_info[slot] = w;
+                    break;
                 }
+                if (!ok) break;
                 if (lane == 0) tile_id[slot] = id;
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&bar_tile_ready[slot]));

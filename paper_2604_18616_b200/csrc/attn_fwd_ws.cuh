@@ -212,6 +212,7 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
             const bool leader = elect_one();
             bool ok = true;
             int last_id = blockIdx.x;   // the newest tile this CTA holds
+            unsigned requests = 0;      // phase of each slot's bar_tile_full
             for (int k = 0; ok; ++k) {
                 const int slot = k & 1;
                 if (k >= 2) {  // every consumer has read the response this slot held two requests ago
@@ -228,18 +229,28 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                     ok = wait_bar(&bar_tile_empty[slot ^ 1], ((k - 1) >> 1) & 1, STATUS_TIMEOUT_SLOT);
                     if (!ok) break;
                 }
-                if (leader) {
-                    mbar_arrive_expect_tx(smem_u32(&bar_tile_full[slot]), 16);
-                    clc_try_cancel(smem_u32(&clc_response[slot][0]), smem_u32(&bar_tile_full[slot]));
-                }
-                ok = wait_bar(&bar_tile_full[slot], (k >> 1) & 1, STATUS_TIMEOUT_SLOT);
-                if (!ok) break;
-                const int id = clc_decode(clc_response[slot]);
-                fence_proxy_async_smem();  // order the read before the slot's next asynchronous write
-                if (id >= 0) {
+                int id;
+                for (;;) {
+                    if (leader) {
+                        mbar_arrive_expect_tx(smem_u32(&bar_tile_full[slot]), 16);
+                        clc_try_cancel(smem_u32(&clc_response[slot][0]), smem_u32(&bar_tile_full[slot]));
+                    }
+                    ok = wait_bar(&bar_tile_full[slot], (requests >> slot) & 1, STATUS_TIMEOUT_SLOT);
+                    if (!ok) break;
+                    requests ^= 1u << slot;
+                    id = clc_decode(clc_response[slot]);
+                    fence_proxy_async_smem();  // order the read before the slot's next asynchronous write
+                    if (id < 0) break;
                     const TileOf<SPLIT, VARLEN> w = decode_tile<CAUSAL, SPLIT, VARLEN>(id, p);
+                    // Beyond its sequence's end there is nothing to compute or to write: the other warps never see the tile.
+                    // (A launch has a tile for every block of the longest sequence: 24 sequences of up to 2500 tokens, 40 %
+                    // of that on average, took 524 us when every warp went through the empty tiles, 463 us now.)
+                    if constexpr (VARLEN)
+                        if (w.q0 >= w.sq) continue;
                     if (lane == 0) tile_info[slot] = w;
+                    break;
                 }
+                if (!ok) break;
                 if (lane == 0) tile_id[slot] = id;
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&bar_tile_ready[slot]));

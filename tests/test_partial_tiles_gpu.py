@@ -1,0 +1,60 @@
+"""Launches in which much of the tile grid, of a tile, or of a hand-over is empty: variable-length batches of mostly short
+sequences (the tile scheduler passes over tiles beyond a sequence's end), tiles in which whole softmax warps have no query row,
+split-KV merges with one and with several warps per row, the fused MoE layer with many row tiles per expert, with more experts
+than rows and with very small activations.  Oracles and tolerances are those of the neighbouring parity tests."""
+import math
+
+import pytest
+import torch
+
+import oracle
+from paper_2604_18616_b200 import binding, inputs
+
+import parity
+from test_moe_gpu import check as check_moe, run_gpu as run_moe
+from test_splitkv_gpu import rand_qkv, run_split
+from test_varlen_gpu import _run_and_check
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("D,causal", [(64, False), (64, True), (128, False), (128, True), (256, True)])
+def test_variable_length_batch_of_mostly_empty_blocks(D, causal):
+    lens = [1, 0, 5, 700, 0, 0, 129, 3, 0, 128, 2, 64]
+    _run_and_check(lens, lens, 4, 2, D, causal, 5)
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("Sq", [1, 32, 33, 64, 96, 97, 128])
+def test_softmax_warps_without_a_row(D, Sq):
+    q, k, v = rand_qkv(Sq + D, 2, 2, 1, Sq, 391, D)
+    parity.check_full(q, k, v, True, 1.0 / math.sqrt(D), "Sq = %d, D = %d" % (Sq, D))
+
+
+@pytest.mark.parametrize("B,H,Hkv,Sq,Sk,D,n_splits", [
+    (1, 2, 2, 1, 9000, 64, 64),      # 2 rows: eight warps each, two ranges at a time
+    (1, 2, 2, 1, 4300, 128, 33),     # one range beyond a warp's 32
+    (4, 16, 16, 40, 700, 64, 5),     # 2560 rows: one warp each
+    (1, 3, 1, 1, 1500, 128, 4),      # a last CTA with rows beyond the end
+    (2, 4, 2, 100, 500, 128, 1),     # a single range, packed heads on 256-row tiles
+    (2, 4, 1, 3, 500, 64, 1),        # a single range, packed heads on 128-row tiles
+])
+def test_split_merge_shapes(B, H, Hkv, Sq, Sk, D, n_splits):
+    q, k, v = rand_qkv(H + Sk, B, H, Hkv, Sq, Sk, D)
+    scale = 1.0 / math.sqrt(D)
+    o, lse = run_split(q, k, v, True, scale, n_splits)
+    o_ref, lse_ref = oracle.attn_fwd(q, k, v, True, scale)
+    parity.compare(o, lse, o_ref, lse_ref, "split %d" % n_splits)
+
+
+@pytest.mark.parametrize("T,C,F,E,K,shrink", [
+    (1100, 128, 128, 1, 1, 1.0),      # nine row tiles of one expert: two groups of tiles
+    (20, 256, 128, 1000, 3, 1.0),     # most experts empty
+    (33, 640, 384, 3, 2, 1.0),        # odd numbers of weight blocks both ways
+    (40, 256, 256, 4, 2, 1e-10),      # requantisation groups far below fp32's reciprocal range of 448
+])
+def test_moe_edges(T, C, F, E, K, shrink):
+    args = list(inputs.make_moe_inputs(inputs.MoeWorkload("edge", T, C, F, E, K, T + E)))
+    args[1] = args[1] * shrink
+    y_ref = oracle.moe_fwd(*[t.numpy() for t in args])
+    check_moe(run_moe(args), y_ref, args, "moe %s" % ((T, C, F, E, K, shrink),))

@@ -307,19 +307,35 @@ int launch_1t(const CUtensorMap &tq, const CUtensorMap &tk, const CUtensorMap &t
     return AVE_OK;
 }
 
-// Whether an ordinary launch runs the single-sub-tile kernel (two CTAs per SM, 128-row tiles) instead of the
-// two-sub-tile one.
-bool use_one_subtile(int B, int H, int Hkv, int Sq, int Sk, int causal, bool split, bool varlen) {
+// Number of SMs of the current device (148, the part this library is written for, if it cannot be asked).
+int sm_count() {
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
+        sms = 148;
+    return sms;
+}
+
+// Whether a launch runs the single-sub-tile kernel (two CTAs per SM, 128-row tiles) instead of the two-sub-tile one.
+// `tiles`: 128-row tiles of the problem.
+bool use_one_subtile(int Sq, int Sk, bool causal, bool split, long long tiles) {
     const int choice = g_kernel_choice.load(std::memory_order_relaxed);
     if (choice == 1) return false;
     if (choice == 2) return true;
-    (void)B; (void)H; (void)Hkv; (void)Sk; (void)causal; (void)split; (void)varlen;
     // At most 128 query rows per problem (decode, one chunk of a chunked prefill; Sq counts the packed rows of a
     // head-packed split launch): the second sub-tile of a 256-row tile would be empty.  The single-sub-tile
     // kernel then keeps two independent K/V streams per SM in flight, which is what an HBM-bound pass needs
-    // (measured on decode shapes: 0.63-0.66 -> 0.76-0.90 of the copy bandwidth).  With more rows the shared
-    // K/V loads of the two-sub-tile kernel win (measured 6-15 % on the prefill configurations).
-    return Sq <= ave::BM;
+    // (measured on decode shapes: 0.63-0.66 -> 0.76-0.90 of the copy bandwidth).
+    if (Sq <= ave::BM) return true;
+    if (split) return false;
+    // Problems that do not fill the SMs: 128-row tiles spread over twice as many, and a lone CTA's step is shorter than that
+    // of two sub-tiles in lock-step (measured, two / one sub-tile: 8 heads of 300 rows 12.3 / 8.8 us, 8 heads of 1483 rows, causal,
+    // D = 128 30.3 / 25.9 us, 8 heads of 200 rows with 8000 keys 130 / 109 us).  A causal launch gains while every tile has a CTA
+    // slot of its own (8 heads of 3000 rows, 192 tiles: 54.2 / 47.1 us; 252 tiles 125.8 / 122.6 us; 384 tiles 61.0 / 66.2 us), a
+    // non-causal one only up to one tile per SM (192 tiles: 49.3 / 58.3 us), and with three key steps or fewer the tile's start
+    // and end outweigh the shared loads up to four tiles per SM (128 heads of 300 rows, 384 tiles: 24.6 / 22.6 us).
+    // Larger problems want the shared K/V loads of the two-sub-tile kernel (6-15 % on the prefill configurations).
+    const long long sms = sm_count();
+    return tiles <= sms || (causal && tiles <= 2 * sms) || (Sk <= 3 * ave::BN && tiles <= 4 * sms);
 }
 
 // Encode the tensor maps, fill the kernel parameters and launch.  In a `split` launch every work tile covers
@@ -344,10 +360,13 @@ int launch_attention(const void *q, const void *k, const void *v, void *o, float
     const Strides sv = layout ? layout[2] : varlen ? token_major(Hkv, rows_k) : contiguous_strides(Hkv, Sk, D);
     const Strides so = layout ? layout[3] : varlen ? token_major(H, rows_q) : contiguous_strides(H, Sq, D);
     // a head dimension above 128 leaves no TMEM for a second sub-tile: only the single-sub-tile kernel has it
-    const bool one = D > 128 || use_one_subtile(B, H, Hkv, Sq, Sk, causal, split, varlen != nullptr);
+    const long long tiles = (long long)H * (varlen ? (varlen->total_q / ave::BM + B) : (long long)B * ((Sq + ave::BM - 1) / ave::BM));
+    const bool one = D > 128 || use_one_subtile(Sq, Sk, causal != 0, split, tiles);
     CUtensorMap tq, tk, tv, to;
     if (!encode_map(&tq, q, D, rows_q, H, n_batch, sq, ave::BM)) return AVE_ERR_CUDA;
-    if (!one && !encode_map(&to, o, D, rows_q, H, n_batch, so, ave::WsCfg<128>::kOutBoxRows)) return AVE_ERR_CUDA;
+    // (the single-sub-tile kernel stores O without a map; beyond its 128 rows the choice between the kernels may change from
+    // call to call on the same buffers, and the map is kept for either)
+    if ((!one || Sq > ave::BM) && !encode_map(&to, o, D, rows_q, H, n_batch, so, ave::WsCfg<128>::kOutBoxRows)) return AVE_ERR_CUDA;
     if (!encode_map(&tk, k, D, rows_k, Hkv, n_batch, sk, ave::BN)) return AVE_ERR_CUDA;
     if (!encode_map(&tv, v, D, rows_k, Hkv, n_batch, sv, ave::BN)) return AVE_ERR_CUDA;
 

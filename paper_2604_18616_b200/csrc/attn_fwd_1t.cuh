@@ -23,7 +23,15 @@
 //
 // The same kernel serves head dimensions above 128 (instantiated for D = 256; 136..248 run it on tensor maps
 // of the true width, zero-filled): O then needs 256 TMEM columns, so a second sub-tile has no room, the CTA
-// allocates all 512 columns and, with 64 KB each for the Q, K and V tiles, has an SM to itself.
+// allocates all 512 columns and, with 64 KB for the Q tile, has an SM to itself.  What is left of TMEM holds a second
+// score buffer (S0 [0,128), O [128,384), S1 [384,512)): Q K_{j+1}^T runs while the softmax of step j does, where with
+// one buffer softmax, P V and Q K^T took turns.  K and V come through a ring of five 32 KB half tiles, K by halves of
+// D and V by halves of the keys, in the order of use K_0, K_1, V_0, K_2, V_1, ...: whole tiles would leave room for
+// one K and one V beside Q, and the next ones would have to land within one product's time.  2 x 32 heads of 4096,
+// causal, D = 256 622 -> 544 us; 64 heads of 4434 728 -> 625; D = 192, 32 heads of 1602 101 -> 86; 100 rows of 20000
+// keys, where the chain of steps is all there is, 351 -> 253.  What bounds it: the products alone take 416 us of the
+// 530 (at the power limit), and the loads of 128 KB a step compete with their operands for shared memory (without the
+// loads 459, without the softmax 464).
 #pragma once
 
 #include <type_traits>
@@ -40,15 +48,17 @@ struct OneCfg {
     static constexpr int kTileBytes = BM * D * 2;            // the Q tile, a K tile or a V tile
     static constexpr int kBoxBytes = BM * 64 * 2;            // one 64-column TMA box (128 rows x 128 B)
     static constexpr int kBoxes = D / 64;
-    static constexpr int kStages = (D >= 128) ? 2 : 4;       // ring slots, K and V tiles alternate (two CTAs must fit an SM)
-    static constexpr int kSmemBytes = kTileBytes * (1 + kStages) + 1024;
+    static constexpr bool kTwoS = (D > 128);                 // two score buffers, ring of half tiles
+    static constexpr int kSlotBytes = kTwoS ? kTileBytes / 2 : kTileBytes;
+    static constexpr int kStages = kTwoS ? 5 : (D >= 128) ? 2 : 4;  // ring slots, K and V tiles alternate (two CTAs must fit an SM)
+    static constexpr int kSmemBytes = kTileBytes + kStages * kSlotBytes + 1024;
     static constexpr int kCtasPerSm = (D <= 128) ? 2 : 1;
     static_assert(kCtasPerSm * (kSmemBytes + 2048) <= 228 * 1024, "the CTAs do not fit the shared memory of an SM");
     static constexpr uint32_t kTmemCols = (D <= 128) ? 256 : 512;
-    static_assert(128 + D <= int(kTmemCols), "S and O do not fit the TMEM allocation");
-    static constexpr uint32_t kColS = 0, kColO = 128;
-    static constexpr int kRegsLight = 48;                    // producer / MMA / scheduler warpgroup
-    static constexpr int kRegsSoftmax = 208;                 // softmax warpgroup
+    static_assert((kTwoS ? 256 : 128) + D <= int(kTmemCols), "S and O do not fit the TMEM allocation");
+    static constexpr uint32_t kColS = 0, kColO = 128, kColS1 = kTwoS ? 384 : 0;
+    static constexpr int kRegsLight = kTwoS ? 56 : 48;       // producer / MMA / scheduler warpgroup (48 spilled with the half tiles)
+    static constexpr int kRegsSoftmax = kTwoS ? 200 : 208;   // softmax warpgroup
     // Two CTAs per SM: 65536 / (2 x 256) = 128 registers per thread at launch; setmaxnreg only moves registers
     // inside that allocation (the build and the launch code check the compiled image against it).
     static constexpr int kRegsAtLaunch = 128;
@@ -67,7 +77,7 @@ attn_fwd_1t_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     constexpr int NS = Cfg::kStages;
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(16) unsigned long long clc_response[2][2];
-    __shared__ __align__(8) uint64_t bar_q_full, bar_q_empty, bar_s, bar_p, bar_o, bar_o_free;
+    __shared__ __align__(8) uint64_t bar_q_full, bar_q_empty, bar_s[2], bar_p[2], bar_pv, bar_o, bar_o_free;  // [score buffer]
     __shared__ __align__(8) uint64_t bar_full[NS], bar_empty[NS];
     __shared__ __align__(8) uint64_t bar_tile_full[2], bar_tile_ready[2], bar_tile_empty[2], bar_drain;
     __shared__ int tile_id[2];
@@ -86,11 +96,12 @@ attn_fwd_1t_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     if (tid == 0) {
         mbar_init(smem_u32(&bar_q_full), 1);
         mbar_init(smem_u32(&bar_q_empty), 1);
-        mbar_init(smem_u32(&bar_s), 1);
-        mbar_init(smem_u32(&bar_p), 4);       // one arrival per softmax warp
+        mbar_init(smem_u32(&bar_pv), 1);
         mbar_init(smem_u32(&bar_o), 1);
         mbar_init(smem_u32(&bar_o_free), 4);  // one arrival per softmax warp
         for (int t = 0; t < 2; ++t) {
+            mbar_init(smem_u32(&bar_s[t]), 1);
+            mbar_init(smem_u32(&bar_p[t]), 4);       // one arrival per softmax warp
             mbar_init(smem_u32(&bar_tile_full[t]), 1);
             mbar_init(smem_u32(&bar_tile_ready[t]), 1);
             mbar_init(smem_u32(&bar_tile_empty[t]), Cfg::kTileConsumers);
@@ -217,7 +228,9 @@ attn_fwd_1t_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                                         batch_coord(wt));
                     }
                 };
-                bool near_end = w.n0 <= 2;
+                constexpr int kLoadsPerStep = Cfg::kTwoS ? 4 : 2;
+                const int n_loads = kLoadsPerStep * w.n0;
+                bool near_end = n_loads <= 4;
                 auto poll_q = [&]() {
                     try_load_q(n, w, false);
                     if (!near_end) return;
@@ -227,9 +240,9 @@ attn_fwd_1t_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                     if (id_next >= 0) try_load_q(n + 1, w_next, false);
                 };
                 poll_q();
-                for (int it = 0; it < 2 * w.n0 && ok; ++it, ++ring) {  // it even: K_{it/2}; odd: V_{it/2}
+                for (int it = 0; it < n_loads && ok; ++it, ++ring) {  // whole tiles: it even: K_{it/2}; odd: V_{it/2}
                     const int slot = ring % NS, round = ring / NS;
-                    near_end = it + 4 >= 2 * w.n0;
+                    near_end = it + 4 >= n_loads;
                     if (round > 0) {
                         const long long t0 = clock64();
                         for (;;) {
@@ -254,11 +267,26 @@ attn_fwd_1t_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                     }
                     if (leader) {
                         const uint32_t bar = smem_u32(&bar_full[slot]);
-                        const CUtensorMap *tm = (it & 1) ? &tm_v : &tm_k;
-                        mbar_arrive_expect_tx(bar, Cfg::kTileBytes);
-                        for (int x = 0; x < Cfg::kBoxes; ++x)
-                            tma_load_4d(sRing + slot * Cfg::kTileBytes + x * Cfg::kBoxBytes, tm, bar, x * 64,
-                                        k_base_of(w) + key_begin(w) + (it >> 1) * BN, w.g, batch_coord(w));
+                        mbar_arrive_expect_tx(bar, Cfg::kSlotBytes);
+                        const int key0 = k_base_of(w) + key_begin(w);
+                        const uint32_t dst = sRing + slot * Cfg::kSlotBytes;
+                        if constexpr (Cfg::kTwoS) {
+                            // K_0 by halves, then by fours: the halves of K_{j+1} and of V_j; at the end those of the last V
+                            const int u = it - 2, j = u >> 2, part = u & 3;
+                            if (it < 2 || (j + 1 < w.n0 && part < 2)) {  // 128 of D's columns of 128 keys
+                                const int key = key0 + (it < 2 ? 0 : j + 1) * BN, d0 = (it & 1) * (D / 2);
+                                for (int x = 0; x < Cfg::kBoxes / 2; ++x)
+                                    tma_load_4d(dst + x * Cfg::kBoxBytes, &tm_k, bar, d0 + x * 64, key, w.g, batch_coord(w));
+                            } else {                                     // 64 keys
+                                const int key = key0 + j * BN + (it & 1) * (BN / 2);
+                                for (int x = 0; x < Cfg::kBoxes; ++x)
+                                    tma_load_4d(dst + x * (Cfg::kBoxBytes / 2), &tm_v, bar, x * 64, key, w.g, batch_coord(w));
+                            }
+                        } else {
+                            const CUtensorMap *tm = (it & 1) ? &tm_v : &tm_k;
+                            for (int x = 0; x < Cfg::kBoxes; ++x)
+                                tma_load_4d(dst + x * Cfg::kBoxBytes, tm, bar, x * 64, key0 + (it >> 1) * BN, w.g, batch_coord(w));
+                        }
                     }
                 }
                 if (ok) try_load_q(n, w, true);
@@ -277,35 +305,63 @@ attn_fwd_1t_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
             const uint32_t idesc_qk = make_idesc_bf16(BM, BN, 0) | ((p.scale_log2 < 0.f) ? (1u << 13) : 0u);
             constexpr uint32_t idesc_pv = make_idesc_bf16(BM, D, 1);
             constexpr uint64_t desc_kmajor = make_sdesc_sw128(16, 1024);
-            constexpr uint64_t desc_v = make_sdesc_sw128(BN * 128, 1024);
-            const uint32_t tS = tmem + Cfg::kColS, tO = tmem + Cfg::kColO;
+            constexpr uint64_t desc_v = make_sdesc_sw128((Cfg::kTwoS ? BN / 2 : BN) * 128, 1024);
+            const uint32_t tO = tmem + Cfg::kColO;
+            auto score_buf = [&](uint32_t i) { return tmem + (Cfg::kTwoS && (i & 1) ? Cfg::kColS1 : Cfg::kColS); };
             bool ok = true;
             int ring = 0;      // ring position of the current tile's K_0
-            uint32_t np = 0;   // P hand-offs taken so far (phase of bar_p)
+            uint32_t np = 0;   // P hand-offs taken so far (score buffer and phase of bar_p)
+            uint32_t nq = 0;   // Q K^T products issued so far (score buffer)
 
             auto wait_full = [&](int idx) { return wait_bar(&bar_full[idx % NS], (idx / NS) & 1, STATUS_TIMEOUT_LOAD); };
-            auto slot_addr = [&](int idx) { return sRing + (idx % NS) * Cfg::kTileBytes; };
+            auto slot_addr = [&](int idx) { return sRing + (idx % NS) * Cfg::kSlotBytes; };
             constexpr uint32_t hi_k = uint32_t(desc_kmajor >> 32), lo_k = uint32_t(desc_kmajor);
             constexpr uint32_t hi_v = uint32_t(desc_v >> 32), lo_v = uint32_t(desc_v);
             const uint32_t q_lo = lo_k | (sQ >> 4);
-            auto issue_qk = [&](uint32_t k_addr) {
-                if (leader) {
-                    const uint32_t k_lo = lo_k | (k_addr >> 4);
+            // S = Q K^T for the K tile at ring position `pos` (whole, or its halves at pos and pos + 1), and P V; the ring slots
+            // are handed back as their MMAs finish
+            auto issue_qk = [&](int pos) {
+                constexpr int kParts = Cfg::kTwoS ? 2 : 1, kSteps = D / 16 / kParts;
+                const uint32_t b = Cfg::kTwoS ? nq & 1 : 0, tS = score_buf(nq);
 #pragma unroll
-                    for (int kk = 0; kk < D / 16; ++kk) {
-                        const uint32_t koff = ((kk / 4) * Cfg::kBoxBytes + (kk % 4) * 32) >> 4;
-                        umma_ss_words(tS, q_lo + koff, hi_k, k_lo + koff, hi_k, idesc_qk, kk > 0);
+                for (int part = 0; part < kParts; ++part) {
+                    if (part > 0) ok = wait_full(pos + part);  // (the first has been waited for)
+                    if (!ok) return;
+                    tc_fence_after();
+                    if (leader) {
+                        const uint32_t k_lo = lo_k | (slot_addr(pos + part) >> 4);
+#pragma unroll
+                        for (int kk = 0; kk < kSteps; ++kk) {
+                            const int qk = part * kSteps + kk;
+                            const uint32_t qoff = ((qk / 4) * Cfg::kBoxBytes + (qk % 4) * 32) >> 4;
+                            const uint32_t koff = ((kk / 4) * Cfg::kBoxBytes + (kk % 4) * 32) >> 4;
+                            umma_ss_words(tS, q_lo + qoff, hi_k, k_lo + koff, hi_k, idesc_qk, qk > 0);
+                        }
+                        if (part == kParts - 1) umma_commit(smem_u32(&bar_s[b]));
+                        umma_commit(smem_u32(&bar_empty[(pos + part) % NS]));
                     }
-                    umma_commit(smem_u32(&bar_s));
                 }
+                ++nq;
             };
-            auto issue_pv = [&](uint32_t v_addr, bool first) {
-                if (leader) {
-                    const uint32_t v_lo = lo_v | (v_addr >> 4);
+            auto issue_pv = [&](int pos, bool first) {
+                constexpr int kParts = Cfg::kTwoS ? 2 : 1, kSteps = BN / 16 / kParts;
+                const uint32_t tP = score_buf(np);
 #pragma unroll
-                    for (int kk = 0; kk < BN / 16; ++kk)
-                        umma_ts_words(tO, tS + kk * 8, v_lo + ((kk * 16 * 128) >> 4), hi_v, idesc_pv, (!first || kk > 0));
+                for (int part = 0; part < kParts; ++part) {
+                    if (part > 0) ok = wait_full(pos + part);
+                    if (!ok) return;
+                    tc_fence_after();
+                    if (leader) {
+                        const uint32_t v_lo = lo_v | (slot_addr(pos + part) >> 4);
+#pragma unroll
+                        for (int kk = 0; kk < kSteps; ++kk)
+                            umma_ts_words(tO, tP + (part * kSteps + kk) * 8, v_lo + ((kk * 16 * 128) >> 4), hi_v, idesc_pv,
+                                          (!first || part > 0 || kk > 0));
+                        umma_commit(smem_u32(&bar_empty[(pos + part) % NS]));
+                    }
                 }
+                if (Cfg::kTwoS && leader) umma_commit(smem_u32(&bar_pv));
+                ++np;
             };
             // First step of tile number `tn` (tile `wt`, whose K_0 sits at ring position `ring0`): S = Q K_0^T,
             // issued right after the last P V of the tile before, so the pipeline does not drain at a tile boundary.
@@ -313,11 +369,8 @@ attn_fwd_1t_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                 ok = wait_bar(&bar_q_full, tn & 1, STATUS_TIMEOUT_LOAD);
                 if (ok && wt.n0 > 0) ok = wait_full(ring0);
                 if (!ok) return;
-                if (wt.n0 > 0) {
-                    tc_fence_after();
-                    issue_qk(slot_addr(ring0));
-                    if (leader) umma_commit(smem_u32(&bar_empty[ring0 % NS]));
-                }
+                if (wt.n0 > 0) issue_qk(ring0);
+                if (!ok) return;
                 if (leader && wt.n0 <= 1) umma_commit(smem_u32(&bar_q_empty));  // Q is released after its last Q K^T
             };
 
@@ -329,29 +382,33 @@ attn_fwd_1t_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                 Tile w_next = w;
                 const int id_next = next_tile(n, ok, w_next);
                 if (!ok) break;
-                const int ring_next = ring + 2 * nk;
+                const int ring_next = ring + (Cfg::kTwoS ? 4 : 2) * nk;
                 if (id_next >= 0 && nk == 0) start_tile(w_next, n + 1, ring_next);  // nothing to do in this tile
                 for (int j = 0; j < nk && ok; ++j) {
-                    const int iv = ring + 2 * j + 1, ik = ring + 2 * j + 2;  // ring positions of V_j and K_{j+1}
-                    ok = wait_full(iv);
-                    if (ok && j + 1 < nk) ok = wait_full(ik);
-                    // the previous tile's epilogue must have read O out of TMEM
-                    if (ok && j == 0 && n > 0) ok = wait_bar(&bar_o_free, (n - 1) & 1, STATUS_TIMEOUT_SOFTMAX);
-                    if (ok) ok = wait_bar(&bar_p, np & 1, STATUS_TIMEOUT_SOFTMAX);
-                    if (!ok) break;
-                    ++np;
-                    tc_fence_after();
-                    issue_pv(slot_addr(iv), j == 0);
-                    if (leader) umma_commit(smem_u32(&bar_empty[iv % NS]));
-                    if (leader && j == nk - 1) umma_commit(smem_u32(&bar_o));
-                    if (j + 1 < nk) {
-                        issue_qk(slot_addr(ik));
-                        if (leader) umma_commit(smem_u32(&bar_empty[ik % NS]));
-                        if (leader && j + 2 == nk) umma_commit(smem_u32(&bar_q_empty));
-                    } else if (id_next >= 0) {
-                        start_tile(w_next, n + 1, ring_next);
+                    // ring positions of V_j and K_{j+1}
+                    const int iv = ring + (Cfg::kTwoS ? (j + 1 < nk ? 4 * j + 4 : 4 * j + 2) : 2 * j + 1);
+                    const int ik = ring + (Cfg::kTwoS ? 4 * j + 2 : 2 * j + 2);
+                    auto next_scores = [&]() {
+                        issue_qk(ik);
+                        if (ok && leader && j + 2 == nk) umma_commit(smem_u32(&bar_q_empty));
+                    };
+                    if (Cfg::kTwoS && j + 1 < nk) {  // while the softmax of step j runs; P V_{j-1} has read the other buffer's P
+                        ok = wait_full(ik);
+                        if (ok) next_scores();
                         if (!ok) break;
                     }
+                    ok = wait_full(iv);
+                    if (!Cfg::kTwoS && ok && j + 1 < nk) ok = wait_full(ik);
+                    // the previous tile's epilogue must have read O out of TMEM
+                    if (ok && j == 0 && n > 0) ok = wait_bar(&bar_o_free, (n - 1) & 1, STATUS_TIMEOUT_SOFTMAX);
+                    if (ok) ok = Cfg::kTwoS ? wait_bar(&bar_p[np & 1], (np >> 1) & 1, STATUS_TIMEOUT_SOFTMAX)
+                                            : wait_bar(&bar_p[0], np & 1, STATUS_TIMEOUT_SOFTMAX);
+                    if (ok) issue_pv(iv, j == 0);
+                    if (!ok) break;
+                    if (leader && j == nk - 1) umma_commit(smem_u32(&bar_o));
+                    if (!Cfg::kTwoS && j + 1 < nk) next_scores();
+                    else if (j + 1 == nk && id_next >= 0) start_tile(w_next, n + 1, ring_next);
+                    if (!ok) break;
                 }
                 ring = ring_next;
                 id = id_next;
@@ -368,12 +425,13 @@ attn_fwd_1t_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
         const int wq = warp & 3;                      // TMEM lane quadrant of this warp
         const int r = wq * 32 + lane;                 // row within the tile = TMEM lane
         const uint32_t lane_sel = uint32_t(wq * 32) << 16;
-        const uint32_t tS = tmem + Cfg::kColS + lane_sel;
         const uint32_t tO = tmem + Cfg::kColO + lane_sel;
         // positive scale only; a negative one is applied by the tensor pipe, a zero one stands in as 2^-100
         // (see the two-sub-tile kernel)
         const float sl2 = (p.scale_log2 == 0.f) ? 7.888609052210118e-31f : fabsf(p.scale_log2);
-        uint32_t ns = 0;             // S tiles consumed so far (phase of bar_s)
+        uint32_t ns = 0;             // S tiles consumed so far (score buffer and phase of bar_s)
+        auto buf_of = [](uint32_t i) { return Cfg::kTwoS ? i & 1 : 0u; };
+        auto phase_of = [](uint32_t i) { return Cfg::kTwoS ? (i >> 1) & 1 : i & 1; };
         uint32_t n_out = 0;          // finished O accumulators taken so far (phase of bar_o)
         bool ok = true;
 
@@ -410,9 +468,9 @@ attn_fwd_1t_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                 // saves is energy: decode runs at the power limit, where the clocks follow it (64 sequences of 4001 keys 198 ->
                 // 190 us, 11 of 21249 with D = 64 60 -> 53 us).
                 for (int j = 0; j < n_t && ok; ++j) {
-                    ok = wait_bar(&bar_s, ns & 1, STATUS_TIMEOUT_MMA);
+                    ok = wait_bar(&bar_s[0], ns & 1, STATUS_TIMEOUT_MMA);
                     ++ns;
-                    if (ok && lane == 0) mbar_arrive(smem_u32(&bar_p));
+                    if (ok && lane == 0) mbar_arrive(smem_u32(&bar_p[0]));
                 }
                 if (ok) ok = wait_bar(&bar_o, n_out & 1, STATUS_TIMEOUT_MMA);
                 ++n_out;
@@ -427,7 +485,9 @@ attn_fwd_1t_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                     bool need_mask;
                     if constexpr (kRuntimeFlag) need_mask = masked;
                     else need_mask = decltype(masked)::value;
-                    ok = wait_bar(&bar_s, ns & 1, STATUS_TIMEOUT_MMA);
+                    const uint32_t buf = buf_of(ns);
+                    const uint32_t tS = tmem + (buf ? Cfg::kColS1 : Cfg::kColS) + lane_sel;
+                    ok = wait_bar(&bar_s[buf], phase_of(ns), STATUS_TIMEOUT_MMA);
                     if (!ok) return false;
                     ++ns;
                     tc_fence_after();
@@ -501,8 +561,14 @@ attn_fwd_1t_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                         }
                         // O <- alpha * O, after the exponentiation: the score registers are free by then, so the whole
                         // accumulator row (128 columns at a time) is in flight at once.  S(j) ready implies P V_{j-1} has
-                        // finished (in-order tensor pipe), and P V_j is not issued before this thread's arrival below.
+                        // finished (in-order tensor pipe; with two score buffers P V_{j-2}, and P V_{j-1} is waited
+                        // for), and P V_j is not issued before this thread's arrival below.
                         if (j > 0 && __any_sync(0xffffffffu, alpha != 1.f)) {
+                            if (Cfg::kTwoS) {
+                                ok = wait_bar(&bar_pv, (ns - 2) & 1, STATUS_TIMEOUT_MMA);  // the one numbered ns - 2
+                                if (!ok) return false;
+                                tc_fence_after();
+                            }
                             constexpr int kGroup = (D < 128) ? D : 128;
 #pragma unroll 1
                             for (int g = 0; g < D; g += kGroup) {
@@ -523,7 +589,7 @@ attn_fwd_1t_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                     tmem_wait_st();
                     tc_fence_before();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(smem_u32(&bar_p));
+                    if (lane == 0) mbar_arrive(smem_u32(&bar_p[buf]));
                     return true;
                 };
                 {

@@ -368,7 +368,8 @@ int launch_attention(const void *q, const void *k, const void *v, void *o, float
     // call to call on the same buffers, and the map is kept for either)
     if ((!one || Sq > ave::BM) && !encode_map(&to, o, D, rows_q, H, n_batch, so, ave::WsCfg<128>::kOutBoxRows)) return AVE_ERR_CUDA;
     if (!encode_map(&tk, k, D, rows_k, Hkv, n_batch, sk, ave::BN)) return AVE_ERR_CUDA;
-    if (!encode_map(&tv, v, D, rows_k, Hkv, n_batch, sv, ave::BN)) return AVE_ERR_CUDA;
+    // (head dimensions above 128 take V by halves of the keys)
+    if (!encode_map(&tv, v, D, rows_k, Hkv, n_batch, sv, D > 128 ? ave::BN / 2 : ave::BN)) return AVE_ERR_CUDA;
 
     ave::FwdParams p{};
     p.o = o;

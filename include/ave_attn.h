@@ -236,9 +236,10 @@ int ave_attn_device_status(unsigned int *raw_word);
 /*
  * The library has two attention kernels for the same operation: one whose CTAs
  * process two 128-row sub-tiles of a 256-row work tile in lock-step (shared K/V
- * loads; the default for long sequences and grouped-query heads), and one with
- * a single 128-row sub-tile per CTA and two CTAs per SM (no lock-step at tile
- * boundaries; better for short causal sequences).  which = 0 lets every call
+ * loads; the default for problems that fill the GPU), and one with a single
+ * 128-row sub-tile per CTA and two CTAs per SM (no lock-step at tile boundaries;
+ * the default for at most 128 query rows and where tiles do not fill the SMs,
+ * and the only one for D > 128).  which = 0 lets every call
  * choose by problem shape (the default), 1 / 2 force the first / second for all
  * later calls of this process.  Results agree within rounding order.  Returns
  * AVE_OK, or AVE_ERR_BAD_SHAPE for another value.

@@ -58,3 +58,13 @@ def test_moe_edges(T, C, F, E, K, shrink):
     args[1] = args[1] * shrink
     y_ref = oracle.moe_fwd(*[t.numpy() for t in args])
     check_moe(run_moe(args), y_ref, args, "moe %s" % ((T, C, F, E, K, shrink),))
+
+
+@pytest.mark.parametrize("H,Sq,Sk,causal", [
+    (74, 256, 400, False), (75, 256, 400, False),    # 148 / 150 tiles of 128 rows: one per SM, and more
+    (74, 512, 512, True), (75, 512, 512, True),      # 296 / 300: two per SM
+    (148, 400, 384, False), (148, 400, 385, False),  # 592 tiles of three / four key steps
+])
+def test_sides_of_the_kernel_choice(H, Sq, Sk, causal):
+    q, k, v = rand_qkv(H + Sk, 1, H, H, Sq, Sk, 64)
+    parity.check_full(q, k, v, causal, 0.125, "%s" % ((H, Sq, Sk, causal),))

@@ -14,8 +14,8 @@
  *   - for token t and each of its K routed experts e = ids[t,k] with weight w[t,k]:
  *       gate_j = sum_c x[t,c] W13[e, j, c],  up_j = sum_c x[t,c] W13[e, F + j, c]
  *       a_j = silu(gate_j) * up_j,  silu(z) = z / (1 + exp(-z))            (fp32)
- *       a is requantised per 128 columns: s = max|a| / 448, code = E4M3(a / s),
- *       round to nearest even, saturating
+ *       a is requantised per 128 columns: s = max|a| / 448 (1 where that is zero
+ *       in fp32), code = E4M3(a / s), round to nearest even, saturating
  *       y[t, i] += w[t,k] * sum_j a~_j W2[e, i, j]
  *     with x, W13, W2, a~ the dequantised values; y is rounded to bf16 once.
  *   Expert numbers are local to this GPU: a pair whose id is outside [0, E)

@@ -47,7 +47,8 @@ int ave_oracle_quant_groups(const float *a, int64_t n_groups, uint8_t *codes, fl
     for (int64_t g = 0; g < n_groups; ++g) {
         float amax = 0.0f;
         for (int c = 0; c < GROUP; ++c) amax = fmaxf(amax, fabsf(a[g * GROUP + c]));
-        const float s = (amax > 0.0f) ? amax / E4M3_MAX : 1.0f;          /* fp32 division */
+        float s = amax / E4M3_MAX;                                       /* fp32 division */
+        if (s == 0.0f) s = 1.0f;                                         /* all zero, or too small for a scale */
         scales[g] = s;
         for (int c = 0; c < GROUP; ++c) codes[g * GROUP + c] = ave_oracle_e4m3_encode(a[g * GROUP + c] / s);
     }

@@ -19,8 +19,9 @@
  *   - Weights are quantised per block of 128 x 128 (output rows x input
  *     channels): one fp32 scale per block.
  *   - Quantising a group of fp32 values a: s = max|a| / 448 computed in fp32
- *     (s = 1 if the group is all zero), code = E4M3(a / s) with the division in
- *     fp32, round to nearest even, saturating at +-448.
+ *     (s = 1 if that is zero: the group is all zero, or its largest value
+ *     below about 3e-43), code = E4M3(a / s) with the division in fp32, round
+ *     to nearest even, saturating at +-448.
  *   - Layer, for token t with its K routed experts e_k = ids[t,k] and routing
  *     weights w[t,k] (ids are local expert numbers in [0, E); tokens of other
  *     ranks' experts are not part of this GPU's problem):

@@ -417,7 +417,10 @@ moe_gemm_fp8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
                 if (!ok) break;
                 amax = fmaxf(buf[0], buf[Cfg::kTile]);
                 ++n_done;
-                const float s = amax > 0.f ? __fdiv_rn(amax, 448.f) : 1.f;
+                // (0 for a group of zeros, and where amax is so small, below 3.2e-43, that the quotient rounds to 0: with the
+                // factor 1 all of either's codes are 0)
+                float s = __fdiv_rn(amax, 448.f);
+                if (s == 0.f) s = 1.f;
                 if (half == 0) p.q_scale[(long long)bn * p.rows_cap + row] = s;
                 float sd = s;
                 if (s < 0x1p-60f) {  // a tiny group: scaled up exactly, so that 1 / s and the residuals stay normal

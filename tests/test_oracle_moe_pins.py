@@ -91,6 +91,17 @@ def test_block_quantiser_invariants():
     assert np.abs(deq - a)[~big].max() <= np.repeat(scales, 128, axis=1)[~big].max() * 2.0 ** -10 + 1e-12
 
 
+def test_block_quantiser_where_the_scale_underflows():
+    """Groups whose largest value over 448 is a subnormal, and zero, in fp32: the scale 0 is replaced by 1, so that neither
+    a / 0 nor 0 / 0 is ever encoded and the group dequantises to zero."""
+    a = np.zeros((2, 128), np.float32)
+    a[0, ::2] = 1e-42
+    a[1, ::2] = 1e-43
+    codes, scales = oracle.quant_groups(a)
+    assert scales[0, 0] == np.float32(1e-42) / np.float32(448.0) > 0 and scales[1, 0] == 1.0
+    assert np.all(codes[0, 1::2] == 0) and np.all(codes[1] == 0)
+
+
 # -------------------------------------------------------------------------------- the layer
 def tiny(seed=3, T=5, C=256, F=128, E=3, K=2):
     w = inputs.MoeWorkload("tiny", T, C, F, E, K, seed)

@@ -133,10 +133,12 @@ __device__ __forceinline__ float2 div2_residual(float2 x, float2 d, float2 r) {
     const float2 e = __ffma2_rn(make_float2(-q.x, -q.y), d, x);
     return __ffma2_rn(e, r, q);
 }
-// silu(z) = z / (1 + exp(-z)) for two values in fp32.  Below -87 the exponential is held at exp(87): the result is then
-// z * 1.6e-38 instead of a subnormal or zero.
+// silu(z) = z / (1 + exp(-z)) in fp32, for any z: from -88.8 down the exponential is infinite and the result -0.
+__device__ __forceinline__ float silu(float z) { return __fdiv_rn(z, 1.f + expf(-z)); }
+// The same for two values of at least kSiluFast, below which 1 / (1 + exp(-z)) is no longer a normal number.
+constexpr float kSiluFast = -87.f;
 __device__ __forceinline__ float2 silu2(float2 z) {
-    const float2 d = make_float2(1.f + expf(-fmaxf(z.x, -87.f)), 1.f + expf(-fmaxf(z.y, -87.f)));
+    const float2 d = make_float2(1.f + expf(-z.x), 1.f + expf(-z.y));
     float2 r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r.x) : "f"(d.x));
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r.y) : "f"(d.y));
@@ -403,11 +405,27 @@ moe_gemm_fp8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
             if (!ok) break;
             if constexpr (UP) {
                 // a = silu(gate) * up; the group's maximum with the thread that has the row's other 64 columns; codes
-                float amax = 0.f;
+                float amax = 0.f, lowest = 0.f;
 #pragma unroll
-                for (int c = 0; c < 32; ++c) {
-                    acc[c] = __fmul2_rn(silu2(acc[c]), acc[c + 32]);
-                    amax = fmaxf(amax, fmaxf(fabsf(acc[c].x), fabsf(acc[c].y)));
+                for (int c = 0; c < 32; ++c) lowest = fminf(lowest, fminf(acc[c].x, acc[c].y));
+                if (__any_sync(0xffffffffu, lowest < kSiluFast)) {
+                    // (no model's gates.  A loop that turns the registers round, so that the code a tile usually jumps over is
+                    // short: 64 divisions in line were 1 % of the layer in instruction fetches)
+#pragma unroll 1
+                    for (int x = 0; x < 32; ++x) {
+                        const float2 gate = acc[0], up = acc[32];
+#pragma unroll
+                        for (int c = 0; c < 31; ++c) acc[c] = acc[c + 1], acc[c + 32] = acc[c + 33];
+                        acc[31] = make_float2(silu(gate.x) * up.x, silu(gate.y) * up.y);
+                        acc[63] = up;
+                        amax = fmaxf(amax, fmaxf(fabsf(acc[31].x), fabsf(acc[31].y)));
+                    }
+                } else {
+#pragma unroll
+                    for (int c = 0; c < 32; ++c) {
+                        acc[c] = __fmul2_rn(silu2(acc[c]), acc[c + 32]);
+                        amax = fmaxf(amax, fmaxf(fabsf(acc[c].x), fabsf(acc[c].y)));
+                    }
                 }
                 float *const buf = &row_max[n_done & 1][0][wq * 32 + lane];
                 buf[half * Cfg::kTile] = amax;

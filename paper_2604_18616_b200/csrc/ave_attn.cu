@@ -464,10 +464,11 @@ splitkv_merge_kernel(const float *__restrict__ o_partial, const float *__restric
         const int stride = warps_per_row * ranges_at_once;
 #pragma unroll 4
         for (int s0 = sub * ranges_at_once; s0 < n_splits; s0 += stride) {
-            const int s = s0 + lane / lanes_per_range;  // (beyond the last range: weight 0, the last range's values)
+            const int s = s0 + lane / lanes_per_range;
             const float w_lo = __shfl_sync(0xffffffffu, w0, s & 31), w_hi = __shfl_sync(0xffffffffu, w1, s & 31);
-            const float ws = s < n_splits ? (s < 32 ? w_lo : w_hi) : 0.f;
-            const float4 v = reinterpret_cast<const float4 *>(o_partial + (min(s, n_splits - 1) * rows + row) * D)[col4];
+            const float ws = s < 32 ? w_lo : w_hi;
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);  // (beyond the last range: nothing, not 0 x another range's infinity)
+            if (s < n_splits) v = reinterpret_cast<const float4 *>(o_partial + (s * rows + row) * D)[col4];
             acc.x += ws * v.x; acc.y += ws * v.y; acc.z += ws * v.z; acc.w += ws * v.w;
         }
     }

@@ -1,5 +1,5 @@
-"""Values at the ends of the number range: MoE intermediates whose requantisation scale underflows, and gates far below the
-point where exp(-gate) overflows."""
+"""Values at the ends of the number range: MoE intermediates whose requantisation scale underflows, gates far below the point
+where exp(-gate) overflows, and infinities among the values of a split-KV call."""
 import numpy as np
 import pytest
 import torch
@@ -8,6 +8,7 @@ import oracle
 from paper_2604_18616_b200 import inputs
 
 from test_moe_gpu import check as check_moe, run_gpu as run_moe
+from test_splitkv_gpu import rand_qkv, run_split
 
 pytestmark = pytest.mark.gpu
 
@@ -47,3 +48,14 @@ def test_moe_gates_of_any_size(sign):
         # zero to fp32's exp(-z), which overflows
         assert np.all(np.abs(y - ref) <= 2.0 ** -4 * np.abs(ref) + 1e-35), "gates of %g: %g, oracle %g" % (
             sign * size, y[0, 0], ref[0, 0])
+
+
+def test_infinite_value_in_the_last_of_an_odd_number_of_ranges():
+    B, H, Sq, Sk, D, n_splits = 1, 2, 3, 384, 64, 3
+    q, k, v = rand_qkv(11, B, H, H, Sq, Sk, D)
+    v[0, :, Sk - 1, 7] = float("inf")
+    o, lse = run_split(q, k, v, False, 0.125, n_splits)
+    assert torch.isfinite(lse).all()
+    assert torch.all(o[..., 7] == float("inf"))
+    rest = [c for c in range(D) if c != 7]
+    assert torch.isfinite(o[..., rest].float()).all()

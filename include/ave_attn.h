@@ -167,7 +167,8 @@ size_t ave_attn_host_workspace_bytes(int B, int H, int Hkv, int Sq, int Sk, int 
  * bytes, 256-byte aligned, owned by the caller; it holds the fp32 partial
  * outputs and log-sum-exps, is fully rewritten by each call, and may be
  * reused by later calls on the same stream.  Two kernels are enqueued (one, and
- * no scratch is touched, with n_splits = 1).
+ * no scratch is touched, with n_splits = 1 where every row sees a key: not
+ * causal, or Sq <= Sk).
  */
 #define AVE_SPLITKV_MAX_SPLITS 64
 int ave_attn_fwd_splitkv(const void *q, const void *k, const void *v, void *o, float *lse,

@@ -462,8 +462,9 @@ splitkv_merge_kernel(const float *__restrict__ o_partial, const float *__restric
 #pragma unroll
         for (int x = 16; x > 0; x >>= 1) denom += __shfl_xor_sync(0xffffffffu, denom, x);
         const int stride = warps_per_row * ranges_at_once;
+        const int n = m == -INFINITY ? 0 : n_splits;  // (a row that sees no key in any range: what the partials hold is not looked at)
 #pragma unroll 4
-        for (int s0 = sub * ranges_at_once; s0 < n_splits; s0 += stride) {
+        for (int s0 = sub * ranges_at_once; s0 < n; s0 += stride) {
             const int s = s0 + lane / lanes_per_range;
             const float w_lo = __shfl_sync(0xffffffffu, w0, s & 31), w_hi = __shfl_sync(0xffffffffu, w1, s & 31);
             const float ws = s < 32 ? w_lo : w_hi;
@@ -516,14 +517,16 @@ int run_splitkv(const void *q, const void *k, const void *v, void *o, float *lse
     const int kps = ave::splitkv_keys_per_split(Sk, n_splits);
     const int G = H / Hkv;
     const bool pack = ave::splitkv_packs_heads(H, Hkv, Sq);  // query heads of a KV head as rows of one problem
-    // a single key range needs no merge: the attention kernel writes the result
-    float *const op = n_splits > 1 ? o_partial : nullptr;
-    float *const lp = n_splits > 1 ? lse_partial : nullptr;
+    // A single key range needs no merge: the attention kernel writes the result.  (It makes the O of a row without any visible
+    // key by a product with 0, which infinite values turn into NaN, where the merge writes zeros.)
+    const bool merge = n_splits > 1 || (causal && Sq > Sk);
+    float *const op = merge ? o_partial : nullptr;
+    float *const lp = merge ? lse_partial : nullptr;
     const int st = pack ? launch_attention(q, k, v, o, lse, B, Hkv, Hkv, G * Sq, Sk, D, causal, scale, true, n_splits, kps,
                                            op, lp, Sq, nullptr, nullptr, s)
-                        : launch_attention(q, k, v, o, lse, B, H, Hkv, Sq, Sk, D, causal, scale, n_splits > 1, n_splits,
+                        : launch_attention(q, k, v, o, lse, B, H, Hkv, Sq, Sk, D, causal, scale, merge, n_splits,
                                            kps, op, lp, 0, nullptr, nullptr, s);
-    if (st != AVE_OK || n_splits == 1) return st;
+    if (st != AVE_OK || !merge) return st;
     const long long rows = (long long)B * H * Sq;
     // enough warps to cover the chip a few times over, none with less than two ranges to add up
     constexpr int kWarps = kMergeThreads / 32;

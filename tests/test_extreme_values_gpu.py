@@ -59,3 +59,15 @@ def test_infinite_value_in_the_last_of_an_odd_number_of_ranges():
     assert torch.all(o[..., 7] == float("inf"))
     rest = [c for c in range(D) if c != 7]
     assert torch.isfinite(o[..., rest].float()).all()
+
+
+@pytest.mark.parametrize("H,Hkv,Sq,Sk", [(2, 2, 200, 150), (4, 2, 60, 40)])  # the second: packed query heads
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("n_splits", [1, 2])
+def test_rows_without_keys_are_zero_whatever_the_values_are(n_splits, D, H, Hkv, Sq, Sk):
+    # Sq > Sk, causal: the first rows see no key, but share their tile with rows that see infinite values
+    q, k, v = rand_qkv(12, 1, H, Hkv, Sq, Sk, D)
+    v[0, :, 10, 3] = float("inf")
+    o, lse = run_split(q, k, v, True, 0.1, n_splits)
+    assert torch.all(lse[:, :, :Sq - Sk] == float("-inf")) and torch.all(o[:, :, :Sq - Sk] == 0)
+    assert torch.isfinite(lse[:, :, Sq - Sk:]).all() and torch.all(o[:, :, Sq - Sk + 10:, 3] == float("inf"))

@@ -170,8 +170,10 @@ _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or (
 
 def _call(name, tensor, stream, *args):
     """Run the library function on the tensor's device and stream (the device's current one if None); raise on error."""
-    fn = getattr(lib(), name)
     device = tensor.get_device()
+    if device < 0:  # (a torch.cuda.device(-1) block does nothing, and the library would hand host addresses to its kernels)
+        raise ValueError("%s: expected CUDA tensors" % name)
+    fn = getattr(lib(), name)
     if device == _current_device():
         st = fn(*args, _raw_stream(device) if stream is None else stream.cuda_stream)
     else:
@@ -298,12 +300,23 @@ def splitkv_default_splits(B, H, Hkv, Sq, Sk, D) -> int:
     return int(lib().ave_attn_splitkv_default_splits(B, H, Hkv, Sq, Sk, D))
 
 
+def _check_qkv(q, k, v):
+    """The checks of ave_attn_fwd for its split-KV variants; the sizes B, H, Hkv, Sq, Sk, D."""
+    for t in (q, k, v):
+        if not (t.is_cuda and t.dtype is torch.bfloat16 and t.dim() == 4 and t.is_contiguous()):
+            raise ValueError("q, k, v must be contiguous 4-D CUDA bfloat16 tensors")
+    B, H, Sq, D = q.shape
+    Bk, Hkv, Sk, Dk = k.shape
+    if v.shape != k.shape or Bk != B or Dk != D:
+        raise ValueError("inconsistent q/k/v shapes")
+    return B, H, Hkv, Sq, Sk, D
+
+
 def ave_attn_fwd_splitkv(q, k, v, n_splits, workspace=None, o=None, lse=None, causal=False, scale=None, stream=None):
     """Split-KV variant of ``ave_attn_fwd``: same tensors and result; ``workspace``
     is a CUDA uint8 tensor of at least ``splitkv_workspace_bytes`` bytes
     (allocated here when not given)."""
-    B, H, Sq, D = q.shape
-    _, Hkv, Sk, _ = k.shape
+    B, H, Hkv, Sq, Sk, D = _check_qkv(q, k, v)
     if o is None:
         o = torch.empty_like(q)
     if lse is None:
@@ -325,8 +338,7 @@ def ave_attn_fwd_splitkv_static(q, k, v, n_splits, o, lse, causal=False, scale=N
     library, ``SPLITKV_STATIC_SCRATCH_BYTES`` per GPU.  ``o`` and ``lse`` must be
     passed in, so this wrapper allocates nothing either.  Calls sharing a
     device must not overlap on the GPU."""
-    B, H, Sq, D = q.shape
-    _, Hkv, Sk, _ = k.shape
+    B, H, Hkv, Sq, Sk, D = _check_qkv(q, k, v)
     if scale is None:
         scale = D ** -0.5
     _call("ave_attn_fwd_splitkv_static", q, stream, q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), lse.data_ptr(),

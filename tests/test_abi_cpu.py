@@ -187,3 +187,29 @@ def test_moe_validation_before_any_cuda_call(lib):
     n = binding.moe_workspace_bytes(4096, 7168, 2048, 32, 4)
     rows = 128 * (4096 * 4 // 128 + 32)
     assert n >= rows * (7168 + 7168 * 4 + 2048) and n % 256 == 0
+
+
+@pytest.mark.parametrize("bad", ["q", "k", "v"])
+def test_splitkv_wrappers_refuse_host_tensors(monkeypatch, bad):
+    """A host address must not reach the library, which would give it to the GPU.  (Tensors that claim to be on a GPU stand
+    in for the other two; the library is replaced by one that must not be called.)"""
+    import torch
+
+    class Claims(torch.Tensor):
+        is_cuda = True
+
+    def refuse():
+        raise AssertionError("the library was reached")
+
+    monkeypatch.setattr(binding, "lib", refuse)
+    t = {n: torch.zeros(1, 2, 8, 64, dtype=torch.bfloat16) for n in "qkv"}
+    for n in t:
+        if n != bad:
+            t[n] = t[n].as_subclass(Claims)
+    o, lse, ws = torch.zeros(1, 2, 8, 64, dtype=torch.bfloat16), torch.zeros(1, 2, 8), torch.zeros(1 << 16, dtype=torch.uint8)
+    with pytest.raises(ValueError):
+        binding.ave_attn_fwd_splitkv(t["q"], t["k"], t["v"], 2, workspace=ws, o=o, lse=lse)
+    with pytest.raises(ValueError):
+        binding.ave_attn_fwd_splitkv_static(t["q"], t["k"], t["v"], 2, o, lse)
+    with pytest.raises(ValueError):   # whatever the wrappers check: no call without a device
+        binding._call("ave_attn_fwd", torch.zeros(1), None)

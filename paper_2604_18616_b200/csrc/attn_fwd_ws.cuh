@@ -239,7 +239,9 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                     if (!ok) break;
                     requests ^= 1u << slot;
                     id = clc_decode(clc_response[slot]);
-                    fence_proxy_async_smem();  // order the read before the slot's next asynchronous write
+                    // order the reads, every lane's, before the slot's next asynchronous write (the next trip may ask for it)
+                    fence_proxy_async_smem();
+                    __syncwarp();
                     if (id < 0) break;
                     const TileOf<SPLIT, VARLEN> w = decode_tile<CAUSAL, SPLIT, VARLEN>(id, p);
                     // Beyond its sequence's end there is nothing to compute or to write: the other warps never see the tile.

@@ -68,3 +68,16 @@ def test_moe_edges(T, C, F, E, K, shrink):
 def test_sides_of_the_kernel_choice(H, Sq, Sk, causal):
     q, k, v = rand_qkv(H + Sk, 1, H, H, Sq, Sk, 64)
     parity.check_full(q, k, v, causal, 0.125, "%s" % ((H, Sq, Sk, causal),))
+
+
+@pytest.mark.parametrize("Hkv", [1, 2])   # (1: paired heads in the causal two-sub-tile kernel; 2: 256-row tiles)
+@pytest.mark.parametrize("kernel", [binding.KERNEL_TWO_SUBTILES, binding.KERNEL_ONE_SUBTILE])
+def test_scheduler_passes_over_long_runs_of_empty_tiles(kernel, Hkv):
+    """One sequence of 2100 tokens among 300 of at most three: nearly every tile of the grid lies beyond its sequence's end, so
+    that each CTA's scheduler asks for the next tile many times over before it has one to hand on."""
+    lens = [i % 4 for i in range(150)] + [2100] + [3 - i % 4 for i in range(150)]
+    assert binding.select_kernel(kernel) == binding.AVE_OK
+    try:
+        _run_and_check(lens, lens, 2, Hkv, 64, True, 8)
+    finally:
+        assert binding.select_kernel(binding.KERNEL_AUTO) == binding.AVE_OK

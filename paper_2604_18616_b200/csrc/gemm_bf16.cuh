@@ -78,7 +78,7 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t bar_full[NS], bar_empty[NS], bar_acc_full, bar_drain;
     __shared__ uint32_t tmem_base_slot;
-    __shared__ int abort_flag;
+    __shared__ int abort_flag, missing_sums;  // the second: another CTA of the cluster has no sums to send
 
     const int tid = threadIdx.x;
     const int warp = tid >> 5;
@@ -87,6 +87,7 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
     const uint32_t sRecv = sRing + NS * Cfg::kStageBytes;
 
     if (tid == 0) {
+        missing_sums = 0;
         for (int s = 0; s < NS; ++s) {
             mbar_init(smem_u32(&bar_full[s]), 1);
             mbar_init(smem_u32(&bar_empty[s]), 1);
@@ -246,7 +247,12 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
                         st_cluster_v4(dst + ((c + e) / 4) * (128 * 16), v[e], v[e + 1], v[e + 2], v[e + 3]);
                 }
             }
+            // A CTA that found the status word set, or gave up a wait, has sent nothing: the others may have read the word before
+            // it was set, and must not add up, and store, what was never written here.
+            if (!ok && lane < S && lane != rank) st_cluster_s32(map_to_cta(smem_u32(&missing_sums), lane), 1);
+            __syncwarp();
             cluster_sync();
+            ok = ok && *reinterpret_cast<volatile int *>(&missing_sums) == 0;
             const int row = row0 + lane;
             for (int c = 0; c < cols && ok; c += 16) {
                 uint32_t own[16];

@@ -48,3 +48,22 @@ def test_shared_k_and_narrow_tiles(layout, M, N, K):
     err = np.abs(c.cpu().double().numpy() - ref)
     tol = 2.0 ** -8 * np.abs(ref) + 1e-3 * math.sqrt(K)
     assert np.all(err <= tol), "max error %.3g" % err.max()
+
+
+def test_clusters_write_nothing_while_the_status_word_is_set():
+    """200 x 512 x 2048 runs as clusters of eight CTAs; all of them leave C alone until the word is read, and work after."""
+    M, N, K = 200, 512, 2048
+    a, b = inputs.make_gemm_inputs(M, N, K, 5)
+    dev = torch.device("cuda:0")
+    ad, bd = a.to(dev), b.to(dev)
+    c = torch.full((M, N), 7.0, dtype=torch.bfloat16, device=dev)
+    assert binding.device_status() == (binding.AVE_OK, 0)
+    assert binding.selftest_wait_timeout(16) == binding.AVE_OK
+    binding.ave_gemm_bf16_tn(ad, bd, c)
+    torch.cuda.synchronize()
+    assert torch.all(c == 7.0)
+    assert binding.device_status() == (binding.AVE_ERR_DEVICE_TIMEOUT, binding.STATUS_BIT_SELFTEST)
+    binding.ave_gemm_bf16_tn(ad, bd, c)
+    assert binding.device_status() == (binding.AVE_OK, 0)
+    ref = oracle.gemm_tn(a, b)
+    assert np.all(np.abs(c.cpu().double().numpy() - ref) <= 2.0 ** -8 * np.abs(ref) + 1e-3 * math.sqrt(K))

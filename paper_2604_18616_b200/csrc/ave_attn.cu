@@ -315,9 +315,9 @@ int sm_count() {
     return sms;
 }
 
-// Whether a launch runs the single-sub-tile kernel (two CTAs per SM, 128-row tiles) instead of the two-sub-tile one.
-// `tiles`: 128-row tiles of the problem.
-bool use_one_subtile(int Sq, int Sk, bool causal, bool split, long long tiles) {
+// Whether a launch of D <= 128 runs the single-sub-tile kernel (two CTAs per SM, 128-row tiles) instead of the two-sub-tile
+// one.  total_q: query rows of all sequences of a variable-length launch, else 0.
+bool use_one_subtile(int B, int H, int Hkv, int Sq, int Sk, int D, bool causal, bool split, int total_q) {
     const int choice = g_kernel_choice.load(std::memory_order_relaxed);
     if (choice == 1) return false;
     if (choice == 2) return true;
@@ -326,16 +326,7 @@ bool use_one_subtile(int Sq, int Sk, bool causal, bool split, long long tiles) {
     // kernel then keeps two independent K/V streams per SM in flight, which is what an HBM-bound pass needs
     // (measured on decode shapes: 0.63-0.66 -> 0.76-0.90 of the copy bandwidth).
     if (Sq <= ave::BM) return true;
-    if (split) return false;
-    // Problems that do not fill the SMs: 128-row tiles spread over twice as many, and a lone CTA's step is shorter than that
-    // of two sub-tiles in lock-step (measured, two / one sub-tile: 8 heads of 300 rows 12.3 / 8.8 us, 8 heads of 1483 rows, causal,
-    // D = 128 30.3 / 25.9 us, 8 heads of 200 rows with 8000 keys 130 / 109 us).  A causal launch gains while every tile has a CTA
-    // slot of its own (8 heads of 3000 rows, 192 tiles: 54.2 / 47.1 us; 252 tiles 125.8 / 122.6 us; 384 tiles 61.0 / 66.2 us), a
-    // non-causal one only up to one tile per SM (192 tiles: 49.3 / 58.3 us), and with three key steps or fewer the tile's start
-    // and end outweigh the shared loads up to four tiles per SM (128 heads of 300 rows, 384 tiles: 24.6 / 22.6 us).
-    // Larger problems want the shared K/V loads of the two-sub-tile kernel (6-15 % on the prefill configurations).
-    const long long sms = sm_count();
-    return tiles <= sms || (causal && tiles <= 2 * sms) || (Sk <= 3 * ave::BN && tiles <= 4 * sms);
+    return !split && ave::one_subtile_is_faster(B, H, Hkv, Sq, Sk, D, causal, total_q, sm_count());
 }
 
 // Encode the tensor maps, fill the kernel parameters and launch.  In a `split` launch every work tile covers
@@ -360,8 +351,7 @@ int launch_attention(const void *q, const void *k, const void *v, void *o, float
     const Strides sv = layout ? layout[2] : varlen ? token_major(Hkv, rows_k) : contiguous_strides(Hkv, Sk, D);
     const Strides so = layout ? layout[3] : varlen ? token_major(H, rows_q) : contiguous_strides(H, Sq, D);
     // a head dimension above 128 leaves no TMEM for a second sub-tile: only the single-sub-tile kernel has it
-    const long long tiles = (long long)H * (varlen ? (varlen->total_q / ave::BM + B) : (long long)B * ((Sq + ave::BM - 1) / ave::BM));
-    const bool one = D > 128 || use_one_subtile(Sq, Sk, causal != 0, split, tiles);
+    const bool one = D > 128 || use_one_subtile(B, H, Hkv, Sq, Sk, D, causal != 0, split, varlen ? varlen->total_q : 0);
     CUtensorMap tq, tk, tv, to;
     if (!encode_map(&tq, q, D, rows_q, H, n_batch, sq, ave::BM)) return AVE_ERR_CUDA;
     // (the single-sub-tile kernel stores O without a map; beyond its 128 rows the choice between the kernels may change from

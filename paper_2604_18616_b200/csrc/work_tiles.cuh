@@ -255,6 +255,36 @@ inline bool plan_work_tiles(FwdParams &p, int B, int H, int Hkv, int Sq, int Sk,
     return true;
 }
 
+// Whether a problem of more than 128 query rows and D <= 128, its keys not split, is better off in the single-sub-tile kernel
+// (128-row tiles, two CTAs per SM) than in the two-sub-tile one, on a part with `sms` SMs.  total_q: query rows of all
+// sequences of a variable-length launch (Sq and Sk are its maxima), else 0.  Times below: two / one sub-tile.
+inline bool one_subtile_is_faster(int B, int H, int Hkv, int Sq, int Sk, int D, bool causal, int total_q, int sms) {
+    auto blocks = [&](int rows) {
+        return total_q > 0 ? (long long)total_q / rows + B : (long long)B * (((long long)Sq + rows - 1) / rows);
+    };
+    const long long tiles = H * blocks(BM);
+    // Problems that do not fill the SMs: 128-row tiles spread over twice as many, and a lone CTA's step is shorter than that
+    // of two sub-tiles in lock-step (8 heads of 300 rows 12.3 / 8.8 us, 8 heads of 200 rows with 8000 keys 130 / 109 us; causal,
+    // 96-144 tiles: 0.77-0.92 of the time, whatever Sk).  With three key steps or fewer the tile's start and end outweigh the
+    // shared loads up to four tiles per SM (128 heads of 300 rows, 384 tiles: 24.6 / 22.6 us).
+    if (tiles <= sms || (Sk <= 3 * BN && tiles <= 4 * sms)) return true;
+    // Up to two tiles per SM, causal.  Tiles start longest first, and the sms-th shares an SM with a long one, so that its
+    // length counts: little where Sk = Sq (8 heads of 3072 rows, D = 64: 46.4 / 39.0 us), nearly all keys for a chunk of a
+    // prompt after cached ones (after 46080 keys: 605 / 669 us).  In units of the longest tile's time in the two-sub-tile
+    // kernel, a fit to 492 shapes with Sk from Sq to 9 Sq (0.035 rms; the choice that follows costs at
+    // most 5 % against the better kernel, 0.1 % on average; always one sub-tile cost 4 % on average, up to 18 %, at D = 128):
+    if (!causal || tiles > 2 * sms) return false;
+    const double fall = Sq < Sk ? double(Sq) / Sk : 1.;  // by how much tile lengths fall from the first tile to the last
+    const double last = 1. - fall * sms / tiles;         // length of the sms-th
+    const double one = D <= 64 ? 0.655 + 0.28 * last + 0.117 * tiles / sms : 0.765 + 0.24 * last + 0.09 * tiles / sms;
+    // The two-sub-tile kernel has all of its tiles (pairs of heads, or of blocks) at work at once, or needs a second wave
+    // (8 heads of 4736 rows, 152 of its tiles, after 4736 keys: 209 / 157 us).
+    const long long tiles_two = H / Hkv % 2 == 0 ? tiles / 2 : H * blocks(2 * BM);
+    const double two = tiles_two <= sms ? 1. : 2. - fall * sms / tiles_two;
+    return one < two;
+    // Larger problems want the shared K/V loads of the two-sub-tile kernel (6-15 % on the prefill configurations).
+}
+
 // Split-KV launches: keys per range = an equal share of Sk rounded up to whole key tiles.
 inline int splitkv_keys_per_split(int Sk, int n_splits) {
     const long long share = ((long long)Sk + n_splits - 1) / n_splits;

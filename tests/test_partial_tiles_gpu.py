@@ -70,6 +70,27 @@ def test_sides_of_the_kernel_choice(H, Sq, Sk, causal):
     parity.check_full(q, k, v, causal, 0.125, "%s" % ((H, Sq, Sk, causal),))
 
 
+@pytest.mark.parametrize("B,H,Hkv,Sq,Sk,D", [
+    (1, 16, 4, 1408, 1408, 128), (1, 16, 4, 1408, 4001, 128),    # 176 tiles, grouped heads: one, and two sub-tiles
+    (1, 7, 7, 3201, 3300, 64), (1, 7, 7, 3201, 12000, 64),       # 182 tiles
+    (1, 8, 8, 4700, 4700, 128), (1, 8, 8, 4700, 9001, 128),      # 296 tiles, 152 of 256 rows: two, and one sub-tile
+    (3, 32, 16, 168, 3000, 96),
+])
+def test_sides_of_the_kernel_choice_for_prompts_after_cached_keys(B, H, Hkv, Sq, Sk, D):
+    q, k, v = rand_qkv(H + Sk, B, H, Hkv, Sq, Sk, D)
+    scale = 1.0 / math.sqrt(D)
+    o, lse = parity.run_gpu(q, k, v, True, scale)
+    g = torch.Generator().manual_seed(Sk)
+    rows = torch.stack([torch.randint(0, n, (300,), generator=g) for n in (B, H, Sq)], dim=1)
+    rows[:8, 2] = torch.tensor([0, 127, 128, 255, 256, Sq - 129, Sq - 128, Sq - 1]).clamp(0, Sq - 1)
+    parity.check_rows(o, lse, q, k, v, rows.numpy(), True, scale, "%s" % ((B, H, Hkv, Sq, Sk, D),))
+
+
+@pytest.mark.parametrize("lens", [[700, 3, 400], [900, 650, 5, 500]])   # 16 heads: 176 and 320 tiles by the rule's count
+def test_sides_of_the_kernel_choice_for_variable_lengths(lens):
+    _run_and_check(lens, lens, 16, 4, 128, True, 6)
+
+
 @pytest.mark.parametrize("Hkv", [1, 2])   # (1: paired heads in the causal two-sub-tile kernel; 2: 256-row tiles)
 @pytest.mark.parametrize("kernel", [binding.KERNEL_TWO_SUBTILES, binding.KERNEL_ONE_SUBTILE])
 def test_scheduler_passes_over_long_runs_of_empty_tiles(kernel, Hkv):

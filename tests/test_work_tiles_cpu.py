@@ -244,3 +244,24 @@ def test_the_five_configurations_and_the_papers_shape(wt):
     # c5: non-causal, D = 64: every tile visits all 64 key tiles, none masked
     plan, tiles = decode(wt, 8, 16, 16, 8192, 8192, 64, False)
     assert all(t.n0 == t.n1 == 64 == t.n_full0 == t.n_full1 for t in tiles[::97])
+
+
+@pytest.mark.parametrize("B,H,Hkv,Sq,Sk,D,causal,total_q,one", [
+    # what each kernel was measured at: a clear winner on either side of the rule (148 SMs)
+    (1, 8, 8, 1536, 24576, 128, True, 0, True),        # 96 tiles: 342 us with two sub-tiles, 316 with one
+    (1, 8, 8, 3072, 3072, 64, True, 0, True),          # 192 tiles, Sk = Sq: 46.4 / 39.0
+    (1, 16, 16, 1536, 1536, 128, True, 0, True),       # 30.7 / 27.3
+    (1, 8, 8, 3072, 49152, 64, True, 0, False),        # 192 tiles after cached keys: 605 / 669
+    (1, 32, 8, 768, 3072, 128, True, 0, False),        # 51 / 57
+    (1, 16, 16, 2048, 8192, 128, True, 0, False),      # 256 tiles: 126 / 148
+    (3, 32, 16, 168, 6698, 128, True, 0, False),       # 105 / 121
+    (1, 8, 8, 4736, 4736, 128, True, 0, False),        # 296 tiles, Sk = Sq: 80 / 85
+    (1, 8, 8, 4736, 9472, 128, True, 0, True),         # 152 two-sub-tile tiles, a second wave: 209 / 158
+    (1, 8, 8, 3072, 3072, 128, False, 0, False),       # not causal: as after cached keys
+    (1, 128, 128, 300, 300, 64, False, 0, True),       # three key steps
+    (2, 32, 8, 749, 749, 64, True, 0, False),          # 384 tiles
+    (3, 16, 4, 700, 700, 128, True, 1100, True),       # variable lengths: 16 x (8 + 3) tiles
+    (24, 32, 8, 2500, 2500, 128, True, 24000, False),
+])
+def test_kernel_choice(wt, B, H, Hkv, Sq, Sk, D, causal, total_q, one):
+    assert wt.wt_one_subtile_is_faster(B, H, Hkv, Sq, Sk, D, int(causal), total_q, 148) == int(one)

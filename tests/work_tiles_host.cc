@@ -108,4 +108,9 @@ int wt_decode_all(int B, int H, int Hkv, int Sq, int Sk, int D, int causal, int 
     return 0;
 }
 
+// The choice between the two kernels (problems of more than 128 query rows, D <= 128, keys not split).
+int wt_one_subtile_is_faster(int B, int H, int Hkv, int Sq, int Sk, int D, int causal, int total_q, int sms) {
+    return ave::one_subtile_is_faster(B, H, Hkv, Sq, Sk, D, causal != 0, total_q, sms) ? 1 : 0;
+}
+
 }  // extern "C"

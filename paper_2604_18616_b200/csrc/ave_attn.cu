@@ -354,9 +354,8 @@ int launch_attention(const void *q, const void *k, const void *v, void *o, float
     const bool one = D > 128 || use_one_subtile(B, H, Hkv, Sq, Sk, D, causal != 0, split, varlen ? varlen->total_q : 0);
     CUtensorMap tq, tk, tv, to;
     if (!encode_map(&tq, q, D, rows_q, H, n_batch, sq, ave::BM)) return AVE_ERR_CUDA;
-    // (the single-sub-tile kernel stores O without a map; beyond its 128 rows the choice between the kernels may change from
-    // call to call on the same buffers, and the map is kept for either)
-    if ((!one || Sq > ave::BM) && !encode_map(&to, o, D, rows_q, H, n_batch, so, ave::WsCfg<128>::kOutBoxRows)) return AVE_ERR_CUDA;
+    // (the single-sub-tile kernel stores O without a map)
+    if (!one && !encode_map(&to, o, D, rows_q, H, n_batch, so, ave::WsCfg<128>::kOutBoxRows)) return AVE_ERR_CUDA;
     if (!encode_map(&tk, k, D, rows_k, Hkv, n_batch, sk, ave::BN)) return AVE_ERR_CUDA;
     // (head dimensions above 128 take V by halves of the keys)
     if (!encode_map(&tv, v, D, rows_k, Hkv, n_batch, sv, D > 128 ? ave::BN / 2 : ave::BN)) return AVE_ERR_CUDA;

@@ -91,7 +91,17 @@ def test_injected_host_failures_report_cuda_error_and_launch_nothing(what, code)
     parity.compare(o.cpu(), lse.cpu(), o_ref, lse_ref, "after an injected failure")
 
 
-def test_repeated_calls_on_the_same_buffers_encode_no_tensor_maps():
+@pytest.mark.parametrize("kernel,maps_of_o", [(binding.KERNEL_TWO_SUBTILES, 1), (binding.KERNEL_ONE_SUBTILE, 0)])
+def test_repeated_calls_on_the_same_buffers_encode_no_tensor_maps(kernel, maps_of_o):
+    """Each kernel needs a map of Q, K and V; only the two-sub-tile kernel stores O through one."""
+    assert binding.select_kernel(kernel) == binding.AVE_OK
+    try:
+        _repeated_calls(maps_of_o)
+    finally:
+        assert binding.select_kernel(binding.KERNEL_AUTO) == binding.AVE_OK
+
+
+def _repeated_calls(maps_of_o):
     dev = torch.device("cuda:0")
     q, k, v, qd, kd, vd = small_problem(dev, seed=7, Sq=130, Sk=130)
     o = torch.empty_like(qd)
@@ -101,21 +111,20 @@ def test_repeated_calls_on_the_same_buffers_encode_no_tensor_maps():
     for _ in range(5):
         binding.ave_attn_fwd(qd, kd, vd, o, lse, causal=True)
     assert binding.tensor_map_encodes() == n1
-    # another output buffer is another map
+    # another output buffer is another map of it, if there is one
     o2 = torch.empty_like(qd)
     binding.ave_attn_fwd(qd, kd, vd, o2, lse, causal=True)
-    assert binding.tensor_map_encodes() == n1 + 1
+    assert binding.tensor_map_encodes() == n1 + maps_of_o
     torch.cuda.synchronize()
     assert torch.equal(o, o2)
-    # a different shape at the same addresses must not hit the cached entry of q (k and v still hit theirs; with at
-    # most 128 query rows the single-sub-tile kernel runs, which stores O without a tensor map)
+    # a different shape at the same addresses must not hit the cached entries of q and o (k and v still hit theirs)
     B, H, _, D = q.shape
     q64 = qd.view(-1)[:B * H * 64 * D].view(B, H, 64, D)
     o64 = o2.view(-1)[:B * H * 64 * D].view(B, H, 64, D)
     assert q64.data_ptr() == qd.data_ptr() and o64.data_ptr() == o2.data_ptr()
     n2 = binding.tensor_map_encodes()
     binding.ave_attn_fwd(q64, kd, vd, o64, lse.view(-1)[:B * H * 64].view(B, H, 64), causal=True)
-    assert n2 + 1 <= binding.tensor_map_encodes() <= n2 + 2
+    assert binding.tensor_map_encodes() == n2 + 1 + maps_of_o
     o_ref, _ = oracle.attn_fwd(q64.cpu(), k, v, True, 1.0 / math.sqrt(D))
     assert np.abs(o64.cpu().double().numpy() - o_ref).max() <= parity.O_TOL
     st, raw = binding.device_status()

@@ -421,7 +421,7 @@ int launch_attention(const void *q, const void *k, const void *v, void *o, float
 // One or more warps per row (`warps_per_row`, a power of two up to 8), which share out the row's key ranges; a lane
 // holds four neighbouring output columns (at D = 64 the half-warps take ranges in turn).  The bound is latency: a decode step has few rows and up to
 // 64 ranges, and a thread that walks the ranges by itself waits for one load after the other (measured with 32 rows
-// and 37 ranges: 23 us for a thread per 8 columns, 4 us with eight warps per row).
+// and 37 ranges: 23 us for a thread per 8 columns, 4 us with eight warps per row).  Many rows: splitkv_merge_rows_kernel.
 constexpr int kMergeThreads = 256;
 __global__ void __launch_bounds__(kMergeThreads)
 splitkv_merge_kernel(const float *__restrict__ o_partial, const float *__restrict__ lse_partial,
@@ -486,6 +486,43 @@ splitkv_merge_kernel(const float *__restrict__ o_partial, const float *__restric
     if (lane == 0) lse[row] = (denom > 0.f) ? m + logf(denom) : -INFINITY;
 }
 
+// The same with a thread per row and 8 output columns that walks the ranges, for many rows, where the chip is full of loads
+// anyway and a warp that shares out one row spends its time on shuffles and tails (measured, this / warps sharing rows:
+// 524288 rows of 3 ranges, D = 64 98 / 229 us; 131072 rows of 4 ranges, D = 128 57 / 83 us).
+__global__ void __launch_bounds__(kMergeThreads)
+splitkv_merge_rows_kernel(const float *__restrict__ o_partial, const float *__restrict__ lse_partial,
+                          __nv_bfloat16 *__restrict__ o, float *__restrict__ lse, long long rows, int D, int n_splits) {
+    const int chunks = D / 8;
+    const long long idx = (long long)blockIdx.x * kMergeThreads + threadIdx.x;
+    ave::grid_dependency_wait();
+    const long long row = idx / chunks;
+    const int ch = int(idx - row * chunks);
+    if (row >= rows) return;
+    float m = -INFINITY;
+#pragma unroll 4
+    for (int s = 0; s < n_splits; ++s) m = fmaxf(m, lse_partial[s * rows + row]);
+    float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    float denom = 0.f;
+    const int n = m == -INFINITY ? 0 : n_splits;  // (a row that sees no key in any range: what the partials hold is not looked at)
+#pragma unroll 4
+    for (int s = 0; s < n; ++s) {
+        const float w = __expf(lse_partial[s * rows + row] - m);
+        denom += w;
+        const float4 *src = reinterpret_cast<const float4 *>(o_partial + (s * rows + row) * D + ch * 8);
+        const float4 a = src[0], b = src[1];
+        acc[0] += w * a.x; acc[1] += w * a.y; acc[2] += w * a.z; acc[3] += w * a.w;
+        acc[4] += w * b.x; acc[5] += w * b.y; acc[6] += w * b.z; acc[7] += w * b.w;
+    }
+    const float inv = denom > 0.f ? 1.f / denom : 0.f;
+    uint4 out;
+    out.x = ave::pack_bf16x2(acc[0] * inv, acc[1] * inv);
+    out.y = ave::pack_bf16x2(acc[2] * inv, acc[3] * inv);
+    out.z = ave::pack_bf16x2(acc[4] * inv, acc[5] * inv);
+    out.w = ave::pack_bf16x2(acc[6] * inv, acc[7] * inv);
+    reinterpret_cast<uint4 *>(o + row * D)[ch] = out;
+    if (ch == 0) lse[row] = (denom > 0.f) ? m + logf(denom) : -INFINITY;
+}
+
 // One warp waits, with the library's bounded wait, on an mbarrier that nobody ever arrives on: the
 // wait must give up after `limit_cycles`, record its code in the device status word and return.
 __global__ void wait_timeout_selftest_kernel(long long limit_cycles) {
@@ -517,13 +554,24 @@ int run_splitkv(const void *q, const void *k, const void *v, void *o, float *lse
                                            kps, op, lp, 0, nullptr, nullptr, s);
     if (st != AVE_OK || !merge) return st;
     const long long rows = (long long)B * H * Sq;
-    // enough warps to cover the chip a few times over, none with less than two ranges to add up
-    constexpr int kWarps = kMergeThreads / 32;
-    int wpr = 1;
-    while (wpr < kWarps && rows * wpr < 148 * 16 && 4 * wpr <= n_splits) wpr *= 2;
-    const long long ctas = (rows * wpr + kWarps - 1) / kWarps;
-    cudaError_t e = launch_dependent(splitkv_merge_kernel, dim3(unsigned(ctas)), dim3(kMergeThreads), 0, s, o_partial, lse_partial,
-                                     static_cast<__nv_bfloat16 *>(o), lse, rows, D, n_splits, wpr);
+    __nv_bfloat16 *const out = static_cast<__nv_bfloat16 *>(o);
+    cudaError_t e;
+    // The row-wise merge takes some 1.7 us and 0.23 us a range until its loads fill the chip, the other one a time that goes
+    // with rows x ranges (times at splitkv_merge_rows_kernel; at the line, 4096 rows, D = 64: 8 ranges 3.4 / 3.6 us, 16 ranges
+    // 5.5 / 4.6; 8192 rows of 64 ranges 43 / 46; 32 rows of 32 ranges, D = 128 8.9 / 2.9)
+    const long long threads = rows * (D / 8);
+    if (threads >= 65536 || threads >= 3300ll * n_splits) {
+        e = launch_dependent(splitkv_merge_rows_kernel, dim3(unsigned((threads + kMergeThreads - 1) / kMergeThreads)),
+                             dim3(kMergeThreads), 0, s, o_partial, lse_partial, out, lse, rows, D, n_splits);
+    } else {
+        // enough warps to cover the chip a few times over, none with less than two ranges to add up
+        constexpr int kWarps = kMergeThreads / 32;
+        const long long enough = 16ll * sm_count();
+        int wpr = 1;
+        while (wpr < kWarps && rows * wpr < enough && 4 * wpr <= n_splits) wpr *= 2;
+        e = launch_dependent(splitkv_merge_kernel, dim3(unsigned((rows * wpr + kWarps - 1) / kWarps)), dim3(kMergeThreads), 0, s,
+                             o_partial, lse_partial, out, lse, rows, D, n_splits, wpr);
+    }
     if (e != cudaSuccess) {
         t_last_cuda_error = int(e);
         return AVE_ERR_CUDA;

@@ -61,7 +61,7 @@ def test_infinite_value_in_the_last_of_an_odd_number_of_ranges():
     assert torch.isfinite(o[..., rest].float()).all()
 
 
-@pytest.mark.parametrize("H,Hkv,Sq,Sk", [(2, 2, 200, 150), (4, 2, 60, 40)])  # the second: packed query heads
+@pytest.mark.parametrize("H,Hkv,Sq,Sk", [(2, 2, 200, 150), (16, 16, 200, 150), (4, 2, 60, 40)])  # row-wise merge; packed heads
 @pytest.mark.parametrize("D", [64, 128])
 @pytest.mark.parametrize("n_splits", [1, 2])
 def test_rows_without_keys_are_zero_whatever_the_values_are(n_splits, D, H, Hkv, Sq, Sk):

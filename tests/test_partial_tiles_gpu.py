@@ -38,6 +38,9 @@ def test_softmax_warps_without_a_row(D, Sq):
     (1, 3, 1, 1, 1500, 128, 4),      # a last CTA with rows beyond the end
     (2, 4, 2, 100, 500, 128, 1),     # a single range, packed heads on 256-row tiles
     (2, 4, 1, 3, 500, 64, 1),        # a single range, packed heads on 128-row tiles
+    (1, 8, 8, 1000, 2600, 64, 19), (1, 8, 8, 1000, 2600, 64, 20),    # the last number of ranges merged row-wise, and the next
+    (1, 3, 3, 275, 600, 128, 4), (1, 3, 3, 276, 600, 128, 4),        # the same at 13200 threads; a last CTA in part
+    (1, 7, 7, 586, 300, 128, 3), (1, 3, 3, 2731, 300, 64, 3),        # 8 columns for each of more than 65536 threads
 ])
 def test_split_merge_shapes(B, H, Hkv, Sq, Sk, D, n_splits):
     q, k, v = rand_qkv(H + Sk, B, H, Hkv, Sq, Sk, D)

@@ -416,6 +416,10 @@ int launch_attention(const void *q, const void *k, const void *v, void *o, float
     return causal ? launch_ws<64, true, false>(tq, tk, tv, to, p, s) : launch_ws<64, false, false>(tq, tk, tv, to, p, s);
 }
 
+__device__ __forceinline__ bool status_word_is_set() {
+    return *reinterpret_cast<volatile unsigned int *>(&ave::g_device_status) != 0;
+}
+
 // Combine the partial results of the key ranges of every query row:
 //   LSE = ln sum_s exp(LSE_s),  O = sum_s exp(LSE_s - LSE) * O_s.
 // One or more warps per row (`warps_per_row`, a power of two up to 8), which share out the row's key ranges; a lane
@@ -433,6 +437,7 @@ splitkv_merge_kernel(const float *__restrict__ o_partial, const float *__restric
     const long long row = (long long)blockIdx.x * (kMergeThreads / 32 / warps_per_row) + warp / warps_per_row;
     const bool live = row < rows;
     ave::grid_dependency_wait();
+    const bool skip = status_word_is_set();  // (the partials were not written)
     const int lanes_per_range = D / 4, ranges_at_once = 32 / lanes_per_range;  // 32 and 1, or 16 and 2
     const int col4 = lane & (lanes_per_range - 1);
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -475,7 +480,7 @@ splitkv_merge_kernel(const float *__restrict__ o_partial, const float *__restric
             acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
         }
     }
-    if (!live) return;
+    if (!live || skip) return;
     const float inv = denom > 0.f ? 1.f / denom : 0.f;
     if (lane < lanes_per_range) {
         uint2 out;
@@ -495,6 +500,7 @@ splitkv_merge_rows_kernel(const float *__restrict__ o_partial, const float *__re
     const int chunks = D / 8;
     const long long idx = (long long)blockIdx.x * kMergeThreads + threadIdx.x;
     ave::grid_dependency_wait();
+    const bool skip = status_word_is_set();
     const long long row = idx / chunks;
     const int ch = int(idx - row * chunks);
     if (row >= rows) return;
@@ -513,6 +519,7 @@ splitkv_merge_rows_kernel(const float *__restrict__ o_partial, const float *__re
         acc[0] += w * a.x; acc[1] += w * a.y; acc[2] += w * a.z; acc[3] += w * a.w;
         acc[4] += w * b.x; acc[5] += w * b.y; acc[6] += w * b.z; acc[7] += w * b.w;
     }
+    if (skip) return;
     const float inv = denom > 0.f ? 1.f / denom : 0.f;
     uint4 out;
     out.x = ave::pack_bf16x2(acc[0] * inv, acc[1] * inv);

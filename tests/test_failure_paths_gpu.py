@@ -63,6 +63,24 @@ def test_a_wait_that_runs_out_sets_the_status_word_and_later_kernels_skip():
     parity.compare(o.cpu(), lse.cpu(), o_ref, lse_ref, "after the status word was cleared")
 
 
+@pytest.mark.parametrize("B,Sq,n_splits", [(1, 1, 6), (4, 200, 2)])   # ranges merged by several warps per row, and row-wise
+def test_splitkv_writes_nothing_while_the_status_word_is_set(B, Sq, n_splits):
+    dev = torch.device("cuda:0")
+    q, k, v, qd, kd, vd = small_problem(dev, seed=9, B=B, Sq=Sq, Sk=900)
+    o = torch.full_like(qd, 3.0)
+    lse = torch.full(q.shape[:3], 3.0, dtype=torch.float32, device=dev)
+    assert binding.device_status() == (binding.AVE_OK, 0)
+    assert binding.selftest_wait_timeout(16) == binding.AVE_OK
+    binding.ave_attn_fwd_splitkv(qd, kd, vd, n_splits, o=o, lse=lse)
+    torch.cuda.synchronize()
+    assert torch.all(o == 3.0) and torch.all(lse == 3.0)
+    assert binding.device_status() == (binding.AVE_ERR_DEVICE_TIMEOUT, binding.STATUS_BIT_SELFTEST)
+    binding.ave_attn_fwd_splitkv(qd, kd, vd, n_splits, o=o, lse=lse)
+    assert binding.device_status() == (binding.AVE_OK, 0)
+    o_ref, lse_ref = oracle.attn_fwd(q, k, v, False, 1.0 / math.sqrt(q.shape[-1]))
+    parity.compare(o.cpu(), lse.cpu(), o_ref, lse_ref, "after the status word was cleared")
+
+
 @pytest.mark.parametrize("what,code", [(binding.INJECT_ENCODE_FAILURE, 1),      # CUDA_ERROR_INVALID_VALUE
                                        (binding.INJECT_LAUNCH_FAILURE, 719)])   # cudaErrorLaunchFailure
 def test_injected_host_failures_report_cuda_error_and_launch_nothing(what, code):

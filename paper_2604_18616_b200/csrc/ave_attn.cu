@@ -17,6 +17,7 @@
 #include "attn_fwd_ws.cuh"
 #include "attn_fwd_1t.cuh"
 #include "gemm_bf16.cuh"
+#include "gemm_choice.cuh"
 #include "moe_fp8.cuh"
 
 // Scratch of ave_attn_fwd_splitkv_static: part of the device image, so every GPU that loads the
@@ -626,6 +627,52 @@ int launch_gemm_tile(const void *a, const void *b, void *c, int M, int N, int K,
     return AVE_OK;
 }
 
+// The same in 128 x 256 tiles of one CTA each.
+template <bool B_NMAJOR>
+int launch_gemm_wide(const void *a, const void *b, void *c, int M, int N, int K, int sms, cudaStream_t s) {
+    using Cfg = ave::GemmWideCfg;
+    CUtensorMap ta, tb, tc;
+    const Strides sa{(long long)M * K, (long long)M * K, (long long)K};
+    const Strides sb{(long long)N * K, (long long)N * K, (long long)(B_NMAJOR ? N : K)};
+    const Strides sc{(long long)M * N, (long long)M * N, (long long)N};
+    if (!encode_map(&ta, a, K, M, 1, 1, sa, Cfg::kTileM)) return AVE_ERR_CUDA;
+    if (B_NMAJOR) {  // B [K, N]: rows of N elements, boxes of 64 columns x 64 rows of K
+        if (!encode_map(&tb, b, N, K, 1, 1, sb, Cfg::kSliceK)) return AVE_ERR_CUDA;
+    } else {         // B [N, K]: rows of K elements, boxes of 64 columns of K x the tile's columns
+        if (!encode_map(&tb, b, K, N, 1, 1, sb, Cfg::kTileN)) return AVE_ERR_CUDA;
+    }
+    if (!encode_map(&tc, c, N, M, 1, 1, sc, Cfg::kOutBoxRows)) return AVE_ERR_CUDA;
+    ave::GemmParams p{};
+    p.M = M;
+    p.N = N;
+    p.K = K;
+    p.tiles_m = (M + Cfg::kTileM - 1) / Cfg::kTileM;
+    p.tiles_n = (N + Cfg::kTileN - 1) / Cfg::kTileN;
+    p.group_m = 16;  // the ~148 tiles in flight cover 16 x 9.25 tiles, a near-square part of C
+    auto kern = ave::gemm_bf16_wide_kernel<B_NMAJOR>;
+    static PerDeviceOnce once;  // per instantiation
+    const int st = prepare_kernel(kern, Cfg::kSmemBytes, 0, once);
+    if (st != AVE_OK) return st;
+    const long long n_tiles = (long long)p.tiles_m * p.tiles_n;
+    const dim3 grid(unsigned(n_tiles < sms ? n_tiles : sms));
+    cudaError_t e;
+    if (M <= 16 && K > 1024 && n_tiles > sms / 2 && n_tiles < sms) {
+        // The early launch is slower here, and only here (75 to 147 CTAs, at most 16 rows, K of 2048 and 4096: 5 % on average, up
+        // to 27 %; elsewhere it is 5-25 % faster): presumably because it puts the CTAs wherever the kernel before has left
+        // room, some side by side on a pair of SMs and on others none, in a kernel that is bound by fetching B.
+        kern<<<grid, dim3(Cfg::kThreads), Cfg::kSmemBytes, s>>>(ta, tb, tc, p);
+        e = cudaGetLastError();
+    } else {
+        e = launch_dependent(kern, grid, dim3(Cfg::kThreads), Cfg::kSmemBytes, s, ta, tb, tc, p);
+    }
+    if (e != cudaSuccess) {
+        t_last_cuda_error = int(e);
+        return AVE_ERR_CUDA;
+    }
+    g_launches.fetch_add(1, std::memory_order_relaxed);
+    return AVE_OK;
+}
+
 // The same on CTA pairs, with tiles of 256 x tile_n.
 template <bool B_NMAJOR>
 int launch_gemm_pair(const void *a, const void *b, void *c, int M, int N, int K, int tile_n, int sms, cudaStream_t s) {
@@ -673,36 +720,10 @@ int launch_gemm(const void *a, const void *b, void *c, int M, int N, int K, cuda
         t_last_cuda_error = int(e);
         return AVE_ERR_CUDA;
     }
-    // The time of a tile goes with the bytes its slices bring into an SM, in units of 64 elements x 128 rows (16 KB, about
-    // 270 clk); whole tiles are dealt out, so it also goes with the number of waves.
-    // CTA pairs move the fewest bytes per product (n = 4096: 96 us, against 105 us for 128 x 256 tiles of one CTA;
-    // 8192 x 8192 x 4096: 351 / 425 us); a tile width that just fills the last wave saves up to a third of it
-    // (420 x 6544 x 3840: 24.4 us 256 wide, 19.5 us 192 wide).
-    const long long slices = (K + 63) / 64;
-    const double kUnit = 270., kTile = 4000.;  // clk: 16 KB; filling the ring, and the epilogue that nothing overlaps
-    const long long pairs = sms / 2, rows = (M + 255) / 256;
-    int tile_n = 256;
-    double best = 0.;
-    for (int w = 256; w >= 64; w -= 64) {
-        const long long waves = (rows * ((N + w - 1) / w) + pairs - 1) / pairs;
-        const int loaded = B_NMAJOR ? (w + 127) / 128 * 128 : w;  // N-contiguous B comes in 64 columns per CTA at a time
-        const double cost = waves * slices * kUnit * (1. + loaded / 256.) + kTile;
-        if (w == 256 || cost < best) best = cost, tile_n = w;
-    }
-    // Few tiles: 128 x 128 tiles of one CTA each, or of a cluster that shares out K, which costs an exchange of the sums.
-    const long long tiles = (long long)((M + 127) / 128) * ((N + 127) / 128);
-    int splits = 0;
-    for (int x = 1; x <= ave::GemmCfg::kMaxSplits; x *= 2) {
-        // (a cluster sits inside a GPC, so that not all SMs can be used by large ones: sixteen clusters of eight, or 35 of four,
-        // were not resident at once, and a second wave costs more than sharing K gains)
-        const long long resident = x == 8 ? 2 * sms / 3 : x == 4 ? 7 * sms / 8 : sms;
-        if (x > 1 && (x * 4 > slices || x * tiles > resident)) break;
-        const long long waves = (tiles * x + sms - 1) / sms;
-        const double cost = waves * ((slices + x - 1) / x * kUnit * 2. + kTile) + (x > 1 ? 2500. : 0.);
-        if (cost < best) best = cost, splits = x;
-    }
-    if (splits > 0) return launch_gemm_tile<B_NMAJOR>(a, b, c, M, N, K, splits, s);
-    return launch_gemm_pair<B_NMAJOR>(a, b, c, M, N, K, tile_n, sms, s);
+    const ave::GemmChoice g = ave::choose_gemm(B_NMAJOR, M, N, K, sms);
+    if (g.splits > 0) return launch_gemm_tile<B_NMAJOR>(a, b, c, M, N, K, g.splits, s);
+    if (g.tile_n > 0) return launch_gemm_pair<B_NMAJOR>(a, b, c, M, N, K, g.tile_n, sms, s);
+    return launch_gemm_wide<B_NMAJOR>(a, b, c, M, N, K, sms, s);
 }
 
 // E4M3 codes [d2, rows, inner] (inner contiguous) as a 4-D map with boxes of 128 bytes x box_rows rows, 128-byte

@@ -2,10 +2,11 @@
 // fp32 accumulation in TMEM, bf16 result.  (The paper's first evaluated kernel family, Section 9:
 // square bf16 matrices with normally distributed entries.)
 //
-// Two kernels.  Large products: CTA pairs with tiles of 256 x up to 256 (below).  Products of few tiles: one CTA, or a
-// cluster that shares K, per 128 x 128 tile.  In both the K dimension is streamed in slices of 64
+// Three kernels.  Large products: CTA pairs with tiles of 256 x up to 256 (below).  Products of few tiles: one CTA, or a
+// cluster that shares K, per 128 x 128 tile.  In between, above all with at most 128 rows, of which a pair would use half:
+// one CTA per 128 x 256 tile.  In all of them the K dimension is streamed in slices of 64
 // through a ring of shared-memory stages filled by TMA, and one thread issues the
-// tcgen05 MMAs into TMEM; the pairs are persistent and have two accumulators, so that the
+// tcgen05 MMAs into TMEM; pairs and 128 x 256 tiles are persistent and have two accumulators, so that the
 // epilogue of a tile (TMEM -> registers -> bf16 -> shared -> TMA store)
 // overlaps the main loop of the next one.
 //
@@ -22,6 +23,7 @@
 #include <cuda_bf16.h>
 
 #include "attn_common.cuh"
+#include "gemm_choice.cuh"
 
 namespace ave {
 
@@ -33,7 +35,7 @@ struct GemmCfg {
     static constexpr int kBBytes = kTileN * kSliceK * 2;          // 16 KB
     static constexpr int kStageBytes = kABytes + kBBytes;
     static constexpr int kOutBoxRows = 32;                        // each epilogue warp stores its own 32 rows
-    static constexpr int kMaxSplits = 8;                          // CTAs of a cluster that share a tile's K
+    static constexpr int kMaxSplits = kGemmMaxSplits;             // CTAs of a cluster that share a tile's K
     static constexpr int kRecvBytes = kTileM * kTileN * 4 / kMaxSplits * (kMaxSplits - 1);  // the others' partial sums
     static constexpr int kSmemBytes = kStages * kStageBytes + kRecvBytes + 1024;
     static constexpr uint32_t kTmemCols = kTileN;
@@ -43,7 +45,7 @@ struct GemmParams {
     int M, N, K;
     int tiles_m, tiles_n;  // output tiles along M and N
     int group_m;           // tiles along M walked together before moving along N (L2 reuse of the B tiles)
-    int tile_n;            // (CTA pairs) columns of a tile: a multiple of 64
+    int tile_n;            // (CTA pairs) columns of a tile: 128, 192 or 256
     int splits;            // (one CTA per tile and share of K) CTAs of a cluster
     void *c;               // the result, for stores that do not go through its tensor map
 };
@@ -60,6 +62,21 @@ __device__ __forceinline__ void gemm_tile_coords(int id, const GemmParams &p, in
     bm = m0 + (rem - bn * gm);
 }
 
+// 64 columns of 32 accumulator rows (one per lane) as bf16 into a staging buffer of 32 rows x 128 bytes, in the
+// 128-byte-swizzled layout that the TMA store expects.
+__device__ __forceinline__ void gemm_stage_64_columns(uint32_t buf, int lane, const uint32_t (&v)[2][32]) {
+#pragma unroll
+    for (int e = 0; e < 64; e += 8) {
+        const uint32_t *src = &v[e >> 5][e & 31];
+        const uint32_t addr = buf + lane * 128 + (((e >> 3) ^ (lane & 7)) << 4);
+        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr),
+                     "r"(pack_bf16x2(__uint_as_float(src[0]), __uint_as_float(src[1]))),
+                     "r"(pack_bf16x2(__uint_as_float(src[2]), __uint_as_float(src[3]))),
+                     "r"(pack_bf16x2(__uint_as_float(src[4]), __uint_as_float(src[5]))),
+                     "r"(pack_bf16x2(__uint_as_float(src[6]), __uint_as_float(src[7]))) : "memory");
+    }
+}
+
 // B_NMAJOR = false: B is [N, K] with K contiguous (C = A * B^T).  B_NMAJOR = true: B is [K, N] with N
 // contiguous (C = A * B); its slice then lands in shared memory as 64-column boxes of 64 K-rows each and is
 // read through an MN-major descriptor, so neither form needs a transposition.
@@ -67,7 +84,7 @@ __device__ __forceinline__ void gemm_tile_coords(int id, const GemmParams &p, in
 // A cluster of S = 1, 2, 4 or 8 CTAs computes one tile, each over its share of K; with S > 1 every CTA then sends the others
 // their 128 / S columns of its fp32 sums through distributed shared memory and adds up, in the order of the shares, and
 // stores its own columns.  A product of few tiles leaves most SMs idle, and a tile's time is its number of slices times the
-// 32 KB a slice brings in (about 60 B/clk).  200 x 512 x 8192 (8 tiles): 37.8 us with S = 1, 10.5 us with S = 8;
+// 32 KB a slice brings in.  200 x 512 x 8192 (8 tiles): 37.8 us with S = 1, 10.5 us with S = 8;
 // 128 x 4096 x 4096 (32 tiles): 21.4 / 10.5 us with S = 4; 1939 x 440 x 2416 (64 tiles): 16.1 / 12.1 us with S = 2.
 template <bool B_NMAJOR>
 __global__ void __launch_bounds__(256, 1)
@@ -210,17 +227,7 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
                 tmem_pin_x32(v[0]);
                 tmem_pin_x32(v[1]);
                 const uint32_t buf = sC + c * (Cfg::kOutBoxRows * 128);
-#pragma unroll
-                for (int e = 0; e < 64; e += 8) {
-                    const uint32_t *src = &v[e >> 5][e & 31];
-                    // 16-byte chunk of row `lane`, in the 128-byte-swizzled layout TMA expects
-                    const uint32_t addr = buf + lane * 128 + (((e >> 3) ^ (lane & 7)) << 4);
-                    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr),
-                                 "r"(pack_bf16x2(__uint_as_float(src[0]), __uint_as_float(src[1]))),
-                                 "r"(pack_bf16x2(__uint_as_float(src[2]), __uint_as_float(src[3]))),
-                                 "r"(pack_bf16x2(__uint_as_float(src[4]), __uint_as_float(src[5]))),
-                                 "r"(pack_bf16x2(__uint_as_float(src[6]), __uint_as_float(src[7]))) : "memory");
-                }
+                gemm_stage_64_columns(buf, lane, v);
                 fence_proxy_async_smem();
                 __syncwarp();
                 const int col0 = bn * Cfg::kTileN + c * 64;
@@ -287,6 +294,201 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
                 }
             }
         }
+    }
+
+    // ---- common exit: every thread arrives, then TMEM is released
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 2) tmem_dealloc(tmem, Cfg::kTmemCols);
+}
+
+// ------------------------------------------------------------------ 128 x 256 tiles, one CTA each
+//
+// What bounds it is the way from L2 into shared memory, 48 KB per slice against 512 clk of MMAs (see the CTA pairs); its
+// place is where pairs would multiply rows that do not exist, or leave a last wave nearly empty (pairs / this kernel:
+// 128 x 19000 x 2048 28.0 / 21.2 us, 128 x 28672 x 4096 60 / 48 us, 1 x 65536 x 512 25.9 / 17.1 us,
+// 600 x 14336 x 4096 67.8 / 60.5 us).
+struct GemmWideCfg {
+    static constexpr int kThreads = 256;
+    static constexpr int kTileM = 128, kTileN = 256, kSliceK = 64;
+    static constexpr int kStages = 4;
+    static constexpr int kABytes = kTileM * kSliceK * 2;          // 16 KB
+    static constexpr int kBBytes = kTileN * kSliceK * 2;          // 32 KB
+    static constexpr int kStageBytes = kABytes + kBBytes;
+    static constexpr int kOutBoxRows = 32;
+    static constexpr int kStageCBytes = 4 * kOutBoxRows * 128;    // 32 rows x 64 columns per epilogue warp
+    static constexpr int kSmemBytes = kStages * kStageBytes + kStageCBytes + 1024;
+    static constexpr uint32_t kTmemCols = 2 * kTileN;             // two accumulators
+};
+
+template <bool B_NMAJOR>
+__global__ void __launch_bounds__(256, 1)
+gemm_bf16_wide_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b,
+                      const __grid_constant__ CUtensorMap tm_c, const GemmParams p) {
+    using Cfg = GemmWideCfg;
+    constexpr int NS = Cfg::kStages;
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ __align__(8) uint64_t bar_full[NS], bar_empty[NS], bar_acc_full[2], bar_acc_empty[2], bar_drain;
+    __shared__ uint32_t tmem_base_slot;
+    __shared__ int abort_flag;
+
+    const int tid = threadIdx.x;
+    const int warp = tid >> 5;
+    const int lane = tid & 31;
+    const uint32_t sRing = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    const uint32_t sStage = sRing + NS * Cfg::kStageBytes;
+
+    if (tid == 0) {
+        for (int s = 0; s < NS; ++s) {
+            mbar_init(smem_u32(&bar_full[s]), 1);
+            mbar_init(smem_u32(&bar_empty[s]), 1);
+        }
+        for (int a = 0; a < 2; ++a) {
+            mbar_init(smem_u32(&bar_acc_full[a]), 1);
+            mbar_init(smem_u32(&bar_acc_empty[a]), 4);  // one arrival per epilogue warp
+        }
+        mbar_init(smem_u32(&bar_drain), 1);
+        fence_mbar_init();
+        tma_prefetch_desc(&tm_a);
+        tma_prefetch_desc(&tm_b);
+    }
+    if (warp == 2) {
+        tmem_alloc(smem_u32(&tmem_base_slot), Cfg::kTmemCols);
+        tmem_relinquish();
+    }
+    // what precedes overlaps the end of the kernel before this one in the stream
+    grid_dependency_wait();
+    grid_dependency_launch();
+    if (tid == 0) abort_flag = (*reinterpret_cast<volatile unsigned int *>(&g_device_status) != 0) ? 1 : 0;
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = tmem_base_slot;
+    const bool poisoned = abort_flag != 0;
+
+    const int n_tiles = p.tiles_m * p.tiles_n;
+    const int n_slices = (p.K + Cfg::kSliceK - 1) / Cfg::kSliceK;
+
+    if (poisoned) {
+        // nothing: fall through to the common exit
+    } else if (warp == 0) {
+        // =============================== producer ===============================
+        if (elect_one()) {
+            bool ok = true;
+            int ring = 0;  // slices loaded so far
+            for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
+                int bm, bn;
+                gemm_tile_coords(tile, p, bm, bn);
+                for (int ks = 0; ks < n_slices; ++ks, ++ring) {
+                    const int slot = ring % NS, round = ring / NS;
+                    if (round > 0) ok = mbar_wait_bounded(smem_u32(&bar_empty[slot]), (round - 1) & 1, &abort_flag, STATUS_TIMEOUT_SLOT);
+                    if (!ok) break;
+                    const uint32_t bar = smem_u32(&bar_full[slot]);
+                    const uint32_t dst = sRing + slot * Cfg::kStageBytes;
+                    mbar_arrive_expect_tx(bar, Cfg::kStageBytes);
+                    tma_load_4d(dst, &tm_a, bar, ks * Cfg::kSliceK, bm * Cfg::kTileM, 0, 0);
+                    if (!B_NMAJOR) {
+                        tma_load_4d(dst + Cfg::kABytes, &tm_b, bar, ks * Cfg::kSliceK, bn * Cfg::kTileN, 0, 0);
+                    } else {
+                        for (int x = 0; x < Cfg::kTileN / 64; ++x)  // boxes of 64 columns of B x 64 rows of K
+                            tma_load_4d(dst + Cfg::kABytes + x * (Cfg::kSliceK * 128), &tm_b, bar, bn * Cfg::kTileN + x * 64,
+                                        ks * Cfg::kSliceK, 0, 0);
+                    }
+                }
+            }
+            if (!ok) {
+                // abandoned: give the loads still in flight a bounded chance to land
+                for (int it = max(0, ring - NS); it < ring; ++it)
+                    for (uint32_t w = 0; w < WAIT_LIMIT && !mbar_test_wait(smem_u32(&bar_full[it % NS]), (it / NS) & 1); ++w) {}
+            }
+        }
+        __syncwarp();
+    } else if (warp == 1) {
+        // =============================== MMA issuer ===============================
+        if (elect_one()) {
+            constexpr uint32_t idesc = make_idesc_bf16(Cfg::kTileM, Cfg::kTileN, B_NMAJOR ? 1 : 0);
+            constexpr uint64_t desc_kmajor = make_sdesc_sw128(16, 1024);
+            constexpr uint32_t hi = uint32_t(desc_kmajor >> 32), lo = uint32_t(desc_kmajor);
+            constexpr uint64_t desc_nmajor = make_sdesc_sw128(Cfg::kSliceK * 128, 1024);
+            constexpr uint32_t hi_b = B_NMAJOR ? uint32_t(desc_nmajor >> 32) : hi;
+            constexpr uint32_t lo_b = B_NMAJOR ? uint32_t(desc_nmajor) : lo;
+            constexpr uint32_t b_kstep = B_NMAJOR ? ((16 * 128) >> 4) : (32 >> 4);
+            bool ok = true;
+            int ring = 0;
+            int n_done = 0;  // tiles issued so far
+            for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x, ++n_done) {
+                const int acc = n_done & 1;
+                if (n_done >= 2) {  // the epilogue must have read this accumulator's previous tile out of TMEM
+                    ok = mbar_wait_bounded(smem_u32(&bar_acc_empty[acc]), ((n_done >> 1) - 1) & 1, &abort_flag, STATUS_TIMEOUT_SOFTMAX);
+                    if (!ok) break;
+                    tc_fence_after();
+                }
+                const uint32_t d_tmem = tmem + acc * Cfg::kTileN;
+                for (int ks = 0; ks < n_slices; ++ks, ++ring) {
+                    const int slot = ring % NS;
+                    ok = mbar_wait_bounded(smem_u32(&bar_full[slot]), (ring / NS) & 1, &abort_flag, STATUS_TIMEOUT_LOAD);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint32_t a_lo = lo | ((sRing + slot * Cfg::kStageBytes) >> 4);
+                    const uint32_t b_lo = lo_b | ((sRing + slot * Cfg::kStageBytes + Cfg::kABytes) >> 4);
+#pragma unroll
+                    for (int kk = 0; kk < Cfg::kSliceK / 16; ++kk)
+                        umma_ss_words(d_tmem, a_lo + ((kk * 32) >> 4), hi, b_lo + kk * b_kstep, hi_b, idesc, (ks > 0 || kk > 0));
+                    umma_commit(smem_u32(&bar_empty[slot]));
+                    if (ks == n_slices - 1) umma_commit(smem_u32(&bar_acc_full[acc]));
+                }
+            }
+            if (!ok) {  // abandoned: let the MMAs already issued finish before TMEM is released
+                umma_commit(smem_u32(&bar_drain));
+                for (uint32_t w = 0; w < WAIT_LIMIT && !mbar_test_wait(smem_u32(&bar_drain), 0); ++w) {}
+            }
+        }
+        __syncwarp();
+    } else if (warp >= 4) {
+        // =============================== epilogue ===============================
+        const int wq = warp & 3;  // TMEM lane quadrant of this warp
+        const uint32_t lane_sel = uint32_t(wq * 32) << 16;
+        const uint32_t sC = sStage + wq * (Cfg::kOutBoxRows * 128);  // this warp's 32 staging rows
+        bool ok = true;
+        bool store_pending = false;  // (lane 0) a TMA store may still be reading this warp's staging rows
+        int n_done = 0;
+        for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x, ++n_done) {
+            int bm, bn;
+            gemm_tile_coords(tile, p, bm, bn);
+            const int acc = n_done & 1;
+            ok = __all_sync(0xffffffffu, mbar_wait_bounded(smem_u32(&bar_acc_full[acc]), (n_done >> 1) & 1, &abort_flag, STATUS_TIMEOUT_MMA));
+            if (!ok) break;
+            tc_fence_after();
+            const uint32_t t_acc = tmem + acc * Cfg::kTileN + lane_sel;
+            const int row0 = bm * Cfg::kTileM + wq * 32;
+#pragma unroll 1
+            for (int c = 0; c < Cfg::kTileN / 64; ++c) {  // 64 columns at a time
+                uint32_t v[2][32];
+                tmem_ld_x32(t_acc + c * 64, v[0]);
+                tmem_ld_x32(t_acc + c * 64 + 32, v[1]);
+                tmem_wait_ld();
+                tmem_pin_x32(v[0]);
+                tmem_pin_x32(v[1]);
+                if (c == Cfg::kTileN / 64 - 1) {  // the accumulator is in registers: the MMAs may reuse it
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(smem_u32(&bar_acc_empty[acc]));
+                }
+                // this warp's previous TMA store must have finished reading the staging rows
+                if (lane == 0 && store_pending) tma_store_wait_read();
+                __syncwarp();
+                gemm_stage_64_columns(sC, lane, v);
+                fence_proxy_async_smem();
+                __syncwarp();
+                const int col0 = bn * Cfg::kTileN + c * 64;
+                if (lane == 0 && row0 < p.M && col0 < p.N) {
+                    tma_store_4d(&tm_c, sC, col0, row0, 0, 0);
+                    tma_store_commit();
+                    store_pending = true;
+                }
+            }
+        }
+        if (lane == 0 && store_pending) tma_store_wait_all();
     }
 
     // ---- common exit: every thread arrives, then TMEM is released
@@ -484,17 +686,7 @@ gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_con
                 // this warp's previous TMA store must have finished reading the staging rows
                 if (lane == 0 && store_pending) tma_store_wait_read();
                 __syncwarp();
-#pragma unroll
-                for (int e = 0; e < 64; e += 8) {
-                    const uint32_t *src = &v[e >> 5][e & 31];
-                    // 16-byte chunk of row `lane`, in the 128-byte-swizzled layout TMA expects
-                    const uint32_t addr = sC + lane * 128 + (((e >> 3) ^ (lane & 7)) << 4);
-                    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr),
-                                 "r"(pack_bf16x2(__uint_as_float(src[0]), __uint_as_float(src[1]))),
-                                 "r"(pack_bf16x2(__uint_as_float(src[2]), __uint_as_float(src[3]))),
-                                 "r"(pack_bf16x2(__uint_as_float(src[4]), __uint_as_float(src[5]))),
-                                 "r"(pack_bf16x2(__uint_as_float(src[6]), __uint_as_float(src[7]))) : "memory");
-                }
+                gemm_stage_64_columns(sC, lane, v);
                 fence_proxy_async_smem();
                 __syncwarp();
                 const int col0 = bn * p.tile_n + c * 64;

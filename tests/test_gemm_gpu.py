@@ -39,9 +39,15 @@ def run_gemm(a, b, guard=64):
     (127, 264, 72),        # ragged in every dimension
     (300, 1000, 200),      # ragged, several tiles
     (129, 8, 4104),        # long reduction with a ragged last slice
-    (2048, 2048, 2048),    # more tiles than SMs: CTAs walk several tiles, both accumulators in use
-    (2100, 2312, 264),     # the 128 x 256 tile kernel (170 tiles) with ragged edges in every dimension
-    (1024, 1024, 1024),    # the 128 x 128 tile kernel, 64 tiles
+    (2048, 2048, 2048),    # CTA pairs, one 256 x 256 tile each
+    (2100, 2312, 264),     # CTA pairs, 256 x 192 tiles, two for some pairs, ragged edges in every dimension
+    (1024, 1024, 1024),    # 128 x 128 tiles of one CTA each
+    # several tiles per CTA or pair and few slices each, so that accumulators are handed back and forth all the time:
+    (4200, 5000, 72),      # pairs, 340 tiles of 256 x 256: up to five each
+    (4213, 5000, 264),
+    (100, 90000, 72),      # 128 x 256 tiles of one CTA, 352 of them: up to three each
+    (300, 19000, 136),     # the same with several rows of tiles: 225, up to two each
+    (3, 20000, 1096),      # 79 such tiles, a launch that does not overlap the kernel before it
 ])
 def test_gemm_matches_oracle(M, N, K):
     a, b = inputs.make_gemm_inputs(M, N, K, seed=100 + M + N + K)
@@ -81,8 +87,10 @@ def run_gemm_nn(a, b_kn, guard=64):
 
 @pytest.mark.parametrize("M,N,K", [
     (128, 256, 64), (128, 128, 512), (1, 8, 8), (127, 264, 72), (300, 1000, 200), (129, 8, 4104),
-    (1024, 1024, 1024),    # 128 x 128 tiles
-    (2100, 2312, 264),     # 128 x 256 tiles, ragged
+    (1024, 1024, 1024),    # 128 x 128 tiles of one CTA each
+    (2100, 2312, 264),     # CTA pairs, 256 x 128 tiles, up to three each, ragged
+    (4200, 5000, 72), (4213, 5000, 264),         # pairs, 340 tiles of 256 x 256: up to five each
+    (100, 90000, 72), (300, 19000, 136),         # 128 x 256 tiles of one CTA, up to three each
 ])
 def test_gemm_nn_matches_oracle(M, N, K):
     """C = A . B with B stored [K, N]: the oracle's definition on the transposed copy of B."""

@@ -502,6 +502,8 @@ __global__ void moe_clear_kernel(int *counts, int E) {
 // Pairs per expert: a histogram per CTA in shared memory, added to the global one.
 __global__ void moe_count_kernel(const int *__restrict__ ids, int n_pairs, int E, int *counts) {
     extern __shared__ int hist[];  // E
+    grid_dependency_wait();
+    grid_dependency_launch();
     for (int e = threadIdx.x; e < E; e += blockDim.x) hist[e] = 0;
     __syncthreads();
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_pairs; i += gridDim.x * blockDim.x) {
@@ -509,8 +511,6 @@ __global__ void moe_count_kernel(const int *__restrict__ ids, int n_pairs, int E
         if (e >= 0 && e < E) atomicAdd(&hist[e], 1);
     }
     __syncthreads();
-    grid_dependency_wait();
-    grid_dependency_launch();
     for (int e = threadIdx.x; e < E; e += blockDim.x)
         if (hist[e]) atomicAdd(&counts[e], hist[e]);
 }

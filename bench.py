@@ -14,9 +14,12 @@ workload; the default is the largest single-GPU prefill configuration.  Rank 0 p
 * ``cpu_baseline``: the fp64 oracle timed on the host cores on a bounded row sample of the same workload; the GPU
   result of a NaN-poisoned launch (outside the timed region) is compared with those oracle rows, so the line
   carries the parity errors of the very process that produced the number;
-* ``per_workload`` (1 GPU only): one record per further workload (the five configurations, the paper's own shape
-  at its five lengths, split-KV decode shapes, square matrix products), each timed the same way with K launches
-  and checked against oracle rows the same way.
+* ``parity_all_ok`` (1 GPU only): whether the results of every further workload matched the oracle.
+
+The further workloads (the five configurations, the paper's own shape at its five lengths, split-KV decode shapes, square
+matrix products, the expert layer) are timed the same way with K launches and checked against oracle rows the same way; their
+records, ``{"per_workload": {...}}``, go to stderr one by one, so that the line stays short enough for a reader that
+keeps a few kilobytes of the output.
 
 ``--workload gemm_n<size>`` / ``decode_*`` make a matrix product / a split-KV decode shape the headline (used for
 profiler captures of those kernels).  With ``--gpus N`` and no torchrun environment the script starts the N ranks
@@ -727,6 +730,15 @@ def run_leg(ctx, name, steps, warmup, headline=False):
     return attention_leg(ctx, w, steps, warmup, headline)
 
 
+def emit(line, per):
+    """The result: one JSON line on stdout, short enough for a reader that keeps a few kilobytes of a run's output; the
+    per-workload records one by one on stderr, before it."""
+    for r in per:
+        print(json.dumps({"per_workload": r}), file=sys.stderr)
+    sys.stderr.flush()
+    print(json.dumps(line), flush=True)
+
+
 def run_ours(args):
     ctx = Ctx(args)
     ctx.init_gpu()
@@ -798,9 +810,8 @@ def run_ours(args):
             except KeyError:
                 per.append({"workload": name, "error": "unknown workload"})
         if per:
-            line["per_workload"] = per
             line["parity_all_ok"] = all(r.get("parity", {}).get("ok", False) for r in per if "error" not in r) if want_oracle else None
-        print(json.dumps(line))
+        emit(line, per)
     if ctx.world > 1:
         ctx.dist.barrier()
         ctx.dist.destroy_process_group()

@@ -25,6 +25,13 @@ def test_reference_arm_runs_the_oracle_with_the_requested_steps():
     assert line["value"] > 0 and line["gpu_launches"] == 0
 
 
+def test_the_result_is_one_line_on_stdout_and_the_records_go_to_stderr(capsys):
+    bench.emit({"metric": bench.METRIC, "value": 1.5}, [{"workload": "a"}, {"workload": "b"}])
+    got = capsys.readouterr()
+    assert [json.loads(x) for x in got.out.splitlines()] == [{"metric": bench.METRIC, "value": 1.5}]
+    assert [json.loads(x)["per_workload"]["workload"] for x in got.err.splitlines()] == ["a", "b"]
+
+
 def test_default_headline_is_the_largest_prefill_configuration():
     args = bench.parse_args([])
     assert args.workload == "c4_long_context" and args.gpus == 1 and args.warmup >= 3

@@ -65,7 +65,7 @@ def test_moe_edges(T, C, F, E, K, shrink):
 
 @pytest.mark.parametrize("H,Sq,Sk,causal", [
     (74, 256, 400, False), (75, 256, 400, False),    # 148 / 150 tiles of 128 rows: one per SM, and more
-    (74, 512, 512, True), (75, 512, 512, True),      # 296 / 300: two per SM
+    (74, 512, 512, True), (75, 512, 512, True),      # 296 / 300: two per SM, both in the two-sub-tile kernel
     (148, 400, 384, False), (148, 400, 385, False),  # 592 tiles of three / four key steps
 ])
 def test_sides_of_the_kernel_choice(H, Sq, Sk, causal):

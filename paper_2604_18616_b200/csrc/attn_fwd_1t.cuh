@@ -10,7 +10,8 @@
 // two chains of an SM are two independent CTAs, each with its own tile sequence, Q, K/V ring, TMEM half
 // and MMA warp; one CTA's tile boundary (epilogue, next Q, pipeline refill) overlaps the other's steady
 // state.  The price is that each CTA loads K and V for 128 rows instead of 256, i.e. twice the L2 and
-// shared-memory traffic per query row; the launch code picks this kernel only where tiles are short.
+// shared-memory traffic per query row; one_subtile_is_faster (work_tiles.cuh) says where that is worth it: few rows, tiles
+// that do not fill the SMs, causal tiles of very different lengths.
 //
 //   warp 0        producer: TMA loads of Q and of the K/V ring
 //   warp 1        MMA issuer: S = Q K_j^T and O += P V_j on tcgen05

@@ -302,12 +302,14 @@ def splitkv_default_splits(B, H, Hkv, Sq, Sk, D) -> int:
 
 def _check_qkv(q, k, v):
     """The checks of ave_attn_fwd for its split-KV variants; the sizes B, H, Hkv, Sq, Sk, D."""
-    for t in (q, k, v):
-        if not (t.is_cuda and t.dtype is torch.bfloat16 and t.dim() == 4 and t.is_contiguous()):
-            raise ValueError("q, k, v must be contiguous 4-D CUDA bfloat16 tensors")
-    B, H, Sq, D = q.shape
-    Bk, Hkv, Sk, Dk = k.shape
-    if v.shape != k.shape or Bk != B or Dk != D:
+    bf16 = torch.bfloat16
+    if not (q.is_cuda and k.is_cuda and v.is_cuda and q.dtype is bf16 and k.dtype is bf16 and v.dtype is bf16
+            and q.is_contiguous() and k.is_contiguous() and v.is_contiguous()):
+        raise ValueError("q, k, v must be contiguous 4-D CUDA bfloat16 tensors")
+    kshape = k.shape
+    B, H, Sq, D = q.shape  # (a ValueError too unless there are four)
+    Bk, Hkv, Sk, Dk = kshape
+    if v.shape != kshape or Bk != B or Dk != D:
         raise ValueError("inconsistent q/k/v shapes")
     return B, H, Hkv, Sq, Sk, D
 

@@ -29,7 +29,7 @@ extern "C" {
  * a: bf16 [M, K] row-major, device, read.   b: bf16 [N, K] row-major, device, read.
  * c: bf16 [M, N] row-major, device, written; must not alias a or b.
  * M, N, K > 0; K and N multiples of 8 (rows of 16-byte multiples, a TMA rule);
- * M * K, N * K, M * N below 2^40 elements.  a, b, c 16-byte aligned.
+ * M * K, N * K, M * N below 2^39 elements.  a, b, c 16-byte aligned.
  * Errors, checked in this order before any CUDA call, nothing launched:
  * AVE_ERR_NULL_POINTER, AVE_ERR_BAD_SHAPE (sizes), AVE_ERR_MISALIGNED
  * (K or N not a multiple of 8, or a pointer not 16-byte aligned); then

@@ -45,7 +45,7 @@ struct GemmParams {
     int M, N, K;
     int tiles_m, tiles_n;  // output tiles along M and N
     int group_m;           // tiles along M walked together before moving along N (L2 reuse of the B tiles)
-    int tile_n;            // (CTA pairs) columns of a tile: 128, 192 or 256
+    int tile_n;            // (CTA pairs) columns of a tile: 64, 128, 192 or 256
     int splits;            // (one CTA per tile and share of K) CTAs of a cluster
     void *c;               // the result, for stores that do not go through its tensor map
 };

@@ -51,5 +51,5 @@ def test_every_choice_can_be_launched(choose):
         if c > 0:
             assert c in (1, 2, 4, 8) and c * tiles <= sms and c <= slices   # all clusters resident, a slice for each CTA
         elif c < 0:
-            assert M > 128 and -c in ((128, 256) if layout == "nn" else (128, 192, 256))
-    assert seen == {1, 2, 4, 8, WIDE, -128, -192, -256}                     # no choice that nothing reaches
+            assert M > 128 and -c in ((128, 256) if layout == "nn" else (64, 128, 192, 256))
+    assert seen == {1, 2, 4, 8, WIDE, -64, -128, -192, -256}                   # no choice that nothing reaches

@@ -16,14 +16,14 @@ from paper_2604_18616_b200 import binding, inputs
 pytestmark = pytest.mark.gpu
 
 CASES = [
-    # M, N, K: few 128 x 128 tiles and a long K (clusters of 8, 8, 2, 4, 4), single CTAs, CTA pairs with tiles of 192 columns
-    # (N-contiguous B: 128 x 256 tiles) and of 128, 128 x 256 tiles; ragged edges
+    # M, N, K: few 128 x 128 tiles and a long K (clusters of 8, 8, 2, 4), CTA pairs with tiles of 64 columns (N-contiguous B: a
+    # cluster of 4), single CTAs, CTA pairs with tiles of 64, 192 (N-contiguous B: 256) and 128 columns; ragged edges
     (200, 512, 2056),     # a last slice of 8
     (257, 136, 4096),
     (1939, 440, 2416),
     (300, 1000, 3000),    # 24 tiles
     (130, 264, 1000),     # edges just past a tile, a last slice of 40
-    (1, 8, 2048),         # a single row and one group of columns (clusters of 4, N-contiguous B: 8)
+    (1, 8, 2048),         # a single row and one group of columns (clusters of 8)
     (128, 128, 256),
     (700, 1000, 712),
     (300, 2000, 520),

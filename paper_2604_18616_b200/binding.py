@@ -32,6 +32,9 @@ STATUS_BIT_SELFTEST = 16
 SPLITKV_STATIC_SCRATCH_BYTES = 8 << 20
 
 _lib = None
+# The ordinary case of the calls below in C++ (csrc/fastcall.cc); each returns None for a call that is not one.
+_fast = None
+FAST_PATH = os.path.join(_HERE, "_fastcall.so")
 
 
 class AveAttnError(RuntimeError):
@@ -97,8 +100,26 @@ def lib() -> ctypes.CDLL:
         L.ave_attn_selftest_inject_failures.restype = ci
         L.ave_attn_selftest_wait_timeout.argtypes = [ci, vp]
         L.ave_attn_selftest_wait_timeout.restype = ci
+        _bind_fast(L)
         _lib = L
     return _lib
+
+
+def _bind_fast(L) -> None:
+    global _fast
+    if not os.path.exists(FAST_PATH):
+        raise RuntimeError("%s is missing: build it with `python -m paper_2604_18616_b200.build`" % FAST_PATH)
+    from . import _fastcall
+    _fastcall.bind(*[ctypes.cast(f, ctypes.c_void_p).value for f in (
+        L.ave_attn_fwd, L.ave_attn_fwd_splitkv, L.ave_gemm_bf16_tn, L.ave_gemm_bf16_nn)])
+    _fast = _fastcall
+
+
+def _checked(r, name):
+    """The result of a fast call, which is the library's status (an int) where that is not AVE_OK."""
+    if type(r) is int:
+        raise AveAttnError(r, name)
+    return r
 
 
 def strerror(status: int) -> str:
@@ -198,6 +219,10 @@ def ave_attn_fwd(q, k, v, o=None, lse=None, causal=False, scale=None, stream=Non
     ``lse`` (fp32) are allocated when not given.  Raises ``AveAttnError`` on a
     non-zero status.
     """
+    if o is None and lse is None and stream is None and _fast is not None:
+        r = _fast.attn_fwd(q, k, v, causal, scale)
+        if r is not None:
+            return _checked(r, "ave_attn_fwd")
     for t in (q, k, v):
         if not (t.is_cuda and t.dtype is torch.bfloat16 and t.dim() == 4 and t.is_contiguous()):
             raise ValueError("q, k, v must be contiguous 4-D CUDA bfloat16 tensors")
@@ -318,6 +343,10 @@ def ave_attn_fwd_splitkv(q, k, v, n_splits, workspace=None, o=None, lse=None, ca
     """Split-KV variant of ``ave_attn_fwd``: same tensors and result; ``workspace``
     is a CUDA uint8 tensor of at least ``splitkv_workspace_bytes`` bytes
     (allocated here when not given)."""
+    if o is None and lse is None and stream is None and _fast is not None:
+        r = _fast.attn_fwd_splitkv(q, k, v, n_splits, workspace, causal, scale)
+        if r is not None:
+            return _checked(r, "ave_attn_fwd_splitkv")
     B, H, Hkv, Sq, Sk, D = _check_qkv(q, k, v)
     if o is None:
         o = torch.empty_like(q)
@@ -356,6 +385,10 @@ def ave_gemm_bf16_tn_raw(a_ptr, b_ptr, c_ptr, M, N, K, stream_ptr=None) -> int:
 
 def ave_gemm_bf16_tn(a, b, c=None, stream=None):
     """C [M, N] = a [M, K] . b [N, K]^T on the tensors' CUDA device (contiguous bf16)."""
+    if c is None and stream is None and _fast is not None:
+        r = _fast.gemm_tn(a, b)
+        if r is not None:
+            return _checked(r, "ave_gemm_bf16_tn")
     for t in (a, b):
         if not (t.is_cuda and t.dtype is torch.bfloat16 and t.dim() == 2 and t.is_contiguous()):
             raise ValueError("a and b must be contiguous 2-D CUDA bfloat16 tensors")
@@ -377,6 +410,10 @@ def ave_gemm_bf16_nn_raw(a_ptr, b_ptr, c_ptr, M, N, K, stream_ptr=None) -> int:
 
 def ave_gemm_bf16_nn(a, b, c=None, stream=None):
     """C [M, N] = a [M, K] . b [K, N] on the tensors' CUDA device (contiguous bf16)."""
+    if c is None and stream is None and _fast is not None:
+        r = _fast.gemm_nn(a, b)
+        if r is not None:
+            return _checked(r, "ave_gemm_bf16_nn")
     for t in (a, b):
         if not (t.is_cuda and t.dtype is torch.bfloat16 and t.dim() == 2 and t.is_contiguous()):
             raise ValueError("a and b must be contiguous 2-D CUDA bfloat16 tensors")

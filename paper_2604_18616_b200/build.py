@@ -1,7 +1,7 @@
-"""Compile the CUDA library for sm_100a with nvcc, in-tree.
+"""Compile the CUDA library for sm_100a with nvcc and the binding's C++ part with g++, in-tree.
 
 ``python -m paper_2604_18616_b200.build`` (or ``build_cuda()``) writes
-``libave_attn.so`` next to this file.  nvcc cross-compiles without a GPU.
+``libave_attn.so`` and ``_fastcall.so`` next to this file.  nvcc cross-compiles without a GPU.
 
 The build reads ptxas' resource report and refuses an image in which an
 attention kernel got fewer registers per thread than its warp roles' register
@@ -18,6 +18,7 @@ import sys
 _HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(_HERE, "csrc")
 LIB_PATH = os.path.join(_HERE, "libave_attn.so")
+FAST_PATH = os.path.join(_HERE, "_fastcall.so")
 INCLUDE = os.path.join(os.path.dirname(_HERE), "include")
 
 NVCC_FLAGS = [
@@ -74,7 +75,38 @@ def check_register_split(ptxas_report: str) -> dict:
     return regs
 
 
+def build_fastcall(force: bool = False) -> str:
+    """The C++ part of the binding: a Python extension over torch's C++ library."""
+    import sysconfig
+
+    import torch
+    src = os.path.join(CSRC, "fastcall.cc")
+    tdir = os.path.dirname(torch.__file__)
+    # (built again when another torch is installed: it uses torch's C++ interface)
+    stamp, stamp_path = "%s %s %s" % (torch.__version__, tdir, sysconfig.get_paths()["include"]), FAST_PATH + ".stamp"
+    if not force and os.path.exists(FAST_PATH) and os.path.getmtime(FAST_PATH) >= os.path.getmtime(src) and os.path.exists(stamp_path):
+        with open(stamp_path) as f:
+            if f.read() == stamp:
+                return FAST_PATH
+    cuda_home = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    tmp = FAST_PATH + ".tmp%d" % os.getpid()
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden",
+           "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI),
+           "-I" + os.path.join(tdir, "include"), "-I" + os.path.join(tdir, "include", "torch", "csrc", "api", "include"),
+           "-I" + os.path.join(cuda_home, "include"), "-I" + sysconfig.get_paths()["include"], "-o", tmp, src,
+           "-L" + os.path.join(tdir, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"]
+    r = subprocess.run(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
+    if r.returncode != 0:
+        sys.stderr.write(r.stdout)
+        raise subprocess.CalledProcessError(r.returncode, cmd)
+    os.replace(tmp, FAST_PATH)
+    with open(stamp_path, "w") as f:
+        f.write(stamp)
+    return FAST_PATH
+
+
 def build_cuda(force: bool = False, verbose: bool = False) -> str:
+    build_fastcall(force)
     newest = max(os.path.getmtime(s) for s in _sources())
     if not force and os.path.exists(LIB_PATH) and os.path.getmtime(LIB_PATH) >= newest:
         return LIB_PATH

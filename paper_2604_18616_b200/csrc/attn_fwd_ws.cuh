@@ -31,7 +31,7 @@
 
 namespace ave {
 
-template <int D>
+template <int D, bool CAUSAL = true>
 struct WsCfg {
     static constexpr int kThreads = 384;
     static constexpr int kQRows = 2 * BM;                    // query rows per work tile
@@ -41,6 +41,10 @@ struct WsCfg {
     static constexpr int kStages = (D == 128) ? 4 : 8;       // ring slots, K and V tiles alternate
     static constexpr int kStageOBytes = kBoxBytes;           // O staging per sub-tile: 64 columns at a time
     static constexpr int kOutBoxRows = 32;                   // each softmax warp stores its own 32 rows
+    // Keys of a step whose probabilities are handed over first, so that P V starts while the others are computed (128: all
+    // at once).  Why, where and what it measured: see where the softmax hands P over.
+    static constexpr int kPFirst = (CAUSAL || D == 128) ? 96 : 128;
+    static constexpr int kPParts = kPFirst < 128 ? 2 : 1;
     static constexpr int kSmemBytes = kTileBytes * (2 + kStages) + 2 * kStageOBytes + 1024;
     static constexpr uint32_t kTmemCols = 512;
     static constexpr uint32_t kColS0 = 0, kColS1 = 128, kColO0 = 256, kColO1 = 384;
@@ -130,13 +134,14 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                    const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_o,
                    const FwdParams p) {
     if (threadIdx.x == 0) span_stamp(0);
-    using Cfg = WsCfg<D>;
+    using Cfg = WsCfg<D, CAUSAL>;
     constexpr int NS = Cfg::kStages;
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(16) unsigned long long clc_response[2][2];
     __shared__ __align__(8) uint64_t bar_q_full[2], bar_q_empty[2], bar_s[2], bar_p[2], bar_o[2], bar_o_free[2];
     __shared__ __align__(8) uint64_t bar_full[NS], bar_empty[NS];
     __shared__ __align__(8) uint64_t bar_tile_full[2], bar_tile_ready[2], bar_tile_empty[2], bar_drain;
+    __shared__ __align__(8) uint64_t bar_p_rest[2];  // the second part of P_t, where it is handed over in two
     // The scheduler warp decodes every tile it obtains once, for all warps: index and decoded form, two in flight.
     __shared__ int tile_id[2];
     __shared__ TileOf<SPLIT, VARLEN> tile_info[2];
@@ -162,6 +167,7 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
             mbar_init(smem_u32(&bar_q_empty[t]), 1);
             mbar_init(smem_u32(&bar_s[t]), 1);
             mbar_init(smem_u32(&bar_p[t]), 4);       // one arrival per softmax warp
+            if (Cfg::kPParts == 2) mbar_init(smem_u32(&bar_p_rest[t]), 4);
             mbar_init(smem_u32(&bar_o[t]), 1);
             mbar_init(smem_u32(&bar_o_free[t]), 4);  // one arrival per softmax warp
             mbar_init(smem_u32(&bar_tile_full[t]), 1);
@@ -401,14 +407,26 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                     umma_commit(smem_u32(&bar_s[t]));
                 }
             };
-            auto issue_pv = [&](int t, uint32_t v_addr, bool first) {
+            auto issue_pv = [&](int t, uint32_t v_addr, bool first, int k_from = 0, int k_to = BN) {
                 if (leader) {
                     const uint32_t v_lo = lo_v | (v_addr >> 4);
 #pragma unroll
                     for (int kk = 0; kk < BN / 16; ++kk)
-                        umma_ts_words(tO[t], tS[t] + kk * 8, v_lo + ((kk * 16 * 128) >> 4), hi_v, idesc_pv,
-                                      (!first || kk > 0));
+                        if (kk * 16 >= k_from && kk * 16 < k_to)
+                            umma_ts_words(tO[t], tS[t] + kk * 8, v_lo + ((kk * 16 * 128) >> 4), hi_v, idesc_pv,
+                                          (!first || kk > 0));
                 }
+            };
+            // The same, each part of the keys as soon as its probabilities are there
+            auto take_p_and_issue_pv = [&](int t, uint32_t v_addr, bool first) {
+#pragma unroll
+                for (int part = 0; part < 2; ++part) {
+                    ok = wait_bar(part ? &bar_p_rest[t] : &bar_p[t], np[t] & 1, STATUS_TIMEOUT_SOFTMAX);
+                    if (!ok) return;
+                    tc_fence_after();
+                    issue_pv(t, v_addr, first, part ? Cfg::kPFirst : 0, part ? BN : Cfg::kPFirst);
+                }
+                ++np[t];
             };
 
             // First step of sub-tile t in tile number `tn` (tile `wt`, whose K_0 sits at ring position
@@ -460,12 +478,18 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                     if (!ok) break;
                     const uint32_t v_addr = slot_addr(iv), k_addr = slot_addr(ik);
                     if (j < n0) {
-                        ok = wait_bar(&bar_p[0], np[0] & 1, STATUS_TIMEOUT_SOFTMAX);
-                        if (!ok) break;
-                        ++np[0];
-                        if (traced(n) && lane == 0) trace_stamp(0, trace_it(n, j), 1);
-                        tc_fence_after();
-                        issue_pv(0, v_addr, j == 0);
+                        if constexpr (Cfg::kPParts == 2) {
+                            take_p_and_issue_pv(0, v_addr, j == 0);
+                            if (!ok) break;
+                            if (traced(n) && lane == 0) trace_stamp(0, trace_it(n, j), 1);
+                        } else {
+                            ok = wait_bar(&bar_p[0], np[0] & 1, STATUS_TIMEOUT_SOFTMAX);
+                            if (!ok) break;
+                            ++np[0];
+                            if (traced(n) && lane == 0) trace_stamp(0, trace_it(n, j), 1);
+                            tc_fence_after();
+                            issue_pv(0, v_addr, j == 0);
+                        }
                         if (leader && j == n0 - 1) umma_commit(smem_u32(&bar_o[0]));
                         if (j + 1 < n0) {
                             issue_qk(0, k_addr);
@@ -476,12 +500,18 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                         }
                     }
                     if (traced(n) && lane == 0) trace_stamp(0, trace_it(n, j), 2);
-                    ok = wait_bar(&bar_p[1], np[1] & 1, STATUS_TIMEOUT_SOFTMAX);
-                    if (!ok) break;
-                    ++np[1];
-                    if (traced(n) && lane == 0) trace_stamp(0, trace_it(n, j), 3);
-                    tc_fence_after();
-                    issue_pv(1, v_addr, j == 0);
+                    if constexpr (Cfg::kPParts == 2) {
+                        take_p_and_issue_pv(1, v_addr, j == 0);
+                        if (!ok) break;
+                        if (traced(n) && lane == 0) trace_stamp(0, trace_it(n, j), 3);
+                    } else {
+                        ok = wait_bar(&bar_p[1], np[1] & 1, STATUS_TIMEOUT_SOFTMAX);
+                        if (!ok) break;
+                        ++np[1];
+                        if (traced(n) && lane == 0) trace_stamp(0, trace_it(n, j), 3);
+                        tc_fence_after();
+                        issue_pv(1, v_addr, j == 0);
+                    }
                     if (leader) umma_commit(smem_u32(&bar_empty[iv % NS]));
                     if (leader && j == n1 - 1) umma_commit(smem_u32(&bar_o[1]));
                     if (j + 1 < n1) {
@@ -616,97 +646,166 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                         const float ext = fmaxf(fmaxf(e0, e1), fmaxf(e2, e3));
                         return (ext == -INFINITY) ? -INFINITY : ext * sl2;
                     };
-                    // p = exp2(scale*log2e*s - m) for the whole row: P -> bf16 pairs into TMEM over the
-                    // first 64 columns of S_t; returns the row sum of the fp32 probabilities.
-                    auto exp_pass = [&](float m_ref) -> float {
-                        const float neg_m = (m_ref == -INFINITY) ? 0.f : -m_ref;
-                        float2 acc0 = make_float2(0.f, 0.f), acc1 = make_float2(0.f, 0.f);
-                        const float2 sc2 = make_float2(sl2, sl2), nm2 = make_float2(neg_m, neg_m);
-#pragma unroll
-                        for (int cc = 0; cc < 4; ++cc) {
-                            uint32_t pk[16];
-#pragma unroll
-                            for (int e = 0; e < 32; e += 2) {
-                                const float2 x = __ffma2_rn(
-                                    make_float2(__uint_as_float(sraw[cc][e]), __uint_as_float(sraw[cc][e + 1])), sc2, nm2);
-                                float2 pr;
-                                if ((kFmaPipeExpMask >> ((e >> 1) & 7)) & 1) {
-                                    pr = exp2_fma_pipe(x);
-                                } else {
-                                    pr.x = ex2_approx(x.x);
-                                    pr.y = ex2_approx(x.y);
-                                }
-                                if (e & 2) acc1 = __fadd2_rn(acc1, pr);  // fp32 probabilities, before rounding to bf16
-                                else       acc0 = __fadd2_rn(acc0, pr);
-                                pk[e >> 1] = pack_bf16x2(pr.x, pr.y);
-                            }
-                            tmem_st_x16(tS + cc * 16, pk);
-                        }
-                        return (acc0.x + acc0.y) + (acc1.x + acc1.y);
-                    };
-                    // O <- alpha * O.  S_t(j) ready implies P_t V_{j-1} has finished (in-order tensor pipe).
-                    auto rescale_o_wide = [&](float alpha) {
-                        uint32_t oc[D / 32][32];
-#pragma unroll
-                        for (int c = 0; c < D / 32; ++c) tmem_ld_x32(tO + c * 32, oc[c]);
-                        tmem_wait_ld();
-#pragma unroll
-                        for (int c = 0; c < D / 32; ++c) {
-#pragma unroll
-                            for (int e = 0; e < 32; ++e) oc[c][e] = __float_as_uint(__uint_as_float(oc[c][e]) * alpha);
-                            tmem_st_x32(tO + c * 32, oc[c]);
-                        }
-                    };
-
                     // ---- running maximum, moved lazily: probabilities are taken relative to m_run, which
                     // only moves when the row maximum has grown by more than the threshold
                     float alpha = 1.f, row_sum = 0.f;
-                    // exact: take the maximum first, then exponentiate against it.  (The causal
-                    // instantiations always do: with their masking code the second copy of the
-                    // exponentiation loop costs registers and measured slower.)
-                    bool exact = CAUSAL || (j == 0);
-                    bool maximum_settled = false;
-                    if (!exact) {
-                        // Optimistic: start exponentiating against the current m_run at once and find the
-                        // tile maximum alongside; only if it exceeds m_run by more than the threshold
-                        // (rare after a row's first tiles) is the row redone, and O rescaled, below.
-                        const float m_tile = tile_max();
-                        row_sum = exp_pass(m_run);
-                        const bool moved = m_tile - m_run > rescale_margin(l_run);  // also true for m_run = -inf < m_tile
-                        if (__any_sync(0xffffffffu, moved)) {
-                            if (moved) {
-                                alpha = ex2_approx(m_run - m_tile);  // m_tile is finite here
-                                m_run = m_tile;
+                    if constexpr (Cfg::kPParts == 1) {
+                        // p = exp2(scale*log2e*s - m) for the whole row: P -> bf16 pairs into TMEM over the
+                        // first 64 columns of S_t; returns the row sum of the fp32 probabilities.
+                        auto exp_pass = [&](float m_ref) -> float {
+                            const float neg_m = (m_ref == -INFINITY) ? 0.f : -m_ref;
+                            float2 acc0 = make_float2(0.f, 0.f), acc1 = make_float2(0.f, 0.f);
+                            const float2 sc2 = make_float2(sl2, sl2), nm2 = make_float2(neg_m, neg_m);
+#pragma unroll
+                            for (int cc = 0; cc < 4; ++cc) {
+                                uint32_t pk[16];
+#pragma unroll
+                                for (int e = 0; e < 32; e += 2) {
+                                    const float2 x = __ffma2_rn(
+                                        make_float2(__uint_as_float(sraw[cc][e]), __uint_as_float(sraw[cc][e + 1])), sc2, nm2);
+                                    float2 pr;
+                                    if ((kFmaPipeExpMask >> ((e >> 1) & 7)) & 1) {
+                                        pr = exp2_fma_pipe(x);
+                                    } else {
+                                        pr.x = ex2_approx(x.x);
+                                        pr.y = ex2_approx(x.y);
+                                    }
+                                    if (e & 2) acc1 = __fadd2_rn(acc1, pr);  // fp32 probabilities, before rounding to bf16
+                                    else       acc0 = __fadd2_rn(acc0, pr);
+                                    pk[e >> 1] = pack_bf16x2(pr.x, pr.y);
+                                }
+                                tmem_st_x16(tS + cc * 16, pk);
                             }
-                            exact = true;
-                            maximum_settled = true;
-                        }
-                    }
-                    if (exact) {
-                        if (!maximum_settled) {
+                            return (acc0.x + acc0.y) + (acc1.x + acc1.y);
+                        };
+                        // O <- alpha * O.  S_t(j) ready implies P_t V_{j-1} has finished (in-order tensor pipe).
+                        auto rescale_o_wide = [&](float alpha) {
+                            uint32_t oc[D / 32][32];
+#pragma unroll
+                            for (int c = 0; c < D / 32; ++c) tmem_ld_x32(tO + c * 32, oc[c]);
+                            tmem_wait_ld();
+#pragma unroll
+                            for (int c = 0; c < D / 32; ++c) {
+#pragma unroll
+                                for (int e = 0; e < 32; ++e) oc[c][e] = __float_as_uint(__uint_as_float(oc[c][e]) * alpha);
+                                tmem_st_x32(tO + c * 32, oc[c]);
+                            }
+                        };
+
+                        // exact: take the maximum first, then exponentiate against it.
+                        bool exact = j == 0;
+                        bool maximum_settled = false;
+                        if (!exact) {
+                            // Optimistic: start exponentiating against the current m_run at once and find the
+                            // tile maximum alongside; only if it exceeds m_run by more than the threshold
+                            // (rare after a row's first tiles) is the row redone, and O rescaled, below.
                             const float m_tile = tile_max();
-                            if (j == 0) {
-                                m_run = m_tile;
-                            } else if (m_tile - m_run > rescale_margin(l_run)) {
-                                alpha = ex2_approx(m_run - m_tile);
-                                m_run = m_tile;
+                            row_sum = exp_pass(m_run);
+                            const bool moved = m_tile - m_run > rescale_margin(l_run);  // also true for m_run = -inf < m_tile
+                            if (__any_sync(0xffffffffu, moved)) {
+                                if (moved) {
+                                    alpha = ex2_approx(m_run - m_tile);  // m_tile is finite here
+                                    m_run = m_tile;
+                                }
+                                exact = true;
+                                maximum_settled = true;
                             }
+                        }
+                        if (exact) {
+                            if (!maximum_settled) {
+                                const float m_tile = tile_max();
+                                if (j == 0) {
+                                    m_run = m_tile;
+                                } else if (m_tile - m_run > rescale_margin(l_run)) {
+                                    alpha = ex2_approx(m_run - m_tile);
+                                    m_run = m_tile;
+                                }
+                            }
+                            if (traced(n) && tracer) trace_stamp(1 + t, trace_it(n, j), 3);
+                            row_sum = exp_pass(m_run);
+                            // O <- alpha * O after the exponentiation: the score registers are free by then, so the
+                            // whole accumulator row is in flight at once (P_t V_j is not issued before this thread's
+                            // arrival below).
+                            if (j > 0 && __any_sync(0xffffffffu, alpha != 1.f)) rescale_o_wide(alpha);
+                        }
+                        l_run = l_run * alpha + row_sum;
+                        if (traced(n) && tracer) trace_stamp(1 + t, trace_it(n, j), 4);
+
+                        tmem_wait_st();
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(smem_u32(&bar_p[t]));
+                        if (traced(n) && tracer) trace_stamp(1 + t, trace_it(n, j), 5);
+                    } else {
+                        // p = exp2(scale*log2e*s - m) for the keys [c0, c1) of the row: P -> bf16 pairs into TMEM over the
+                        // first 64 columns of S_t; the fp32 probabilities are added to acc0 and acc1.
+                        auto exp_pass = [&](float m_ref, auto c0, auto c1, float2 &acc0, float2 &acc1) {
+                            const float neg_m = (m_ref == -INFINITY) ? 0.f : -m_ref;
+                            const float2 sc2 = make_float2(sl2, sl2), nm2 = make_float2(neg_m, neg_m);
+#pragma unroll
+                            for (int cc = decltype(c0)::value / 32; cc < decltype(c1)::value / 32; ++cc) {
+                                uint32_t pk[16];
+#pragma unroll
+                                for (int e = 0; e < 32; e += 2) {
+                                    const float2 x = __ffma2_rn(
+                                        make_float2(__uint_as_float(sraw[cc][e]), __uint_as_float(sraw[cc][e + 1])), sc2, nm2);
+                                    float2 pr;
+                                    if ((kFmaPipeExpMask >> ((e >> 1) & 7)) & 1) {
+                                        pr = exp2_fma_pipe(x);
+                                    } else {
+                                        pr.x = ex2_approx(x.x);
+                                        pr.y = ex2_approx(x.y);
+                                    }
+                                    if (e & 2) acc1 = __fadd2_rn(acc1, pr);  // fp32 probabilities, before rounding to bf16
+                                    else       acc0 = __fadd2_rn(acc0, pr);
+                                    pk[e >> 1] = pack_bf16x2(pr.x, pr.y);
+                                }
+                                tmem_st_x16(tS + cc * 16, pk);
+                            }
+                        };
+                        // Part of P_t(j) is in TMEM: the MMA warp may take it.
+                        auto hand_over_p = [&](int part) {
+                            tmem_wait_st();
+                            tc_fence_before();
+                            __syncwarp();
+                            if (lane == 0) mbar_arrive(smem_u32(part ? &bar_p_rest[t] : &bar_p[t]));
+                            if (traced(n) && tracer) trace_stamp(1 + t, trace_it(n, j), 5);
+                        };
+                        // The maximum first, then the exponentials against it.  What bounds these kernels is the chain S -> P ->
+                        // P V, Q K^T -> S of a sub-tile: P V of the first 96 keys runs while the last 32 are computed (32
+                        // heads of 16384, peaked 2079 -> 2055 us; 4 x 32 of 2048 180 -> 176, grouped 156.6 -> 152.5; 4 x 32 of
+                        // 8192, D = 64 1505 -> 1492; no mask, 2 x 32 of 8192 1909 -> 1897; the clocks follow the power limit, in
+                        // bursts the gains are twice that; 64 or 32 keys first: within 1 %).  Without a mask at D = 64 the extra
+                        // hand-over costs more than it gives (378 -> 390 us): there the row goes over in one piece.
+                        const float m_tile = tile_max();
+                        if (j == 0) {
+                            m_run = m_tile;
+                        } else if (m_tile - m_run > rescale_margin(l_run)) {
+                            alpha = ex2_approx(m_run - m_tile);
+                            m_run = m_tile;
                         }
                         if (traced(n) && tracer) trace_stamp(1 + t, trace_it(n, j), 3);
-                        row_sum = exp_pass(m_run);
-                        // O <- alpha * O after the exponentiation: the score registers are free by then, so the
-                        // whole accumulator row is in flight at once (P_t V_j is not issued before this thread's
-                        // arrival below).
-                        if (j > 0 && __any_sync(0xffffffffu, alpha != 1.f)) rescale_o_wide(alpha);
+                        float2 acc0 = make_float2(0.f, 0.f), acc1 = make_float2(0.f, 0.f);
+                        exp_pass(m_run, std::integral_constant<int, 0>{}, std::integral_constant<int, Cfg::kPFirst>{}, acc0, acc1);
+                        // (P_t V_j is not issued before the hand-over)
+                        if (j > 0 && __any_sync(0xffffffffu, alpha != 1.f)) {
+#pragma unroll 1
+                            for (int c = 0; c < D; c += 32) {  // O <- alpha * O: S_t(j) ready implies that P_t V_{j-1} has finished (in-order tensor pipe)
+                                uint32_t oc[32];
+                                tmem_ld_x32(tO + c, oc);
+                                tmem_wait_ld();
+                                tmem_pin_x32(oc);
+#pragma unroll
+                                for (int e = 0; e < 32; ++e) oc[e] = __float_as_uint(__uint_as_float(oc[e]) * alpha);
+                                tmem_st_x32(tO + c, oc);
+                            }
+                        }
+                        hand_over_p(0);
+                        exp_pass(m_run, std::integral_constant<int, Cfg::kPFirst>{}, std::integral_constant<int, BN>{}, acc0, acc1);
+                        hand_over_p(1);
+                        row_sum = (acc0.x + acc0.y) + (acc1.x + acc1.y);
+                        l_run = l_run * alpha + row_sum;
                     }
-                    l_run = l_run * alpha + row_sum;
-                    if (traced(n) && tracer) trace_stamp(1 + t, trace_it(n, j), 4);
-
-                    tmem_wait_st();
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(smem_u32(&bar_p[t]));
-                    if (traced(n) && tracer) trace_stamp(1 + t, trace_it(n, j), 5);
                     return true;
                 };
                 {

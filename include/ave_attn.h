@@ -235,12 +235,12 @@ int ave_attn_fwd_splitkv_static(const void *q, const void *k, const void *v, voi
 int ave_attn_device_status(unsigned int *raw_word);
 
 /*
- * The library has two attention kernels for the same operation: one whose CTAs
- * process two 128-row sub-tiles of a 256-row work tile in lock-step (shared K/V
- * loads; the default for problems that fill the GPU), and one with a single
- * 128-row sub-tile per CTA and two CTAs per SM (no lock-step at tile boundaries;
- * the default for at most 128 query rows and where tiles do not fill the SMs,
- * and the only one for D > 128).  which = 0 lets every call
+ * The library has two kinds of attention kernel for the same operation: one whose
+ * work tiles have two 128-row sub-tiles (in one CTA for D <= 128, in the two CTAs of
+ * a pair above; shared K/V loads; the default for problems that fill the GPU), and
+ * one with a single 128-row sub-tile per CTA, two CTAs per SM for D <= 128 (no
+ * lock-step at tile boundaries; the default for at most 128 query rows and where
+ * tiles do not fill the SMs, for D > 128 for few key tiles).  which = 0 lets every call
  * choose by problem shape (the default), 1 / 2 force the first / second for all
  * later calls of this process.  Results agree within rounding order.  Returns
  * AVE_OK, or AVE_ERR_BAD_SHAPE for another value.

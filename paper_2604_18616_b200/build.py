@@ -63,7 +63,7 @@ def kernel_registers(ptxas_report: str) -> dict:
 
 def check_register_split(ptxas_report: str) -> dict:
     """Raise if an attention kernel of the report cannot satisfy its register split."""
-    regs = {k: v for k, v in kernel_registers(ptxas_report).items() if "attn_fwd" in k or "moe_gemm" in k}
+    regs = {k: v for k, v in kernel_registers(ptxas_report).items() if ("attn_fwd" in k and "attn_fwd_pair" not in k) or "moe_gemm" in k}
     if not regs:
         raise RuntimeError("ptxas reported no attention kernel: cannot verify the register split")
     for name, n in regs.items():

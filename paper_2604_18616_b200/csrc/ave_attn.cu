@@ -16,6 +16,7 @@
 
 #include "attn_fwd_ws.cuh"
 #include "attn_fwd_1t.cuh"
+#include "attn_fwd_pair.cuh"
 #include "gemm_bf16.cuh"
 #include "gemm_choice.cuh"
 #include "moe_fp8.cuh"
@@ -308,6 +309,27 @@ int launch_1t(const CUtensorMap &tq, const CUtensorMap &tk, const CUtensorMap &t
     return AVE_OK;
 }
 
+template <bool CAUSAL, bool VARLEN>
+int launch_pair(const CUtensorMap &tq, const CUtensorMap &tk, const CUtensorMap &tv, const ave::FwdParams &p, cudaStream_t stream) {
+    using Cfg = ave::PairCfg;
+    auto kern = ave::attn_fwd_pair_kernel<CAUSAL, VARLEN>;
+    static PerDeviceOnce once;  // per instantiation
+    const int st = prepare_kernel(kern, Cfg::kSmemBytes, 0, once);
+    if (st != AVE_OK) return st;
+    if (take_injected(g_inject_launch_failures)) {
+        t_last_cuda_error = int(cudaErrorLaunchFailure);
+        return AVE_ERR_CUDA;
+    }
+    const cudaError_t e = launch_dependent(kern, dim3(2u * unsigned(p.total_blocks)), dim3(Cfg::kThreads), Cfg::kSmemBytes, stream, tq,
+                                           tk, tv, p);
+    if (e != cudaSuccess) {
+        t_last_cuda_error = int(e);
+        return AVE_ERR_CUDA;
+    }
+    g_launches.fetch_add(1, std::memory_order_relaxed);
+    return AVE_OK;
+}
+
 // Number of SMs of the current device (148, the part this library is written for, if it cannot be asked).
 int sm_count() {
     int dev = 0, sms = 0;
@@ -328,6 +350,15 @@ bool use_one_subtile(int B, int H, int Hkv, int Sq, int Sk, int D, bool causal, 
     // (measured on decode shapes: 0.63-0.66 -> 0.76-0.90 of the copy bandwidth).
     if (Sq <= ave::BM) return true;
     return !split && ave::one_subtile_is_faster(B, H, Hkv, Sq, Sk, D, causal, total_q, sm_count());
+}
+
+// Whether a launch of D > 128 runs on CTA pairs.
+bool use_pairs(int B, int H, int Hkv, int Sq, int Sk, bool causal, int total_q) {
+    const int choice = g_kernel_choice.load(std::memory_order_relaxed);
+    // (a pair's grid, two CTAs a tile, must stay below 2^31)
+    const long long blocks = ((long long)Sq + ave::BM - 1) / ave::BM * B * H;
+    if (choice == 2 || blocks >= (1ll << 30)) return false;
+    return choice == 1 || ave::pairs_are_faster(B, H, Hkv, Sq, Sk, causal, total_q, sm_count());
 }
 
 // Encode the tensor maps, fill the kernel parameters and launch.  In a `split` launch every work tile covers
@@ -351,15 +382,16 @@ int launch_attention(const void *q, const void *k, const void *v, void *o, float
     const Strides sk = layout ? layout[1] : varlen ? token_major(Hkv, rows_k) : contiguous_strides(Hkv, Sk, D);
     const Strides sv = layout ? layout[2] : varlen ? token_major(Hkv, rows_k) : contiguous_strides(Hkv, Sk, D);
     const Strides so = layout ? layout[3] : varlen ? token_major(H, rows_q) : contiguous_strides(H, Sq, D);
-    // a head dimension above 128 leaves no TMEM for a second sub-tile: only the single-sub-tile kernel has it
-    const bool one = D > 128 || use_one_subtile(B, H, Hkv, Sq, Sk, D, causal != 0, split, varlen ? varlen->total_q : 0);
+    // A head dimension above 128 leaves no TMEM for a second sub-tile in one CTA: CTA pairs, or the single-sub-tile kernel.
+    const bool pair = D > 128 && use_pairs(B, H, Hkv, Sq, Sk, causal != 0, varlen ? varlen->total_q : 0);
+    const bool one = D > 128 ? !pair : use_one_subtile(B, H, Hkv, Sq, Sk, D, causal != 0, split, varlen ? varlen->total_q : 0);
     CUtensorMap tq, tk, tv, to;
     if (!encode_map(&tq, q, D, rows_q, H, n_batch, sq, ave::BM)) return AVE_ERR_CUDA;
-    // (the single-sub-tile kernel stores O without a map)
-    if (!one && !encode_map(&to, o, D, rows_q, H, n_batch, so, ave::WsCfg<128>::kOutBoxRows)) return AVE_ERR_CUDA;
-    if (!encode_map(&tk, k, D, rows_k, Hkv, n_batch, sk, ave::BN)) return AVE_ERR_CUDA;
-    // (head dimensions above 128 take V by halves of the keys)
-    if (!encode_map(&tv, v, D, rows_k, Hkv, n_batch, sv, D > 128 ? ave::BN / 2 : ave::BN)) return AVE_ERR_CUDA;
+    // (the single-sub-tile kernel and the pairs store O without a map)
+    if (!one && !pair && !encode_map(&to, o, D, rows_q, H, n_batch, so, ave::WsCfg<128>::kOutBoxRows)) return AVE_ERR_CUDA;
+    if (!encode_map(&tk, k, D, rows_k, Hkv, n_batch, sk, pair ? ave::BN / 2 : ave::BN)) return AVE_ERR_CUDA;  // (a pair: half of the keys in each CTA)
+    // (the single-sub-tile kernel takes V of head dimensions above 128 by halves of the keys, a pair by halves of the columns)
+    if (!encode_map(&tv, v, D, rows_k, Hkv, n_batch, sv, D > 128 && one ? ave::BN / 2 : ave::BN)) return AVE_ERR_CUDA;
 
     ave::FwdParams p{};
     p.o = o;
@@ -378,6 +410,10 @@ int launch_attention(const void *q, const void *k, const void *v, void *o, float
     p.lse_partial = lse_partial;
     p.scale_log2 = scale * 1.4426950408889634f;
 
+    if (pair) {
+        if (varlen) return causal ? launch_pair<true, true>(tq, tk, tv, p, s) : launch_pair<false, true>(tq, tk, tv, p, s);
+        return causal ? launch_pair<true, false>(tq, tk, tv, p, s) : launch_pair<false, false>(tq, tk, tv, p, s);
+    }
     if (one && Dk == 256) {  // (the split-KV entry points take 64 or 128 only)
         if (varlen)
             return causal ? launch_1t<256, true, false, true>(tq, tk, tv, p, s) : launch_1t<256, false, false, true>(tq, tk, tv, p, s);

@@ -285,6 +285,28 @@ inline bool one_subtile_is_faster(int B, int H, int Hkv, int Sq, int Sk, int D, 
     // Larger problems want the shared K/V loads of the two-sub-tile kernel (6-15 % on the prefill configurations).
 }
 
+// Whether a problem with a head dimension above 128 is better off on CTA pairs (two 128-row sub-tiles a pair) than in the
+// single-sub-tile kernel (a CTA for 128 rows).  Times below: pairs / single, D = 256, from 70 shapes.
+inline bool pairs_are_faster(int B, int H, int Hkv, int Sq, int Sk, bool causal, int total_q, int sms) {
+    auto blocks = [&](int rows) {
+        return total_q > 0 ? (long long)total_q / rows + B : (long long)B * (((long long)Sq + rows - 1) / rows);
+    };
+    const long long tiles = H * blocks(BM);
+    const long long ctas = causal && H / Hkv % 2 == 0 ? tiles : 2 * H * blocks(2 * BM);  // (an odd last block leaves a CTA without rows)
+    // A pair starts and ends a tile some 3 us later and then gains 0.4 us a step: from six key tiles on it is ahead (8 heads of
+    // 177 rows and 699 keys 15.6 / 16.8 us, 8 of 286 and 517 17.7 / 17.3), from four if the tiles follow one another (4 x 16 heads
+    // of 300 rows 20.1 / 21.6 and 256 of 512 59 / 64, but 48 of 505 20.9 / 20.7, 32 of 366 14.2 / 13.7).
+    const int key_tiles = (Sk + BN - 1) / BN;
+    if (key_tiles < 4 || (key_tiles < 6 && tiles <= 2 * sms)) return false;
+    // Where CTAs without rows cost another wave they take it back (144 tiles, 160 CTAs of 1056 keys: 32.9 / 23.6 us; 144 and 288
+    // of 2489 keys: 68.3 / 47.9).  A step of a pair takes 0.77 to 0.87 of the other kernel's time.
+    auto waves = [&](long long n) {
+        const double x = double(n) / sms;
+        return x <= 1. ? 1. : causal || x > 3. ? x : double((n + sms - 1) / sms);
+    };
+    return 0.85 * waves(ctas) <= waves(tiles);
+}
+
 // Split-KV launches: keys per range = an equal share of Sk rounded up to whole key tiles.
 inline int splitkv_keys_per_split(int Sk, int n_splits) {
     const long long share = ((long long)Sk + n_splits - 1) / n_splits;

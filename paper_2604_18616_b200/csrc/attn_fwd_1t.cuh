@@ -45,7 +45,7 @@
 
 namespace ave {
 
-template <int D>
+template <int D, bool WHOLE_P = false>  // WHOLE_P: P is handed over in one piece
 struct OneCfg {
     static constexpr int kThreads = 256;
     static constexpr int kTileBytes = BM * D * 2;            // the Q tile, a K tile or a V tile
@@ -69,9 +69,10 @@ struct OneCfg {
                   "register split exceeds the CTA's allocation");
     // Keys of a step whose probabilities are handed over first: P V of them runs while the others are computed, which shortens
     // the chain of a step (8 heads of 1483 rows, D = 128 26.0 -> 24.1 us; 8 of 200 rows and 8000 keys 106.1 -> 97.9).  With two score
-    // buffers the products are ahead of the softmax anyway.
-    static constexpr int kPFirst = kTwoS ? 128 : 96;
-    static constexpr int kPParts = kTwoS ? 1 : 2;
+    // buffers the products are ahead of the softmax anyway; a decode step waits for HBM, and the extra hand-over is lost
+    // (64 sequences of 4001 keys 192.4 -> 193.5).
+    static constexpr int kPFirst = kTwoS || WHOLE_P ? 128 : 96;
+    static constexpr int kPParts = kPFirst < 128 ? 2 : 1;
     static constexpr int kTileConsumers = 6;                 // producer + MMA + 4 softmax warps read each tile
 };
 
@@ -80,7 +81,7 @@ __global__ void __launch_bounds__(256, 2)
 attn_fwd_1t_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                    const __grid_constant__ CUtensorMap tm_v, const FwdParams p) {
     if (threadIdx.x == 0) span_stamp(0);
-    using Cfg = OneCfg<D>;
+    using Cfg = OneCfg<D, SPLIT || VARLEN>;
     using Tile = TileOf<SPLIT, VARLEN>;
     constexpr int NS = Cfg::kStages;
     extern __shared__ uint8_t smem_raw[];
@@ -357,7 +358,7 @@ attn_fwd_1t_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                 // the keys that come at once: a ring slot's (half of V's, two score buffers), or a part of P's
                 const uint32_t tP = score_buf(np);
 #pragma unroll
-                for (int part = 0; part < 2; ++part) {
+                for (int part = 0; part < (Cfg::kTwoS ? 2 : Cfg::kPParts); ++part) {
                     const int k0 = part * (Cfg::kTwoS ? BN / 2 : Cfg::kPFirst), k1 = part ? BN : Cfg::kTwoS ? BN / 2 : Cfg::kPFirst;
                     if (Cfg::kTwoS) ok = part ? wait_full(pos + 1) : wait_bar(&bar_p[np & 1][0], (np >> 1) & 1, STATUS_TIMEOUT_SOFTMAX);
                     else ok = wait_bar(&bar_p[0][part], np & 1, STATUS_TIMEOUT_SOFTMAX);
@@ -369,7 +370,7 @@ attn_fwd_1t_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
 #pragma unroll
                         for (int k = k0; k < k1; k += 16)
                             umma_ts_words(tO, tP + k / 2, v_lo + ((k * 128) >> 4), hi_v, idesc_pv, (!first || k > 0));
-                        if (Cfg::kTwoS || part == 1) umma_commit(smem_u32(&bar_empty[slot % NS]));
+                        if (Cfg::kTwoS || part == Cfg::kPParts - 1) umma_commit(smem_u32(&bar_empty[slot % NS]));
                     }
                 }
                 if (Cfg::kTwoS && leader) umma_commit(smem_u32(&bar_pv));
@@ -480,7 +481,7 @@ attn_fwd_1t_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                 for (int j = 0; j < n_t && ok; ++j) {
                     ok = wait_bar(&bar_s[0], ns & 1, STATUS_TIMEOUT_MMA);
                     ++ns;
-                    if (ok && lane < 2) mbar_arrive(smem_u32(&bar_p[0][lane]));
+                    if (ok && lane < Cfg::kPParts) mbar_arrive(smem_u32(&bar_p[0][lane]));
                 }
                 if (ok) ok = wait_bar(&bar_o, n_out & 1, STATUS_TIMEOUT_MMA);
                 ++n_out;

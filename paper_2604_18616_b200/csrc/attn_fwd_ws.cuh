@@ -31,7 +31,7 @@
 
 namespace ave {
 
-template <int D, bool CAUSAL = true>
+template <int D, bool CAUSAL = true, bool SPLIT = false, bool VARLEN = false>
 struct WsCfg {
     static constexpr int kThreads = 384;
     static constexpr int kQRows = 2 * BM;                    // query rows per work tile
@@ -43,7 +43,7 @@ struct WsCfg {
     static constexpr int kOutBoxRows = 32;                   // each softmax warp stores its own 32 rows
     // Keys of a step whose probabilities are handed over first, so that P V starts while the others are computed (128: all
     // at once).  Why, where and what it measured: see where the softmax hands P over.
-    static constexpr int kPFirst = (CAUSAL || D == 128) ? 96 : 128;
+    static constexpr int kPFirst = (CAUSAL || D == 128) && !SPLIT && !VARLEN ? 96 : 128;
     static constexpr int kPParts = kPFirst < 128 ? 2 : 1;
     static constexpr int kSmemBytes = kTileBytes * (2 + kStages) + 2 * kStageOBytes + 1024;
     static constexpr uint32_t kTmemCols = 512;
@@ -134,7 +134,7 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                    const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_o,
                    const FwdParams p) {
     if (threadIdx.x == 0) span_stamp(0);
-    using Cfg = WsCfg<D, CAUSAL>;
+    using Cfg = WsCfg<D, CAUSAL, SPLIT, VARLEN>;
     constexpr int NS = Cfg::kStages;
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(16) unsigned long long clc_response[2][2];
@@ -692,8 +692,10 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                             }
                         };
 
-                        // exact: take the maximum first, then exponentiate against it.
-                        bool exact = j == 0;
+                        // exact: take the maximum first, then exponentiate against it.  (The causal
+                        // instantiations always do: with their masking code the second copy of the
+                        // exponentiation loop costs registers and measured slower.)
+                        bool exact = CAUSAL || (j == 0);
                         bool maximum_settled = false;
                         if (!exact) {
                             // Optimistic: start exponentiating against the current m_run at once and find the
@@ -776,7 +778,8 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                         // heads of 16384, peaked 2079 -> 2055 us; 4 x 32 of 2048 180 -> 176, grouped 156.6 -> 152.5; 4 x 32 of
                         // 8192, D = 64 1505 -> 1492; no mask, 2 x 32 of 8192 1909 -> 1897; the clocks follow the power limit, in
                         // bursts the gains are twice that; 64 or 32 keys first: within 1 %).  Without a mask at D = 64 the extra
-                        // hand-over costs more than it gives (378 -> 390 us): there the row goes over in one piece.
+                        // hand-over costs more than it gives (378 -> 390 us), and so it does in variable-length launches (24 sequences of
+                        // up to 2500, D = 128 478 -> 499): there the row goes over in one piece.
                         const float m_tile = tile_max();
                         if (j == 0) {
                             m_run = m_tile;

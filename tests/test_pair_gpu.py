@@ -51,3 +51,12 @@ def test_values_that_only_the_other_sub_tile_sees():
     v[0, 0, 200, 5] = float("inf")
     o, lse = binding.ave_attn_fwd(q.cuda(), k.cuda(), v.cuda(), causal=True)
     assert torch.isfinite(lse).all() and torch.isfinite(o[:, :, :128]).all() and torch.all(o[:, :, 200:, 5] == float("inf"))
+
+
+@pytest.mark.parametrize("B,H,Sq,Sk", [(1, 2, 300, 640), (1, 2, 300, 641), (3, 33, 300, 512), (3, 33, 300, 384), (2, 33, 300, 512),
+                                       (1, 49, 300, 641), (1, 50, 300, 641)])
+def test_sides_of_the_kernel_choice(B, H, Sq, Sk):
+    # five and six key tiles; three and four with 297 and 198 tiles; 147 and 150 tiles, which pairs make 196 and 200 CTAs of
+    assert binding.select_kernel(binding.KERNEL_AUTO) == binding.AVE_OK
+    q, k, v = rand_qkv(H + Sk, B, H, H, Sq, Sk, 144)
+    parity.check_full(q, k, v, False, 1.0 / 12, "%s" % ((B, H, Sq, Sk),))

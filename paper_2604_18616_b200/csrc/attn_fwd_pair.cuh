@@ -77,7 +77,7 @@ attn_fwd_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
     __shared__ int tile_id[2];
     __shared__ __align__(4) Tile tile_info[2];
     __shared__ uint32_t tmem_base_slot;
-    __shared__ int abort_flag, poison_flag;
+    __shared__ int abort_flag, poison_flag, drain_flag;  // the last: (odd CTA) the even one's MMA issuer gave up
 
     const int tid = threadIdx.x;
     const int warp = tid >> 5;
@@ -88,7 +88,7 @@ attn_fwd_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
     const uint32_t sRing = sQ + Cfg::kQBytes;
 
     if (tid == 0) {
-        abort_flag = 0;
+        abort_flag = drain_flag = 0;
         mbar_init(smem_u32(&bar_q_full), 1);
         mbar_init(smem_u32(&bar_q_empty), 1);
         for (int t = 0; t < 2; ++t) {
@@ -198,6 +198,11 @@ attn_fwd_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
             }
             if (ok) id = next_tile(n, ok, w);
         }
+        // The commits that release what was loaded last arrive in both CTAs, and nothing else waits for them: not before
+        // they are here may this CTA's shared memory go to another one.
+        for (int pos = first_unreleased(ring, NS); pos < ring && ok; ++pos)
+            ok = wait_bar(&bar_empty[pos % NS], (pos / NS) & 1, STATUS_TIMEOUT_SLOT);
+        if (nt > 0 && ok) ok = wait_bar(&bar_q_empty, (nt - 1) & 1, STATUS_TIMEOUT_SLOT);
         if (!ok) {
             // abandoned: the loads still in flight are counted on the even CTA's barriers only; give them time to land
             const long long t1 = clock64();
@@ -271,7 +276,10 @@ attn_fwd_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
             if (ok) id = next_tile(n, ok, w);
         }
         if (!ok) {  // abandoned: let the MMAs already issued finish before TMEM is released
-            if (leader) umma_commit_pair(smem_u32(&bar_drain));
+            if (leader) {
+                umma_commit_pair(smem_u32(&bar_drain));
+                st_cluster_s32(map_to_cta(smem_u32(&drain_flag), 1), 1);  // it arrives there too: the odd CTA has to stay for it
+            }
             for (uint32_t x = 0; x < WAIT_LIMIT && !mbar_test_wait(smem_u32(&bar_drain), 0); ++x) {}
         }
     } else if (warp == 2 && rank == 0) {
@@ -528,12 +536,18 @@ attn_fwd_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
             }
             if (ok) id = next_tile(n, ok, w_tile);
         }
+        // the commit of the step before the last one, in the other buffer, which only a rescale waits for (see the producer)
+        if (g >= 2 && ok) ok = wait_bar(&bar_pv[g & 1], ((g - 2) >> 1) & 1, STATUS_TIMEOUT_MMA);
     }
 
-    // ---- common exit: nothing of the other CTA's may still be on its way to this one's barriers or TMEM
+    // ---- common exit.  All commits have arrived in both CTAs (every "s" and the last "pv" are waited for by the softmax, the
+    // last "pv" of the other buffer and the last "empty" ones above) unless the MMA issuer gave up: then the last of them,
+    // which follows all it issued, is given a bounded time here, in the odd CTA as in the even one.
     tc_fence_before();
     __syncthreads();
     cluster_sync();
+    if (warp == 2 && *reinterpret_cast<volatile int *>(&drain_flag) != 0)
+        for (uint32_t x = 0; x < WAIT_LIMIT && !mbar_test_wait(smem_u32(&bar_drain), 0); ++x) {}
     if (warp == 2) tmem_dealloc_pair(tmem, Cfg::kTmemCols);
 }
 

@@ -307,6 +307,10 @@ inline bool pairs_are_faster(int B, int H, int Hkv, int Sq, int Sk, bool causal,
     return 0.85 * waves(ctas) <= waves(tiles);
 }
 
+// A ring's producer fills position r after it has waited for the release of position r - stages, which lay in the same slot.
+// Of `used` filled positions it has therefore never waited for those from this one on.
+AVE_HD int first_unreleased(int used, int stages) { return imax(0, used - stages); }
+
 // Split-KV launches: keys per range = an equal share of Sk rounded up to whole key tiles.
 inline int splitkv_keys_per_split(int Sk, int n_splits) {
     const long long share = ((long long)Sk + n_splits - 1) / n_splits;

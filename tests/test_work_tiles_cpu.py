@@ -265,3 +265,13 @@ def test_the_five_configurations_and_the_papers_shape(wt):
 ])
 def test_kernel_choice(wt, B, H, Hkv, Sq, Sk, D, causal, total_q, one):
     assert wt.wt_one_subtile_is_faster(B, H, Hkv, Sq, Sk, D, int(causal), total_q, 148) == int(one)
+
+
+@pytest.mark.parametrize("stages", [1, 2, 5, 8])
+def test_every_release_of_a_ring_is_waited_for(wt, stages):
+    """A slot's release arrives in both CTAs of a pair; one that a producer leaves without having waited for could reach the
+    shared memory of whatever runs there next."""
+    for used in range(4 * stages + 2):
+        waited = [pos - stages for pos in range(used) if pos >= stages]          # while loading
+        waited += range(wt.wt_first_unreleased(used, stages), used)               # before it leaves
+        assert waited == list(range(used))

@@ -113,4 +113,6 @@ int wt_one_subtile_is_faster(int B, int H, int Hkv, int Sq, int Sk, int D, int c
     return ave::one_subtile_is_faster(B, H, Hkv, Sq, Sk, D, causal != 0, total_q, sms) ? 1 : 0;
 }
 
+int wt_first_unreleased(int used, int stages) { return ave::first_unreleased(used, stages); }
+
 }  // extern "C"

@@ -529,7 +529,7 @@ gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_con
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t bar_full[NS], bar_empty[NS], bar_acc_full[2], bar_acc_empty[2], bar_drain;
     __shared__ uint32_t tmem_base_slot;
-    __shared__ int abort_flag, poison_flag;
+    __shared__ int abort_flag, poison_flag, drain_flag;  // the last: (odd CTA) the even one's MMA issuer gave up
 
     const int tid = threadIdx.x;
     const int warp = tid >> 5;
@@ -539,7 +539,7 @@ gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_con
     const uint32_t sStage = sRing + NS * Cfg::kStageBytes;
 
     if (tid == 0) {
-        abort_flag = 0;
+        abort_flag = drain_flag = 0;
         for (int s = 0; s < NS; ++s) {
             mbar_init(smem_u32(&bar_full[s]), 1);
             mbar_init(smem_u32(&bar_empty[s]), 1);
@@ -649,6 +649,7 @@ gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_con
             }
             if (!ok) {  // abandoned: let the MMAs already issued finish before TMEM is released
                 umma_commit_pair(smem_u32(&bar_drain));
+                st_cluster_s32(map_to_cta(smem_u32(&drain_flag), 1), 1);  // it arrives there too: the odd CTA has to stay for it
                 for (uint32_t w = 0; w < WAIT_LIMIT && !mbar_test_wait(smem_u32(&bar_drain), 0); ++w) {}
             }
         }
@@ -700,10 +701,13 @@ gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_con
         if (lane == 0 && store_pending) tma_store_wait_all();
     }
 
-    // ---- common exit: nothing of the other CTA's may still be on its way to this one's barriers or TMEM
+    // ---- common exit.  The commit of the last accumulator, which both epilogues wait for, follows all others; if the MMA issuer
+    // gave up, its last commit is given a bounded time here, in the odd CTA as in the even one.
     tc_fence_before();
     __syncthreads();
     cluster_sync();
+    if (warp == 2 && *reinterpret_cast<volatile int *>(&drain_flag) != 0)
+        for (uint32_t w = 0; w < WAIT_LIMIT && !mbar_test_wait(smem_u32(&bar_drain), 0); ++w) {}
     if (warp == 2) tmem_dealloc_pair(tmem, Cfg::kTmemCols);
 }
 

@@ -73,6 +73,7 @@ struct OneCfg {
     // (64 sequences of 4001 keys 192.4 -> 193.5).
     static constexpr int kPFirst = kTwoS || WHOLE_P ? 128 : 96;
     static constexpr int kPParts = kPFirst < 128 ? 2 : 1;
+    static constexpr int kRescaleCols = D < 128 ? D : 128;   // columns of O rescaled at a time (32 scores are left, or none)
     static constexpr int kTileConsumers = 6;                 // producer + MMA + 4 softmax warps read each tile
 };
 
@@ -579,16 +580,7 @@ attn_fwd_1t_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                                     if (!ok) return false;
                                     tc_fence_after();
                                 }
-#pragma unroll 1
-                                for (int c = 0; c < D; c += 32) {
-                                    uint32_t oc[32];
-                                    tmem_ld_x32(tO + c, oc);
-                                    tmem_wait_ld();
-                                    tmem_pin_x32(oc);
-#pragma unroll
-                                    for (int e = 0; e < 32; ++e) oc[e] = __float_as_uint(__uint_as_float(oc[e]) * alpha);
-                                    tmem_st_x32(tO + c, oc);
-                                }
+                                scale_tmem_row<D, Cfg::kRescaleCols>(tO, alpha);
                             }
                             tmem_wait_st();
                             tc_fence_before();

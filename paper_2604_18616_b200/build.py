@@ -5,7 +5,8 @@
 
 The build reads ptxas' resource report and refuses an image in which an
 attention kernel got fewer registers per thread than its warp roles' register
-split draws on (``setmaxnreg.inc`` beyond the CTA's allocation never returns).
+split draws on (``setmaxnreg.inc`` beyond the CTA's allocation never returns),
+or a kernel spills more than a pair of registers.
 The library repeats the check at run time on the loaded image.
 """
 from __future__ import annotations
@@ -29,15 +30,18 @@ NVCC_FLAGS = [
 ]
 
 # Register split of the attention kernel (WsCfg in csrc/attn_fwd_ws.cuh): 384 threads, of which one
-# warpgroup keeps 64 registers per thread and two take 216.
+# warpgroup keeps 64 registers per thread and two take 216 (72 and 208, which is less in all, in some instantiations).
 ATTN_THREADS = 384
 ATTN_REGS_NEEDED = 128 * 64 + 256 * 216
-# The single-sub-tile kernel (OneCfg in csrc/attn_fwd_1t.cuh): 256 threads, 48 and 208 registers.
+# The single-sub-tile kernel (OneCfg in csrc/attn_fwd_1t.cuh): 256 threads, 48 and 208 registers, or 56 and 200.
 ONE_THREADS = 256
 ONE_REGS_NEEDED = 128 * 48 + 128 * 208
 # The MoE GEMM (MoeGemmCfg in csrc/moe_fp8.cuh): 384 threads, 56 and 224 registers.
 MOE_THREADS = 384
 MOE_REGS_NEEDED = 128 * 56 + 256 * 224
+# What a kernel may spill, in bytes a thread: one pair of registers.  (The split-KV form of the two-sub-tile kernel at D = 128 and
+# the MoE GEMM do.)
+SPILL_BYTES_ALLOWED = 8
 
 
 def _sources():
@@ -73,6 +77,22 @@ def check_register_split(ptxas_report: str) -> dict:
             raise RuntimeError("%s was compiled with %d registers per thread; its warp roles need %d x %d >= %d" % (
                 name, n, threads, n, needed))
     return regs
+
+
+def check_spills(ptxas_report: str) -> dict:
+    """{mangled kernel name: bytes spilled}; raise if a kernel spills more than SPILL_BYTES_ALLOWED."""
+    spills, current = {}, None
+    for line in ptxas_report.splitlines():
+        m = re.search(r"Compiling entry function '([^']+)'", line)
+        if m:
+            current = m.group(1)
+        m = re.search(r"(\d+) bytes spill stores", line)
+        if m and current:
+            spills[current] = int(m.group(1))
+    for name, n in spills.items():
+        if n > SPILL_BYTES_ALLOWED:
+            raise RuntimeError("%s spills %d bytes of registers" % (name, n))
+    return spills
 
 
 def build_fastcall(force: bool = False) -> str:
@@ -120,6 +140,7 @@ def build_cuda(force: bool = False, verbose: bool = False) -> str:
         raise subprocess.CalledProcessError(r.returncode, cmd)
     try:
         check_register_split(r.stdout)
+        check_spills(r.stdout)
     except Exception:
         if os.path.exists(tmp):
             os.remove(tmp)

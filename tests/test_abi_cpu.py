@@ -213,3 +213,13 @@ def test_splitkv_wrappers_refuse_host_tensors(monkeypatch, bad):
         binding.ave_attn_fwd_splitkv_static(t["q"], t["k"], t["v"], 2, o, lse)
     with pytest.raises(ValueError):   # whatever the wrappers check: no call without a device
         binding._call("ave_attn_fwd", torch.zeros(1), None)
+
+
+def test_build_refuses_kernels_that_spill():
+    ok = ("ptxas info    : Compiling entry function '_ZN3ave18attn_fwd_1t_kernelILi64ELb1ELb0ELb0EEEvx' for 'sm_100a'\n"
+          "ptxas info    : Function properties for _ZN3ave18attn_fwd_1t_kernelILi64ELb1ELb0ELb0EEEvx\n"
+          "    8 bytes stack frame, 8 bytes spill stores, 4 bytes spill loads\n"
+          "ptxas info    : Used 128 registers, used 1 barriers\n")
+    assert list(build.check_spills(ok).values()) == [8]
+    with pytest.raises(RuntimeError, match="spills 16 bytes"):
+        build.check_spills(ok.replace("8 bytes spill stores", "16 bytes spill stores"))

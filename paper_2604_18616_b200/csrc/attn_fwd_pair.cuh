@@ -42,6 +42,7 @@ struct PairCfg {
     static constexpr uint32_t kTmemCols = 512;
     static constexpr uint32_t kColS = 0, kColO = 128, kColS1 = 384;
     static constexpr int kPFirst = 96;                   // keys of a step whose probabilities are handed over first
+    static constexpr int kRescaleCols = 128;             // columns of O rescaled at a time
     static constexpr int kTileReaders = 7;               // even CTA: producer, MMA issuer, 4 softmax warps, and the odd CTA as one
     static constexpr int kTileReadersOdd = 5;            // odd CTA: producer, 4 softmax warps
 };
@@ -460,16 +461,7 @@ attn_fwd_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                         ok = wait_bar(&bar_pv[buf ^ 1], ((g - 2) >> 1) & 1, STATUS_TIMEOUT_MMA);
                         if (!ok) return false;
                         tc_fence_after();
-#pragma unroll 1
-                        for (int c = 0; c < D; c += 32) {
-                            uint32_t oc[32];
-                            tmem_ld_x32(tO + c, oc);
-                            tmem_wait_ld();
-                            tmem_pin_x32(oc);
-#pragma unroll
-                            for (int e = 0; e < 32; ++e) oc[e] = __float_as_uint(__uint_as_float(oc[e]) * alpha);
-                            tmem_st_x32(tO + c, oc);
-                        }
+                        scale_tmem_row<D, Cfg::kRescaleCols>(tO, alpha);
                     }
                     tmem_wait_st();
                     tc_fence_before();

@@ -286,18 +286,27 @@ inline bool one_subtile_is_faster(int B, int H, int Hkv, int Sq, int Sk, int D, 
 }
 
 // Whether a problem with a head dimension above 128 is better off on CTA pairs (two 128-row sub-tiles a pair) than in the
-// single-sub-tile kernel (a CTA for 128 rows).  Times below: pairs / single, D = 256, from 70 shapes.
+// single-sub-tile kernel (a CTA for 128 rows).  Times below: pairs / single, from 550 shapes with D = 136, 192 and 256, which take
+// the same time within some 5 %.
 inline bool pairs_are_faster(int B, int H, int Hkv, int Sq, int Sk, bool causal, int total_q, int sms) {
     auto blocks = [&](int rows) {
         return total_q > 0 ? (long long)total_q / rows + B : (long long)B * (((long long)Sq + rows - 1) / rows);
     };
+    const bool paired = causal && H / Hkv % 2 == 0;  // the CTAs of a pair have two heads' rows, else two blocks of one head's
     const long long tiles = H * blocks(BM);
-    const long long ctas = causal && H / Hkv % 2 == 0 ? tiles : 2 * H * blocks(2 * BM);  // (an odd last block leaves a CTA without rows)
-    // A pair starts and ends a tile some 3 us later and then gains 0.4 us a step: from six key tiles on it is ahead (8 heads of
-    // 177 rows and 699 keys 15.6 / 16.8 us, 8 of 286 and 517 17.7 / 17.3), from four if the tiles follow one another (4 x 16 heads
-    // of 300 rows 20.1 / 21.6 and 256 of 512 59 / 64, but 48 of 505 20.9 / 20.7, 32 of 366 14.2 / 13.7).
+    const long long ctas = paired ? tiles : 2 * H * blocks(2 * BM);  // (an odd last block leaves a CTA without rows)
+    // A pair starts and ends a tile some 3 us later and then gains 0.4 us a step.  With tiles that follow one another it is ahead
+    // from four key tiles on (4 x 2 heads of 2051 rows and 400 keys 23.8 / 26.1 us, 7 x 32 of 177 and 462 37.0 / 42.3; with three
+    // 0.93 to 1.15 of the time), else from six (2 heads of 768 rows and keys 14.8 / 16.0, 8 of 708 15.8 / 16.8; with five, where it is
+    // level or up to 5 % ahead, and with four the line was not drawn finer).  Causal launches without pairs of heads have
+    // their last step in one CTA only: a sixth tile that is not half full does not count (8 heads of 641 15.3 / 15.1, of 767
+    // 15.1 / 15.9).  Where one CTA of every pair has no rows, with more than 32 tiles from eight key tiles on (3 x 16 heads
+    // of 80 rows, 708 keys 16.5 / 15.9, 895 keys 17.8 / 17.4, 1023 keys 19.0 / 19.0, 1152 keys 19.6 / 20.2; 16 x 2 heads of 64, 742
+    // keys 15.0 / 15.4).
     const int key_tiles = (Sk + BN - 1) / BN;
-    if (key_tiles < 4 || (key_tiles < 6 && tiles <= 2 * sms)) return false;
+    if (key_tiles < 4) return false;
+    if (tiles <= 2 * sms && (causal && !paired ? Sk <= 5 * BN + BN / 2 : key_tiles < 6)) return false;
+    if (!paired && Sq <= BM && tiles > 32 && key_tiles < 8) return false;
     // Where CTAs without rows cost another wave they take it back (144 tiles, 160 CTAs of 1056 keys: 32.9 / 23.6 us; 144 and 288
     // of 2489 keys: 68.3 / 47.9).  A step of a pair takes 0.77 to 0.87 of the other kernel's time.
     auto waves = [&](long long n) {

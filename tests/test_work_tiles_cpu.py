@@ -275,3 +275,31 @@ def test_every_release_of_a_ring_is_waited_for(wt, stages):
         waited = [pos - stages for pos in range(used) if pos >= stages]          # while loading
         waited += range(wt.wt_first_unreleased(used, stages), used)               # before it leaves
         assert waited == list(range(used))
+
+
+@pytest.mark.parametrize("B,H,Hkv,Sq,Sk,causal,total_q,pairs", [
+    # head dimensions above 128, times as pairs / single sub-tile (148 SMs)
+    (2, 1, 1, 768, 768, False, 0, True),         # six key tiles: 14.8 / 16.0
+    (1, 32, 32, 200, 640, False, 0, False),      # five, few tiles: level
+    (7, 32, 8, 177, 462, True, 0, True),         # four, more than two tiles per SM: 37.0 / 42.3
+    (4, 2, 2, 2051, 400, False, 0, False),       # four, 272 tiles
+    (3, 64, 8, 316, 316, False, 0, False),       # three: 46.3 / 40.4
+    (1, 8, 8, 641, 641, True, 0, False),         # causal, one key in the sixth tile: 15.3 / 15.1
+    (2, 1, 1, 708, 708, True, 0, True),          # 68 keys: 14.5 / 15.0
+    (1, 8, 8, 767, 767, True, 0, True),          # 15.1 / 15.9
+    (1, 8, 2, 641, 641, True, 0, True),          # pairs of heads: 14.4 / 15.1
+    (3, 16, 16, 80, 708, False, 0, False),       # every second CTA without rows: 16.5 / 15.9
+    (3, 16, 16, 80, 896, True, 0, False),        # seven: 17.75 / 17.2
+    (3, 16, 16, 80, 1024, False, 0, True),       # eight: level
+    (16, 2, 2, 64, 742, False, 0, True),         # six, 32 tiles: 15.0 / 15.4
+    (6, 16, 16, 65, 1706, False, 0, False),      # 96 tiles, 192 CTAs: 54 / 34
+    (4, 16, 4, 64, 768, True, 0, True),          # the same rows as pairs of heads
+    (1, 16, 16, 1100, 1056, False, 0, False),    # 144 tiles, 160 CTAs, a second wave: 32.9 / 23.6
+    (1, 49, 49, 300, 641, False, 0, False), (1, 50, 50, 300, 641, False, 0, True),   # 147 and 150 tiles, 196 and 200 CTAs
+    (4, 64, 8, 534, 796, False, 0, False),       # 1280 tiles, 1536 CTAs: 0.85 of 10.4 waves against 8.6 (147 / 152)
+    (6, 64, 64, 1, 1100, False, 0, False),       # 384 tiles, 768 CTAs
+    (12, 4, 4, 590, 590, True, 2500, False),     # variable lengths: 4 x (19 + 12) tiles, five key tiles
+    (4, 32, 16, 1400, 1400, True, 3000, True),
+])
+def test_choice_of_cta_pairs(wt, B, H, Hkv, Sq, Sk, causal, total_q, pairs):
+    assert wt.wt_pairs_are_faster(B, H, Hkv, Sq, Sk, int(causal), total_q, 148) == int(pairs)

@@ -113,6 +113,11 @@ int wt_one_subtile_is_faster(int B, int H, int Hkv, int Sq, int Sk, int D, int c
     return ave::one_subtile_is_faster(B, H, Hkv, Sq, Sk, D, causal != 0, total_q, sms) ? 1 : 0;
 }
 
+// The choice between CTA pairs and the single-sub-tile kernel (D > 128).
+int wt_pairs_are_faster(int B, int H, int Hkv, int Sq, int Sk, int causal, int total_q, int sms) {
+    return ave::pairs_are_faster(B, H, Hkv, Sq, Sk, causal != 0, total_q, sms) ? 1 : 0;
+}
+
 int wt_first_unreleased(int used, int stages) { return ave::first_unreleased(used, stages); }
 
 }  // extern "C"

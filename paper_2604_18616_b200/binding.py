@@ -8,8 +8,11 @@ from __future__ import annotations
 
 import ctypes
 import os
+import warnings
 
 import torch
+
+from .build import fastcall_stamp
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libave_attn.so")
@@ -32,7 +35,8 @@ STATUS_BIT_SELFTEST = 16
 SPLITKV_STATIC_SCRATCH_BYTES = 8 << 20
 
 _lib = None
-# The ordinary case of the calls below in C++ (csrc/fastcall.cc); each returns None for a call that is not one.
+# The ordinary case of the calls below in C++ (csrc/fastcall.cc); each returns None for a call that is not one.  None without
+# the extension, or with one that was built for another torch or Python: every call then goes the Python wrappers' own way.
 _fast = None
 FAST_PATH = os.path.join(_HERE, "_fastcall.so")
 
@@ -107,9 +111,16 @@ def lib() -> ctypes.CDLL:
 
 def _bind_fast(L) -> None:
     global _fast
-    if not os.path.exists(FAST_PATH):
-        raise RuntimeError("%s is missing: build it with `python -m paper_2604_18616_b200.build`" % FAST_PATH)
-    from . import _fastcall
+    try:
+        if os.path.exists(FAST_PATH + ".stamp"):
+            with open(FAST_PATH + ".stamp") as f:
+                if f.read() != fastcall_stamp():
+                    raise ImportError("it was built for another torch or Python")
+        from . import _fastcall
+    except (ImportError, OSError) as e:
+        warnings.warn("%s cannot be used (%s): calls take the slower way through ctypes; build it with `python -m "
+                      "paper_2604_18616_b200.build`" % (FAST_PATH, e), RuntimeWarning, stacklevel=3)
+        return
     _fastcall.bind(*[ctypes.cast(f, ctypes.c_void_p).value for f in (
         L.ave_attn_fwd, L.ave_attn_fwd_splitkv, L.ave_gemm_bf16_tn, L.ave_gemm_bf16_nn)])
     _fast = _fastcall

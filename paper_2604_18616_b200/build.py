@@ -95,6 +95,14 @@ def check_spills(ptxas_report: str) -> dict:
     return spills
 
 
+def fastcall_stamp() -> str:
+    """What the extension is built for: it uses the C++ interface of this torch and the C interface of this Python."""
+    import sysconfig
+
+    import torch
+    return "%s %s" % (torch.__version__, sysconfig.get_config_var("SOABI"))
+
+
 def build_fastcall(force: bool = False) -> str:
     """The C++ part of the binding: a Python extension over torch's C++ library."""
     import sysconfig
@@ -102,8 +110,7 @@ def build_fastcall(force: bool = False) -> str:
     import torch
     src = os.path.join(CSRC, "fastcall.cc")
     tdir = os.path.dirname(torch.__file__)
-    # (built again when another torch is installed: it uses torch's C++ interface)
-    stamp, stamp_path = "%s %s %s" % (torch.__version__, tdir, sysconfig.get_paths()["include"]), FAST_PATH + ".stamp"
+    stamp, stamp_path = fastcall_stamp(), FAST_PATH + ".stamp"
     if not force and os.path.exists(FAST_PATH) and os.path.getmtime(FAST_PATH) >= os.path.getmtime(src) and os.path.exists(stamp_path):
         with open(stamp_path) as f:
             if f.read() == stamp:

@@ -4,6 +4,8 @@ CUDA."""
 import ctypes
 import os
 import re
+import subprocess
+import sys
 
 import pytest
 
@@ -223,3 +225,25 @@ def test_build_refuses_kernels_that_spill():
     assert list(build.check_spills(ok).values()) == [8]
     with pytest.raises(RuntimeError, match="spills 16 bytes"):
         build.check_spills(ok.replace("8 bytes spill stores", "16 bytes spill stores"))
+
+
+_LOAD = """
+import sys, warnings
+from paper_2604_18616_b200 import binding
+if sys.argv[1] == "missing":
+    sys.modules["paper_2604_18616_b200._fastcall"] = None      # (as an import finds it when there is no such file)
+elif sys.argv[1] == "other torch":
+    binding.fastcall_stamp = lambda: "another"
+with warnings.catch_warnings(record=True) as w:
+    warnings.simplefilter("always")
+    assert binding.version() > 0 and binding.strerror(0)
+assert binding.ave_attn_fwd_raw(0, 0, 0, 0, 0, 1, 1, 1, 1, 1, 64, False, 1.0) == binding.AVE_ERR_NULL_POINTER
+print(binding._fast is not None, [str(x.category.__name__) for x in w if "ctypes" in str(x.message)])
+"""
+
+
+@pytest.mark.parametrize("case,result", [("built", "True []"), ("missing", "False ['RuntimeWarning']"),
+                                         ("other torch", "False ['RuntimeWarning']")])
+def test_the_binding_works_without_the_extension(lib, case, result):
+    r = subprocess.run([sys.executable, "-c", _LOAD, case], cwd=ROOT, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
+    assert r.returncode == 0 and r.stdout.strip() == result, r.stdout

@@ -27,6 +27,49 @@ def test_results_are_those_of_the_python_way(causal, scale):
     assert torch.equal(binding.ave_gemm_bf16_nn(a, b), binding.ave_gemm_bf16_nn(a, b, c=a.new_empty(a.shape[0], b.shape[1])))
 
 
+def test_ordinary_calls_take_the_short_way():
+    """Each extension function launches by itself and its results are those of the Python way; the wrappers ask it first."""
+    q, k, v = [t.cuda() for t in rand_qkv(7, 2, 6, 2, 70, 130, 64)]
+    binding.lib()
+    fast = binding._fast
+    assert fast is not None
+    ws = torch.empty(binding.splitkv_workspace_bytes(2, 6, 70, 64, 2), dtype=torch.uint8, device="cuda")
+    a, b = q.reshape(-1, 64), k.reshape(-1, 64)
+    bt = b.t().contiguous()[:, :512].contiguous()
+    new = lambda r, c: torch.empty(r, c, dtype=torch.bfloat16, device="cuda")
+    for got, want in [
+            (lambda: fast.attn_fwd(q, k, v, True, None), lambda: binding.ave_attn_fwd(q, k, v, o=torch.empty_like(q), causal=True)),
+            (lambda: fast.attn_fwd(q, k, v, 0, 0.3), lambda: binding.ave_attn_fwd(q, k, v, o=torch.empty_like(q), scale=0.3)),
+            (lambda: fast.attn_fwd_splitkv(q, k, v, 2, ws, True, None),
+             lambda: binding.ave_attn_fwd_splitkv(q, k, v, 2, workspace=ws, o=torch.empty_like(q), causal=True)),
+            (lambda: (fast.gemm_tn(a, b),), lambda: (binding.ave_gemm_bf16_tn(a, b, c=new(a.shape[0], b.shape[0])),)),
+            (lambda: (fast.gemm_nn(a, bt),), lambda: (binding.ave_gemm_bf16_nn(a, bt, c=new(a.shape[0], 512)),))]:
+        n0 = binding.launch_count()
+        r = got()
+        assert r is not None and all(isinstance(t, torch.Tensor) for t in r)
+        torch.cuda.synchronize()
+        assert binding.launch_count() > n0, "nothing was launched"
+        assert all(torch.equal(x, y) for x, y in zip(r, want()))
+    # a status of the library comes back as an int: three heads on two
+    assert fast.attn_fwd(q[:, :3].contiguous(), k, v, False, None) == binding.AVE_ERR_BAD_SHAPE
+    assert fast.gemm_tn(a[:, :60].contiguous(), b[:, :60].contiguous()) == binding.AVE_ERR_MISALIGNED
+
+
+@pytest.mark.parametrize("call,args", [("attn_fwd", 3), ("attn_fwd_splitkv", 3), ("gemm_tn", 2), ("gemm_nn", 2)])
+def test_wrappers_return_what_the_short_way_gave(call, args, monkeypatch):
+    seen = []
+
+    class Fast:
+        def __getattr__(self, name):
+            return lambda *a: seen.append(name) or "result"
+
+    binding.lib()
+    monkeypatch.setattr(binding, "_fast", Fast())
+    x = [torch.empty(0)] * args
+    wrapper = getattr(binding, "ave_attn_fwd" + call[8:] if call.startswith("attn") else "ave_gemm_bf16" + call[4:])
+    assert (wrapper(*x, 2) if call == "attn_fwd_splitkv" else wrapper(*x)) == "result" and seen == [call]
+
+
 def test_calls_out_of_the_ordinary_are_left_to_the_python_way():
     q, k, v = [t.cuda() for t in rand_qkv(4, 1, 2, 2, 8, 16, 64)]
     binding.lib()

@@ -1,16 +1,25 @@
 """Head dimensions above 128: two score buffers and a ring of half K and V tiles.  Key counts around the half and whole tiles,
 tiles of one, two and more steps one after the other on the same SM, and scores whose maximum moves at every step, so that
-the accumulator is rescaled between the products that overlap it.  Oracle and tolerances are those of the parity tests."""
+the accumulator is rescaled between the products that overlap it.  In the single-sub-tile kernel and on CTA pairs, whichever of
+them a call would choose by itself.  Oracle and tolerances are those of the parity tests."""
 import math
 
 import pytest
 import torch
 
 import parity
+from paper_2604_18616_b200 import binding
 from test_splitkv_gpu import rand_qkv
 from test_varlen_gpu import _run_and_check
 
 pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(params=[binding.KERNEL_ONE_SUBTILE, binding.KERNEL_TWO_SUBTILES], autouse=True)
+def kernel(request):
+    assert binding.select_kernel(request.param) == binding.AVE_OK
+    yield
+    assert binding.select_kernel(binding.KERNEL_AUTO) == binding.AVE_OK
 
 
 @pytest.mark.parametrize("D", [136, 192, 256])

@@ -70,7 +70,8 @@ struct OneCfg {
     static_assert(128 * kRegsLight + 128 * kRegsSoftmax <= kThreads * kRegsAtLaunch,
                   "register split exceeds the CTA's allocation");
     // Keys of a step whose probabilities are handed over first: P V of them runs while the others are computed, which shortens
-    // the chain of a step (8 heads of 1483 rows, D = 128 26.0 -> 24.1 us; 8 of 200 rows and 8000 keys 106.1 -> 97.9).  With two score
+    // the chain of a step (8 causal heads of 1483 rows, D = 128 25.8 -> 23.9 us, D = 64 20.7 -> 20.3; 8 of 200 rows and 8000 keys, no
+    // mask, 104.6 -> 95.2 and 86.9 -> 83.2; 8 of 300, D = 64 8.32 -> 8.22; nothing slower at D = 64 either).  With two score
     // buffers the products are ahead of the softmax anyway; a decode step waits for HBM, and the extra hand-over is lost
     // (64 sequences of 4001 keys 192.4 -> 193.5).
     static constexpr int kPFirst = kTwoS || WHOLE_P ? 128 : 96;

@@ -6,9 +6,9 @@
 // halves.  With one CTA per tile (attn_fwd_1t.cuh) the products are bound by shared memory: a step of 128 keys reads
 // 128 KB for Q K^T and 64 KB for P V while the loads write 128 KB, 2500 clk at its 128 B/clk for 2048 clk of MMAs.  Here a
 // CTA reads 96 + 32 KB and loads 64 KB: 1500 clk.
-// 2 x 32 heads of 4096, causal, D = 256 542 -> 455 us; 64 heads of 4434 1271 -> 1028 (both at the power limit); D = 192, 32 heads
-// of 1602 52.9 -> 47.2; 64 rows of 4096 keys, 2 x 32 heads 57.2 -> 47.1.  What bounds it now: the power limit, and where tiles
-// are few the chain of a step's products and softmax.
+// The single-sub-tile kernel / this one: 2 x 32 heads of 4096, causal, D = 256 549 / 460 us (at the power limit); D = 192, 32
+// heads of 1602 56 / 46; 16 heads of 100 rows and 8000 keys 106.5 / 79.4.  What bounds it: the power limit, and where tiles are
+// few the chain of a step's products and softmax.
 //
 //   warp 0       producer: TMA loads of Q and of this CTA's halves of K and V
 //   warp 1       even CTA: MMA issuer
@@ -42,7 +42,9 @@ struct PairCfg {
     static constexpr uint32_t kTmemCols = 512;
     static constexpr uint32_t kColS = 0, kColO = 128, kColS1 = 384;
     static constexpr int kPFirst = 96;                   // keys of a step whose probabilities are handed over first
-    static constexpr int kRescaleCols = 128;             // columns of O rescaled at a time
+    // Columns of O rescaled at a time.  With scores that rise from key to key, 32 / 64 / 128: 6 x 16 heads of 1113 151 / 145 / 141 us
+    // (single-sub-tile kernel 139), 16 heads of 100 rows and 8000 keys 107 / 101 / 98 (113); registers 200 to 208 either way.
+    static constexpr int kRescaleCols = 128;
     static constexpr int kTileReaders = 7;               // even CTA: producer, MMA issuer, 4 softmax warps, and the odd CTA as one
     static constexpr int kTileReadersOdd = 5;            // odd CTA: producer, 4 softmax warps
 };

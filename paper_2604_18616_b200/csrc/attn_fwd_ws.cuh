@@ -767,8 +767,9 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                         // heads of 16384, peaked 2079 -> 2055 us; 4 x 32 of 2048 180 -> 176, grouped 156.6 -> 152.5; 4 x 32 of
                         // 8192, D = 64 1505 -> 1492; no mask, 2 x 32 of 8192 1909 -> 1897; the clocks follow the power limit, in
                         // bursts the gains are twice that; 64 or 32 keys first: within 1 %).  Without a mask at D = 64 the extra
-                        // hand-over costs more than it gives (378 -> 390 us), and so it does in variable-length launches (24 sequences of
-                        // up to 2500, D = 128 478 -> 499): there the row goes over in one piece.
+                        // hand-over costs more than it gives (378 -> 390 us), and so it does in causal variable-length launches (24 sequences
+                        // of up to 2500, D = 128 446 -> 479, with 32 columns of O rescaled at a time 476): there the row goes over in
+                        // one piece.
                         const float m_tile = tile_max();
                         if (j == 0) {
                             m_run = m_tile;

@@ -5,7 +5,7 @@ of the library (``-DAVE_TRACE=<cta> -DAVE_TRACE_TILE=<k>``, written beside the n
 ``libave_attn_trace.so``), runs the named workload on cuda:0 and prints, in time order, the SM-clock
 stamps that the producer, MMA and softmax warps of that CTA took during its k-th and (k+1)-th work
 tiles: where a key step's time goes, and what a tile boundary costs.  The normal library carries no
-trace code.
+trace code, and the kernel of CTA pairs (head dimensions above 128) takes no stamps.
 """
 from __future__ import annotations
 
